@@ -49,7 +49,9 @@ extern "C" {
 #define QSIM_C128 1 /* complex128: float64 real and imaginary parts */
 
 /* Arithmetic used for fused dense blocks (Sec. 2.1: fusion trades flops for arithmetic intensity). */
-#define QSIM_PREC_SIMT 0   /* CUDA-core FMA in the state's own precision */
+#define QSIM_PREC_SIMT 0   /* the state's own precision: CUDA-core FMA, or, for fused blocks of
+                              up to 5 qubits where it is faster, exact integer products on the
+                              tensor cores, whose error is no larger */
 #define QSIM_PREC_TF32X3 1 /* tensor cores: 3 TF32 products (hi*hi + hi*lo + lo*hi), FP32 accumulation */
 #define QSIM_PREC_BF16X3 2 /* tensor cores: 2-way BF16 split, 3 products, FP32 accumulation. REDUCED
                               accuracy (~16 significant bits per product, not complex64 level): ~1e-8

@@ -140,6 +140,16 @@ cudaError_t launch_tc7_prepare(const double* dU, void* dB, cudaStream_t s);
 cudaError_t launch_tc7_apply(void* psi, int n, const int* targets, const void* dB, unsigned* dev_err, cudaStream_t s,
                              const DevInfo& d, const uint64_t* from_basis);
 
+// ---- blocks of up to 5 qubits in the state's own precision on the tensor cores (k_tcx.cu) -------------------
+// True when a block of k qubits of an n-qubit state can take this path (k <= 5, n >= 12).
+bool tcx_supported(int n, int k);
+// Bytes of the prepared operand, and its preparation from a device FP64 matrix U (2^k x 2^k complex).
+size_t tcx_operand_bytes(int dtype);
+cudaError_t launch_tcx_prepare(int dtype, const double* dU, int k, void* dB, cudaStream_t s);
+// Apply the prepared block; with from_basis its input is the basis state |*from_basis>, generated instead of read.
+cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targets, const void* dB, unsigned* dev_err,
+                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis = nullptr);
+
 // ---- two 6-qubit blocks in one pass (k_tc_pair.cu, FP16 split products) -------------------------------------
 // True when blocks on t1 and then t2 (6 targets each, in their matrices' index order) fit one 13-bit tile of
 // an n-qubit state (|t1 u t2| <= 12, n >= 13).

@@ -1,0 +1,679 @@
+// k_tcx.cu -- a fused block of up to 5 qubits in the state's own precision (QSIM_PREC_SIMT plans) on the
+// tensor cores, by exact integer slices.
+//
+// Paper Sec. 2.1: a fused block is one small dense matrix applied to every group of 2^k amplitudes. On CUDA
+// cores a 5-qubit block is 128 FMAs an amplitude: 3.5 ms at 24 qubits in complex128 (FP64 runs at 1.05 TFLOP/s
+// here; moving the state takes 0.08 ms), 0.46 ms at 26 qubits in complex64 (0.16 ms to move it). The tensor
+// cores have the rate, so the block is computed as sums of integer products that they add without rounding (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump 2012, on FP16 operands as Mukunoki, Ozaki, Ogita and
+// Imamura 2020):
+//   * the 64 reals of a row (a group's 32 complex amplitudes) become fixed-point numbers relative to the row's
+//     largest exponent E, 2^54 (complex128) or 2^30 (complex64) steps, cut into signed base-256 digits
+//     (7 or 4); U likewise. Digits are integers in [-128, 127], exact in FP16.
+//   * D_d = sum over digit positions s + t = d of X_s U_t^T accumulates in FP32 tensor memory: at most 7 * 64
+//     products of at most 2^14, below 2^24, so every sum is an exact integer. Positions d < 8 (complex128; 34
+//     of 49 products) or d < 4 (complex64; 10 of 16) are kept; the first one left out is worth 2^-59
+//     (2^-28) of the row's scale.
+//   * y = 2^(E') sum_d D_d 2^(-8d): in complex128 summed in a 64-bit integer and rounded once, in complex64 by
+//     three FMAs.
+// The errors are those of the fixed-point steps, 2^-55 (2^-31) of the row's scale, and of the final rounding:
+// smaller than the accumulated roundings of 64 FMAs (against 64 bits, 23-qubit brickwork of depth 10: 1.6e-15,
+// by FMAs 1.8e-15; 26-qubit random pairs in complex64: 2.3e-7, by FMAs 1.0e-6). A row with an infinity or NaN
+// gives NaN.
+//
+// Layout. A tile is 128 rows (the 7 lowest index bits outside the block) by 32 columns; blocks of fewer qubits
+// take idle qubits as further columns (U x I). Digit plane s of a tile is a K-major operand of 128 x 64 FP16
+// (16 KiB, SWIZZLE_128B) in shared memory, digit planes of U are stacked as 64-row operands. Because D_d and
+// D_{d+1} are neighbouring 64-column blocks of tensor memory, one MMA of X_s against the stacked rows of
+// U_t..U_{t+3} (N = 256) adds to four digit positions at once, at the full rate of the tensor cores (with N = 64
+// the reads of A from shared memory would bound it).
+//
+// Roles, one CTA per SM: input warps load a tile, convert it and write its planes; one warp issues the MMAs;
+// output warps sum the positions, convert back and store. In complex64 (16 input, 8 output warps) planes and
+// accumulators are double-buffered, and the next tile's loads are in flight in registers. In complex128 the 8
+// positions take all of tensor memory and the planes half of shared memory, so a tile's MMAs commit in four
+// groups of planes: as a group retires, the input (8 warps) writes the next tile's planes over it and the output
+// (16 warps) adds the positions it finished.
+// Bound: complex64 (26 qubits, 246 us, 0.65 of the copy rate) the input's loads and conversion; complex128 (24
+// qubits, 190 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
+// and on the integer pipe about as fast, so they are spread over both; the tensor cores work a quarter of the
+// time. Measured and left: one set of warps for input and output (281 us at 24 qubits), 8 output warps (208),
+// the next tile staged by cp.async (204), L2 prefetch of the next tile (212), the D_d to integers by F2I (213).
+// Every mbarrier wait is bounded (2 s); on expiry the kernel records DEVERR_TIMEOUT, waits once more (bounded)
+// for its MMAs, frees its tensor memory and returns.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "common.cuh"
+#include "internal.h"
+#include "tc_ptx.cuh"
+
+namespace qsim {
+namespace tcx {
+
+using namespace qsim::tc;
+
+constexpr int K = 5, D = 1 << K;   // targets (padded), complex columns of a tile
+constexpr int NR = 2 * D;          // reals of a row: K and N of one digit product
+constexpr int kRowBits = 7;        // 128 rows per tile (MMA M = 128)
+constexpr int kPlaneA = 128 * NR * 2;  // bytes of one digit plane of a tile (16 KiB)
+constexpr int kPlaneB = NR * NR * 2;   // bytes of one digit plane of U (8 KiB)
+
+template <typename R> struct Cfg;
+template <> struct Cfg<float> {
+    static constexpr int S = 4, ND = 4;        // digits; digit positions kept
+    static constexpr int BUF = 2;              // tiles in flight: A planes and accumulators
+    static constexpr int GROUPS = 1;           // commits per tile
+    static constexpr int IN = 16, OUT = 8, MMA = 1;  // warps: tile loads and digit planes; accumulators and stores; MMAs
+    static constexpr int kStepsU = 30;         // U in 2^-30 steps
+    __host__ __device__ static constexpr int group_end(int) { return S; }
+};
+template <> struct Cfg<double> {
+    static constexpr int S = 7, ND = 8;
+    static constexpr int BUF = 1;
+    static constexpr int GROUPS = 4;           // planes 0-1, 2-3, 4-5, 6
+    // Whole warpgroups, so that registers can move between them: launched with 72 a thread (28 warps, 64512 in
+    // all), the input takes 96, the output keeps 64, the MMA warpgroup (one warp works) 56: 64512.
+    static constexpr int IN = 8, OUT = 16, MMA = 4;
+    static constexpr int kRegIn = 96, kRegOut = 64, kRegMma = 56;
+    static constexpr int kStepsU = 54;
+    __host__ __device__ static constexpr int group_end(int g) { return g < 3 ? 2 * g + 2 : S; }
+};
+template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
+template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
+template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 1; }
+template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
+// planes, column offsets, row exponents of the input [2][IN / 4][128] and of tiles in flight
+// [row_slots][128], barriers, the TMEM slot, alignment
+template <typename R> constexpr size_t smem_bytes() {
+    return smem_planes<R>() + 8 * D + 4 * (2 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
+           8 * bars<R>() + 8 + 1024;
+}
+static_assert(smem_bytes<float>() <= 227 * 1024 && smem_bytes<double>() <= 227 * 1024, "");
+
+// How a thread moves its columns: one amplitude per access (lane = row); the columns of qubit 0 (target 0) as
+// one vector of two; the columns of qubits 0 and 1 (targets 0 and 1) as one 32-byte vector of four (complex64).
+enum Mode { kRows = 0, kPairs = 1, kQuads = 2 };
+
+struct Args {
+    int nS;              // 12 index bits covered by a tile
+    int spos[12];        // those bit positions, ascending
+    int rpos[kRowBits];  // row bit j <-> index bit rpos[j]
+    int tpos[K];         // column bit j <-> index bit tpos[j]
+    uint64_t ntiles;
+    int from_basis;      // the input is |basis>, generated in registers instead of read
+    uint64_t basis;
+    int32_t w[4];        // 2^30, 2^22, 2^14, 2^6 (as parameters, so that they stay multiplications)
+};
+
+__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                       uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 ad, bd;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 ad, {%1, %3};\n\t"
+        "mov.b64 bd, {%2, %3};\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %4, p;\n}"
+        :: "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
+}
+
+// `words` 32-bit words (2, 4 or 8) between registers and global memory, aligned to their size.
+template <int N> __device__ __forceinline__ void ld_words(const void* p, uint32_t* w) {
+    if constexpr (N == 8)
+        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                     : "l"(p) : "memory");
+    else if constexpr (N == 4)
+        asm volatile("ld.global.v4.b32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p) : "memory");
+    else
+        asm volatile("ld.global.v2.b32 {%0,%1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p) : "memory");
+}
+template <int N> __device__ __forceinline__ void st_words(void* p, const uint32_t* w) {
+    if constexpr (N == 8)
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                     :: "l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    else if constexpr (N == 4)
+        asm volatile("st.global.v4.b32 [%0], {%1,%2,%3,%4};"
+                     :: "l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+    else
+        asm volatile("st.global.v2.b32 [%0], {%1,%2};" :: "l"(p), "r"(w[0]), "r"(w[1]) : "memory");
+}
+
+// Rows whose largest exponent is below this are scaled up first (rare), so that a zero or subnormal amplitude
+// next to a larger one falls below the fixed-point step and needs no case of its own.
+template <typename R> constexpr uint32_t kLowE = sizeof(R) == 8 ? 64 : 32;
+template <typename R> constexpr int kLowScale = sizeof(R) == 8 ? 200 : 64;  // 2^200 (2^64)
+constexpr uint32_t kHighE = 1076;  // complex128 rows above it are scaled down by 2^-1000: to_fixed adds 1076 - E to exponents
+
+// The fixed-point value of a real whose row has largest biased exponent E, plus 128 in every base-256 digit
+// (so that the bytes of the result are the digits plus 128). |x| < 2^(E - 1022) maps to 2^54 steps. Two ways that
+// give the same value but for ties: shifts on the integer pipe (19 instructions), or a conversion, which the FP64
+// units run at two a cycle and SM. The input warps alternate them, so that both units work.
+__device__ __forceinline__ void to_fixed_int(uint32_t& lo, uint32_t& hi, uint32_t E) {
+    const uint32_t sh = min(E - ((hi >> 20) & 0x7FFu), 63u);
+    uint64_t v = (((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 2;  // four times the 53-bit significand
+    v = ((v >> sh) + 1) >> 1;                                                  // to nearest
+    const uint64_t s = (uint64_t)(int64_t)((int32_t)hi >> 31);
+    v = ((v ^ s) - s) + 0x0080808080808080ull;
+    lo = (uint32_t)v;
+    hi = (uint32_t)(v >> 32);
+}
+__device__ __forceinline__ void to_fixed_cvt(uint32_t& lo, uint32_t& hi, uint32_t E) {
+    // x 2^(1076 - E) by its exponent field; a zero or subnormal becomes a value below 2^-10, which rounds to 0
+    const double x = __hiloint2double((int)(hi + ((kHighE - E) << 20)), (int)lo);
+    const uint64_t v = (uint64_t)__double2ll_rn(x) + 0x0080808080808080ull;
+    lo = (uint32_t)v;
+    hi = (uint32_t)(v >> 32);
+}
+
+// Y * 2^(E - 1080) to nearest, for kLowE <= E <= 2039, likewise.
+__device__ __forceinline__ void to_double_int(int64_t Y, int E, uint32_t& lo, uint32_t& hi) {
+    const uint64_t a = (uint64_t)(Y < 0 ? -Y : Y);
+    const int lz = __clzll((long long)a);
+    const uint64_t t = a << lz;                                           // leading one at bit 63 (a = 0: see below)
+    uint64_t r = t >> 11;                                                 // 53 bits; to nearest, ties to even,
+    r += (((uint32_t)t & 0x7FFu) + ((uint32_t)r & 1u)) > 0x400u ? 1 : 0;  // which may carry to 2^53
+    const uint32_t h = (uint32_t)(r >> 32) + ((uint32_t)(E + 5 - lz) << 20);  // exponent less one: the leading one adds it
+    lo = (uint32_t)r;
+    hi = a ? h | ((uint32_t)(Y >> 32) & 0x80000000u) : 0u;
+}
+__device__ __forceinline__ void to_double_cvt(int64_t Y, int E, uint32_t& lo, uint32_t& hi) {
+    const double y = __ll2double_rn(Y);
+    const uint32_t h = (uint32_t)__double2hiint(y);
+    lo = (uint32_t)__double2loint(y);
+    hi = h ? h + ((uint32_t)(E - 1080) << 20) : 0u;
+}
+
+template <typename R, int MODE>
+__global__ void __launch_bounds__(threads<R>(), 1)
+k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a, const uint4* __restrict__ bops,
+            unsigned* __restrict__ err) {
+    using C = Cfg<R>;
+    using T = typename Amp<R>::T;
+    constexpr bool DBL = sizeof(R) == 8;
+    constexpr int S = C::S, ND = C::ND, BUF = C::BUF, GROUPS = C::GROUPS, kIn = C::IN, kOut = C::OUT;
+    constexpr int CPI = 128 / kIn, CPO = 128 / kOut;  // complex columns per input and output thread
+    constexpr int AW = sizeof(T) / 4;            // words per amplitude
+    constexpr int VEC = MODE == kQuads ? 4 : (MODE == kPairs ? 2 : 1);  // amplitudes per access
+    constexpr int W = CPI * AW;                  // words of an input thread's share of a tile
+    constexpr uint32_t TCOLS = 64 * ND * BUF;
+    static_assert(TCOLS == 512 && VEC * AW <= 8, "");
+
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* sA = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char* sB = sA + BUF * S * kPlaneA;
+    uint64_t* sCol = reinterpret_cast<uint64_t*>(sB + S * kPlaneB);
+    uint32_t* sE = reinterpret_cast<uint32_t*>(sCol + D);             // [2][kIn / 4][128]
+    int* sRow = reinterpret_cast<int*>(sE + 2 * (kIn / 4) * 128);     // [row_slots][128]
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sRow + row_slots<R>() * 128);
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + bars<R>());
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // barriers: per buffer, A stored (full), accumulators read (freed), MMAs of a plane group retired (done)
+    auto full = [&](uint32_t b) { return smem_u32(mbar + b); };
+    auto freed = [&](uint32_t b) { return smem_u32(mbar + BUF + b); };
+    auto done = [&](uint32_t b, int g) { return smem_u32(mbar + (2 + g) * BUF + b); };
+    const uint32_t bbar = smem_u32(mbar + bars<R>() - 1);
+    for (int c = tid; c < D; c += threads<R>()) sCol[c] = deposit((uint64_t)c, a.tpos, K);
+    if (tid == 0) {
+        for (int j = 0; j < bars<R>(); ++j) {
+            const int count = j < BUF ? kIn : (j < 2 * BUF ? kOut : 1);
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar + j)), "r"(count) : "memory");
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(tslot)), "r"(TCOLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tbase = *tslot;
+    // programmatic dependent launch: the set-up above overlapped the previous kernel's tail
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t t0 = blockIdx.x, G = gridDim.x;  // (fewer than 2^32 tiles: checked by the host)
+    const uint32_t m = t0 < a.ntiles ? (uint32_t)((a.ntiles - t0 + G - 1) / G) : 0u;  // tiles of this CTA
+    auto tile = [&](uint32_t i) { return (uint64_t)t0 + (uint64_t)i * G; };
+    auto buf = [&](uint32_t i) { return i % BUF; };
+    auto par = [&](uint32_t i) { return (i / BUF) & 1; };  // phase parity of tile i on its buffer's barriers
+    // warp-uniform bounded wait (the TMEM accesses that follow are .sync.aligned)
+    auto wait = [&](uint32_t bar, uint32_t p) -> bool {
+        const bool ok = !__any_sync(0xffffffffu, !mbar_wait_bounded(bar, p));
+        fence_after();
+        return ok;
+    };
+    // input and output warps: thread = row r of the tile, columns c0 ..
+    const int quad = warp & 3, r = quad * 32 + lane;
+
+    bool bad = false;
+    if (warp >= kIn + kOut) {
+        // ---- MMA issuer ----
+        if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegMma));
+        if (warp == kIn + kOut && lane == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bbar), "r"(S * kPlaneB) : "memory");
+#pragma unroll 1
+            for (int j = 0; j < S; ++j)
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             :: "r"(smem_u32(sB) + j * kPlaneB), "l"(reinterpret_cast<const char*>(bops) + j * kPlaneB),
+                                "r"(kPlaneB), "r"(bbar) : "memory");
+            const uint64_t d0 = sdesc_sw128(smem_u32(sA));
+            const uint32_t hi = (uint32_t)(d0 >> 32), alo0 = (uint32_t)d0;
+            const uint32_t blo = (uint32_t)sdesc_sw128(smem_u32(sB));
+            uint32_t issued = 0;  // tiles issued
+            bad = !mbar_wait_bounded(bbar, 0);
+            if (bad) mbar_wait_bounded(bbar, 0);  // once more for the copy still in flight
+            for (uint32_t i = 0; i < m && !bad; ++i) {
+                const uint32_t b = buf(i);
+                if (i >= BUF && !mbar_wait_bounded(freed(b), par(i - BUF))) { bad = true; break; }
+                if (!mbar_wait_bounded(full(b), par(i))) { bad = true; break; }
+                fence_after();
+                const uint32_t alo = alo0 + b * ((S * kPlaneA) >> 4), dcol = tbase + b * 64 * ND;
+                int g = 0;
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    // plane s against U_0 .. U_{cnt-1}, into D_s .. D_{s+cnt-1}; the digit positions that no plane
+                    // before s reached (all of them for s = 0, the last one for s = 1 when ND > S) start here
+                    const int cnt = S < ND - s ? S : ND - s;
+                    const bool split = s == 1 && ND > S;  // U_{S-1} apart: it starts D_{ND-1}
+#pragma unroll
+                    for (int u = 0; u < cnt;) {
+                        int w = cnt - u < 4 ? cnt - u : 4;
+                        if (split && u < cnt - 1 && u + w > cnt - 1) w = cnt - 1 - u;
+                        const bool fresh = s == 0 || (split && u == cnt - 1);
+                        const uint32_t idesc = (1u << 4) | ((uint32_t)((64 * w) >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+#pragma unroll
+                        for (int kk = 0; kk < NR / 16; ++kk)
+                            mma_ss(dcol + 64 * (s + u), alo + ((s * kPlaneA + 32 * kk) >> 4), blo + ((u * kPlaneB + 32 * kk) >> 4),
+                                   hi, idesc, fresh && kk == 0 ? 0u : 1u);
+                        u += w;
+                    }
+                    if (s + 1 == C::group_end(g)) {
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(done(b, g)) : "memory");
+                        ++g;
+                    }
+                }
+                issued = i + 1;
+            }
+            if (bad) {
+                atomicOr(err, DEVERR_TIMEOUT);
+                if (issued) mbar_wait_bounded(done(buf(issued - 1), GROUPS - 1), par(issued - 1));  // the MMAs already issued
+            }
+        }
+        __syncwarp();
+    } else if (warp < kIn) {
+        // ---- input: load a tile, convert it to fixed point, write its digit planes ----
+        if constexpr (DBL) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegIn));
+        const int c0 = CPI * (warp >> 2);
+        const volatile uint64_t* vCol = sCol + c0;
+        const T* const prow = psi + deposit((uint64_t)r, a.rpos, kRowBits);
+        unsigned char* const arow = sA + (r >> 3) * 1024 + (r & 7) * 128;
+        auto load_tile = [&](uint32_t (&X)[W], uint64_t t) {
+            const uint64_t b = insert_zeros(t, a.spos, a.nS);
+            if (a.from_basis) {
+                const uint64_t rb = b + deposit((uint64_t)r, a.rpos, kRowBits);
+#pragma unroll
+                for (int j = 0; j < CPI; ++j) {
+#pragma unroll
+                    for (int k = 0; k < AW; ++k) X[AW * j + k] = 0;
+                    if (rb + vCol[j] == a.basis) X[AW * j + (DBL ? 1 : 0)] = DBL ? 0x3FF00000u : 0x3F800000u;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < CPI; j += VEC) ld_words<VEC * AW>(prow + b + vCol[j], X + AW * j);
+            }
+        };
+        // The largest magnitude (upper word) of the thread's reals: waits for the tile's loads, so that those of the
+        // next tile can start.
+        auto top = [&](const uint32_t (&X)[W]) {
+            uint32_t e = 0;
+#pragma unroll
+            for (int j = DBL ? 1 : 0; j < W; j += DBL ? 2 : 1) e = max(e, X[j] & 0x7FFFFFFFu);
+            asm volatile("" : "+r"(e) :: "memory");  // before any later load is issued (loads share scoreboards)
+            return e;
+        };
+        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow.
+        auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) {
+            constexpr int EB = DBL ? 20 : 23;  // exponent position in a real's upper word
+            uint32_t* const ex = sE + (i & 1) * (kIn / 4 * 128) + r;
+            ex[(warp >> 2) * 128] = e;
+            asm volatile("bar.sync %0, %1;" :: "r"(1 + quad), "n"(kIn * 8) : "memory");  // the warps of the quadrant
+#pragma unroll
+            for (int k = 0; k < kIn / 4; ++k) e = max(e, ex[k * 128]);
+            uint32_t E = max(e >> EB, kLowE<R>);
+            int scaled = 0;  // the row was multiplied by 2^scaled
+            const bool low = e != 0 && (e >> EB) < kLowE<R>, high = DBL && (e >> EB) > kHighE;
+            if (__any_sync(0xffffffffu, low || high)) {
+                if (low || high) {
+                    if constexpr (DBL) {
+                        scaled = low ? kLowScale<R> : -1000;
+                        const double f = __longlong_as_double((long long)(1023 + scaled) << 52);
+                        const uint32_t E2 = (uint32_t)__double2hiint(__hiloint2double((int)e, low ? -1 : 0) * f) >> EB;
+                        E = (e >> EB) == 0x7FF ? kHighE : max(E2, kLowE<R>);
+                        if ((e >> EB) == 0x7FF) scaled = (int)kHighE - 0x7FF;  // E - scaled says so
+#pragma unroll
+                        for (int j = 0; j < W; j += 2) {
+                            const double x = __hiloint2double((int)X[j + 1], (int)X[j]) * f;
+                            X[j] = (uint32_t)__double2loint(x);
+                            X[j + 1] = (uint32_t)__double2hiint(x);
+                        }
+                    } else {
+                        scaled = kLowScale<R>;
+                        const float f = __uint_as_float((uint32_t)(127 + kLowScale<R>) << 23);
+                        E = max(__float_as_uint(__uint_as_float(e) * f) >> EB, kLowE<R>);
+#pragma unroll
+                        for (int j = 0; j < W; ++j) X[j] = __float_as_uint(__uint_as_float(X[j]) * f);
+                    }
+                }
+            }
+            // read by the output warps after this tile's MMAs. The planes of tile i - 1 were stored, so the MMAs of
+            // tile i - 1 - BUF have run, for which tile i - 1 - 2 BUF had been read: 2 BUF + 1 slots or more will do
+            if (warp < 4) sRow[i % row_slots<R>() * 128 + r] = (int)E - scaled;
+            if constexpr (DBL) {
+#pragma unroll
+                for (int j = 0; j < W; j += 2) {
+                    if (j & 6) to_fixed_int(X[j], X[j + 1], E);
+                    else to_fixed_cvt(X[j], X[j + 1], E);
+                }
+            } else {
+                const float up = __uint_as_float((283u - min(E, 255u)) << 23);  // 2^(156 - E): |x| < 2^(E - 126) to 2^30 steps
+#pragma unroll
+                for (int j = 0; j < W; ++j) X[j] = (uint32_t)__float2int_rn(__uint_as_float(X[j]) * up) + 0x80808080u;
+            }
+        };
+        // Digit plane s of the tile: byte S-1-s of every real, less 128, as FP16 pairs (re, im).
+        auto store_plane = [&](const uint32_t (&X)[W], int s, uint32_t b) {
+            const int by = (S - 1 - s) & 3, wd = DBL ? (S - 1 - s) >> 2 : 0;
+            const uint32_t sel = (uint32_t)by | ((uint32_t)(4 + by) << 8);  // that byte of re to byte 0, of im to byte 2
+            unsigned char* const ap = arow + b * (S * kPlaneA) + s * kPlaneA;
+#pragma unroll
+            for (int q = 0; q < CPI / 4; ++q) {
+                uint32_t h[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int j = AW * (4 * q + k);
+                    const uint32_t v = (__byte_perm(X[j + wd], X[j + AW / 2 + wd], sel) & 0x00FF00FFu) | 0x64006400u;  // 1024 + byte
+                    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6480)));  // - 1152
+                    h[k] = *reinterpret_cast<const uint32_t*>(&d);
+                }
+                *reinterpret_cast<uint4*>(ap + (((c0 / 4 + q) ^ (r & 7)) << 4)) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+        };
+        // Tile i: fixed point, then its planes as the planes of tile i - BUF retire.
+        auto put = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) -> bool {
+            convert(X, i, e);
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                if (i >= BUF && !wait(done(buf(i), g), par(i - BUF))) return false;
+#pragma unroll
+                for (int s = g ? C::group_end(g - 1) : 0; s < C::group_end(g); ++s) store_plane(X, s, buf(i));
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full(buf(i)));
+            return true;
+        };
+        if constexpr (DBL) {
+            uint32_t X[W];
+            for (uint32_t i = 0; i < m; ++i) {
+                load_tile(X, tile(i));
+                if (!put(X, i, top(X))) { bad = true; break; }
+            }
+        } else {  // one tile ahead in registers
+            uint32_t XA[W], XB[W];
+            if (m > 0) load_tile(XA, tile(0));
+            for (uint32_t i = 0; i < m; i += 2) {
+                const uint32_t ea = top(XA);
+                if (i + 1 < m) load_tile(XB, tile(i + 1));
+                if (!put(XA, i, ea)) { bad = true; break; }
+                if (i + 1 >= m) break;
+                const uint32_t eb = top(XB);
+                if (i + 2 < m) load_tile(XA, tile(i + 2));
+                if (!put(XB, i + 1, eb)) { bad = true; break; }
+            }
+        }
+        if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
+    } else {
+        // ---- output: sum the digit positions, convert back, store ----
+        if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegOut));
+        const int c0 = CPO * ((warp - kIn) >> 2);
+        const volatile uint64_t* vCol = sCol + c0;
+        T* const prow = psi + deposit((uint64_t)r, a.rpos, kRowBits);
+        const uint32_t trow = tbase + ((uint32_t)(quad * 32) << 16) + 2 * c0;
+        constexpr int kNan = DBL ? 0x7FF : 0xFF;  // the row held an infinity or NaN
+        // whether every |D_d| <= 2^22: the digits of X are at most 128, so the sum of a row of U's bounds them
+        const int* const sums = reinterpret_cast<const int*>(reinterpret_cast<const char*>(bops) + S * kPlaneB);
+        [[maybe_unused]] const bool bounded = !__any_sync(0xffffffffu, max(sums[lane], sums[lane + 32]) > (1 << 15));
+        auto finish = [&](uint32_t i) {  // the accumulators have been read
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(freed(buf(i)));
+        };
+        for (uint32_t i = 0; i < m; ++i) {
+            const uint32_t td = trow + buf(i) * 64 * ND;
+            if constexpr (DBL) {
+                // Y = sum_d D_d 2^(46 - 8d), the last two positions together and rounded; y = Y 2^(E - 1080).
+                // The integers come as q + kMagic: the bits of D + 1.5 2^23 where |D| <= 2^22, else by conversion
+                // (on the XU unit, which would bound this kernel); Y starts at what that adds.
+                constexpr uint32_t kMagic = 0x4B400000u;
+                constexpr int64_t kOff = (int64_t)kMagic * ((1ll << 30) + (1ll << 22) + (1ll << 14) + (1ll << 6));
+                constexpr uint64_t kY0 = 0ull - (uint64_t)kOff - ((uint64_t)((kMagic << 14) + (kMagic << 6)) << 32);
+                int64_t Y[2 * CPO];
+#pragma unroll
+                for (int g = 0; g < GROUPS; ++g) {
+                    if (!wait(done(buf(i), g), par(i))) { bad = true; break; }
+#pragma unroll
+                    for (int c = 0; c < 2 * CPO; c += 8) {
+                        uint32_t v[8], v2[8];
+                        tmem_ld<8>(td + 64 * (2 * g) + c, v);
+                        tmem_ld<8>(td + 64 * (2 * g + 1) + c, v2);
+                        wait_ld();
+                        if (bounded) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                v[j] = __float_as_uint(__fadd_rn(__uint_as_float(v[j]), 12582912.0f));
+                                v2[j] = __float_as_uint(__fadd_rn(__uint_as_float(v2[j]), 12582912.0f));
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                v[j] = (uint32_t)__float2int_rn(__uint_as_float(v[j])) + kMagic;
+                                v2[j] = (uint32_t)__float2int_rn(__uint_as_float(v2[j])) + kMagic;
+                            }
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if (g == 0) {
+                                const uint32_t h = (v[j] << 14) + (v2[j] << 6) + (uint32_t)(kY0 >> 32);
+                                Y[c + j] = (int64_t)(((uint64_t)h << 32) | (uint32_t)kY0);
+                            } else if (g < 3) {
+                                asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Y[c + j]) : "r"(v[j]), "r"(a.w[2 * g - 2]));
+                                asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Y[c + j]) : "r"(v2[j]), "r"(a.w[2 * g - 1]));
+                            } else {
+                                Y[c + j] += (int32_t)((v[j] << 8) + v2[j] + (512u - (kMagic << 8) - kMagic)) >> 10;
+                            }
+                        }
+                    }
+                }
+                if (bad) break;
+                const int E = sRow[i % row_slots<R>() * 128 + r];
+                finish(i);
+                // rows near either end of the exponent range take a multiplication that can overflow or underflow
+                const bool rare = __any_sync(0xffffffffu, E < (int)kLowE<R> || E > kNan - 8);
+                T* const pt = prow + insert_zeros(tile(i), a.spos, a.nS);
+#pragma unroll
+                for (int j = 0; j < CPO; j += VEC) {
+                    uint32_t w[VEC * AW];
+#pragma unroll
+                    for (int k = 0; k < 2 * VEC; ++k) {
+                        const int64_t Yk = Y[2 * j + k];
+                        if (rare) {  // two steps: 2^(E - 1080) alone may be below the range
+                            double y = __ll2double_rn(Yk) * 0x1p-58;
+                            y = E >= kNan ? __hiloint2double(0x7FF80000, 0)
+                                          : E > 0 ? (y * 2.0) * __hiloint2double(E << 20, 0)
+                                                  : (y * __hiloint2double((E + 256) << 20, 0)) * 0x1p-255;
+                            w[2 * k] = (uint32_t)__double2loint(y);
+                            w[2 * k + 1] = (uint32_t)__double2hiint(y);
+                        } else if (((2 * j + k) & 3) == 0) {
+                            to_double_int(Yk, E, w[2 * k], w[2 * k + 1]);
+                        } else {
+                            to_double_cvt(Yk, E, w[2 * k], w[2 * k + 1]);
+                        }
+                    }
+                    st_words<VEC * AW>(pt + vCol[j], w);
+                }
+            } else {
+                // y = 2^(E - 138) sum_d D_d 2^(-8d)
+                if (!wait(done(buf(i), 0), par(i))) { bad = true; break; }
+                const int E = sRow[i % row_slots<R>() * 128 + r];
+                const bool rare = __any_sync(0xffffffffu, E < (int)kLowE<R> || E > kNan - 8);
+                const float sc = __uint_as_float((uint32_t)(E - 11) << 23);
+                T* const pt = prow + insert_zeros(tile(i), a.spos, a.nS);
+#pragma unroll
+                for (int c = 0; c < 2 * CPO; c += 8) {
+                    uint32_t v[4][8], w[8];
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) tmem_ld<8>(td + 64 * d + c, v[d]);
+                    wait_ld();
+                    if (c + 8 == 2 * CPO) finish(i);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float y = __uint_as_float(v[3][j]);
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[2][j]));
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[1][j]));
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
+                        if (rare) {
+                            y *= 0x1p-12f;
+                            y = E >= kNan ? __uint_as_float(0x7FC00000u)
+                                          : E > 0 ? (y * 2.0f) * __uint_as_float((uint32_t)E << 23)
+                                                  : (y * __uint_as_float((uint32_t)(E + 96) << 23)) * 0x1p-95f;
+                        } else {
+                            y *= sc;
+                        }
+                        w[j] = __float_as_uint(y);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
+                }
+            }
+        }
+        if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tbase), "r"(TCOLS) : "memory");
+    }
+}
+
+// The digit planes of U (x I on the padding columns): real form B[2i][2c] = Re U_ic, B[2i][2c+1] = -Im U_ic,
+// B[2i+1][2c] = Im U_ic, B[2i+1][2c+1] = Re U_ic in fixed point, plane t = digit t (most significant first).
+// After the planes, the sum of |digits| over all planes of each row (64 integers). One block per row n.
+template <typename R>
+__global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U, int k, unsigned char* __restrict__ out) {
+    using C = Cfg<R>;
+    const int Du = 1 << k, n = blockIdx.x, kk = threadIdx.x, i = n >> 1, c = kk >> 1;
+    __shared__ int total[2];
+    double v = 0.0;
+    if ((i >> k) == (c >> k)) {
+        const int e = 2 * ((i & (Du - 1)) * Du + (c & (Du - 1)));
+        v = (n & 1) == (kk & 1) ? U[e] : ((n & 1) ? U[e + 1] : -U[e + 1]);
+    }
+    const uint64_t f = (uint64_t)__double2ll_rn(scalbn(v, C::kStepsU)) + (sizeof(R) == 8 ? 0x0080808080808080ull : 0x80808080ull);
+    const uint32_t off = sw128_offset(n, kk, NR, 2);
+    int sum = 0;
+    for (int t = 0; t < C::S; ++t) {
+        const int b = (int)((f >> (8 * (C::S - 1 - t))) & 0xFF) - 128;
+        sum += b < 0 ? -b : b;
+        *reinterpret_cast<__half*>(out + t * kPlaneB + off) = __int2half_rn(b);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((kk & 31) == 0) total[kk >> 5] = sum;
+    __syncthreads();
+    if (kk == 0) reinterpret_cast<int*>(out + C::S * kPlaneB)[n] = total[0] + total[1];
+}
+
+}  // namespace tcx
+
+bool tcx_supported(int n, int k) { return k >= 1 && k <= tcx::K && n >= tcx::K + tcx::kRowBits && n <= 43; }
+
+size_t tcx_operand_bytes(int dtype) {
+    return (size_t)tcx::kPlaneB * (dtype == QSIM_C64 ? tcx::Cfg<float>::S : tcx::Cfg<double>::S) + sizeof(int) * tcx::NR;
+}
+
+cudaError_t launch_tcx_prepare(int dtype, const double* dU, int k, void* dB, cudaStream_t s) {
+    if (k < 1 || k > tcx::K) return cudaErrorInvalidValue;
+    unsigned char* out = static_cast<unsigned char*>(dB);
+    if (dtype == QSIM_C64) tcx::k_tcx_prepare<float><<<tcx::NR, tcx::NR, 0, s>>>(dU, k, out);
+    else tcx::k_tcx_prepare<double><<<tcx::NR, tcx::NR, 0, s>>>(dU, k, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targets, const void* dB, unsigned* dev_err,
+                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis) {
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(psi);
+    if (!tcx_supported(n, k) || (reinterpret_cast<uintptr_t>(dB) & 15) != 0 || (addr & 15) != 0) return cudaErrorInvalidValue;
+    tcx::Args a;
+    std::memset(&a, 0, sizeof(a));
+    uint64_t tmask = 0;
+    for (int j = 0; j < k; ++j) {
+        if (targets[j] < 0 || targets[j] >= n || ((tmask >> targets[j]) & 1)) return cudaErrorInvalidValue;
+        a.tpos[j] = targets[j];
+        tmask |= 1ull << targets[j];
+    }
+    for (int q = n - 1, j = k; j < tcx::K; --q)  // padding: the highest idle qubits
+        if (!((tmask >> q) & 1)) {
+            a.tpos[j++] = q;
+            tmask |= 1ull << q;
+        }
+    int nr = 0;
+    for (int q = 0; q < n && nr < tcx::kRowBits; ++q)
+        if (!((tmask >> q) & 1)) a.rpos[nr++] = q;
+    uint64_t smask = tmask;
+    for (int j = 0; j < tcx::kRowBits; ++j) smask |= 1ull << a.rpos[j];
+    for (int q = 0; q < n; ++q)
+        if ((smask >> q) & 1) a.spos[a.nS++] = q;
+    a.ntiles = 1ull << (n - a.nS);
+    if (a.ntiles >> 32) return cudaErrorInvalidValue;  // 32-bit tile counters in the kernel
+    if (from_basis) {
+        a.from_basis = 1;
+        a.basis = *from_basis;
+    }
+    for (int j = 0; j < 4; ++j) a.w[j] = 1 << (30 - 8 * j);
+    auto launch = [&](auto kern, auto* p, int threads, size_t smem) -> cudaError_t {
+        cudaError_t e = smem_optin(reinterpret_cast<const void*>(kern), (int)smem);
+        if (e != cudaSuccess) return e;
+        // programmatic dependent launch, as for the other block kernels (griddepcontrol.wait before any access)
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)std::min<uint64_t>((uint64_t)d.num_sms, a.ntiles), 1, 1);
+        cfg.blockDim = dim3((unsigned)threads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, p, a, reinterpret_cast<const uint4*>(dB), dev_err);
+    };
+    using namespace tcx;
+    if (dtype == QSIM_C64) {
+        float2* p = reinterpret_cast<float2*>(psi);
+        constexpr size_t sm = smem_bytes<float>();
+        constexpr int th = threads<float>();
+        if (a.tpos[0] == 0 && a.tpos[1] == 1 && (addr & 31) == 0) return launch(k_tcx_block<float, kQuads>, p, th, sm);
+        if (a.tpos[0] == 0) return launch(k_tcx_block<float, kPairs>, p, th, sm);
+        return launch(k_tcx_block<float, kRows>, p, th, sm);
+    }
+    double2* p = reinterpret_cast<double2*>(psi);
+    constexpr size_t sm = smem_bytes<double>();
+    constexpr int th = threads<double>();
+    if (a.tpos[0] == 0 && (addr & 31) == 0) return launch(k_tcx_block<double, kPairs>, p, th, sm);
+    return launch(k_tcx_block<double, kRows>, p, th, sm);
+}
+
+}  // namespace qsim

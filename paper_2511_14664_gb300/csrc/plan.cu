@@ -46,11 +46,28 @@ struct PlanOp {
     PhaseForm form;            // OP_PHASE (and the epilogue it becomes): the combined phase
     bool has_epi = false;      // OP_TC: the output gets the phase of `form` (the pass that followed it)
     bool lines = false;        // OP_TC: line-group data path (B prepared in its column order)
+    bool tcx = false;          // OP_DENSE_SMALL, OP_DENSE_TILE of a composed block: run on the tensor cores in
+                               // the state's own precision (k_tcx.cu); its operand is at dev_off
     TcEpiPacked epi;           // OP_TC with has_epi: launch parameters; tables at epi_off
     size_t epi_off = 0;
     int targets2[6] = {0};     // OP_TC_PAIR: the second block's targets (the first block's are `targets`)
     int compose_idx2 = -1;     // OP_TC_PAIR: the second block's composition
 };
+
+// Where a composed block of k qubits leaves the CUDA cores for k_tcx.cu, by the time of one pass (microseconds, CUDA
+// cores / k_tcx, targets from qubit 6 up): complex128 k = 1 n = 18 / 19 / 20: 8.3 / 11.6, 12.4 / 11.8, 20.6 / 16.5;
+// k = 2 n = 18 / 19: 11.0 / 11.5, 22.6 / 11.8; k = 3 n = 17: 12.4 / 11.4; k = 5 n = 17: 67.7 / 11.5, n = 24: 3457 / 190.
+// complex64 k = 5 n = 18 / 19: 6.2 / 6.4, 8.2 / 6.5, n = 26: 461 / 246; k = 4 n = 20 / 21 / 24: 21.6 / 8.5, 11.6 / 12.9,
+// 61.5 / 66.2, and with qubit 0 among the targets n = 24: 129 / 79. Below 17 qubits plans run resident (k_small.cu).
+constexpr int kTcxMinQubits = 17;
+static bool tcx_pays(int dtype, int n, int k, const int* targets) {
+    if (dtype == QSIM_C128) return n >= (k == 1 ? 20 : (k == 2 ? 19 : kTcxMinQubits));
+    if (k == 5) return n >= kTcxMinQubits;  // (level up to 18, and the error is smaller)
+    if (k != 4 || n < kTcxMinQubits) return false;
+    bool q0 = false;
+    for (int j = 0; j < k; ++j) q0 = q0 || targets[j] == 0;
+    return n <= 20 || q0;
+}
 
 struct PlanExtra {
     size_t epi_scratch_off = 0;  // per-tile factors of phase epilogues (shared: passes run in order)
@@ -451,6 +468,12 @@ static int enqueue_ops(qsim_state* h, const qsim_plan* p, size_t first = 0, size
     for (size_t oi = first; oi < last; ++oi) {
         const PlanOp& op = p->ops[oi];
         const uint64_t* fb = oi == first ? first_from_basis : nullptr;
+        if (op.tcx) {
+            e = launch_tcx_apply(h->dtype, h->psi, h->n, op.k, op.targets, static_cast<char*>(p->dbuf) + op.dev_off,
+                                 h->derr, h->stream, h->dev, fb);
+            if (e != cudaSuccess) return cuda_fail(e, "plan pass launch");
+            continue;
+        }
         switch (op.kind) {
             case OP_DENSE_SMALL:
                 e = launch_dense_small(h->dtype, h->psi, h->n, op.k, op.targets, op.nc, op.controls, op.mat.data(),
@@ -572,6 +595,11 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     // 7-qubit tensor-core blocks need n >= 14 (a tile is 7 row bits x 7 targets); plans with global qubits
     // keep 6-qubit blocks
     if (!dry && kmax == 7 && (n < 14 || remap_later)) kmax = 6;
+    // composed blocks in the state's own precision on the tensor cores (k_tcx.cu): up to 5 qubits, so wider
+    // groupings, which would run on CUDA cores, stay at 5
+    const bool own_prec = dtype == QSIM_C128 || opts.precision == QSIM_PREC_SIMT;
+    const bool tcx_ok = !dry && opts.mode == QSIM_RUN_FUSED && own_prec && n >= kTcxMinQubits;
+    if (tcx_ok && kmax == 6) kmax = 5;
     const bool tc7 = kmax == 7 && opts.precision == QSIM_PREC_FP16X3 && dtype == QSIM_C64 && n >= 14;
     // 7-qubit blocks keep off qubits 0..2: on those the 7-qubit kernel moves partly used lines (4.0-5.5 ms at 30
     // qubits against 2.9-3.2 ms above them), while 6-qubit blocks there have the line-group and pair-rows paths
@@ -816,12 +844,13 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
             // the larger operand
             const int room_prec = opts.precision == QSIM_PREC_FP16X3 ? QSIM_PREC_TF32X3 : opts.precision;
             dev_bytes = align(dev_bytes + std::max(tc_operand_bytes(kb, opts.precision), tc_operand_bytes(kb, room_prec)));
-        } else if (kb <= 4) {
-            op.kind = OP_DENSE_SMALL;
         } else {
-            op.kind = OP_DENSE_TILE;
-            op.dev_off = dev_bytes;
-            dev_bytes = align(dev_bytes + (amp << (2 * kb)));
+            op.kind = kb <= 4 ? OP_DENSE_SMALL : OP_DENSE_TILE;
+            op.tcx = tcx_ok && op.nc == 0 && tcx_supported(n, kb) && tcx_pays(dtype, n, kb, op.targets);
+            if (op.tcx || op.kind == OP_DENSE_TILE) {
+                op.dev_off = dev_bytes;
+                dev_bytes = align(dev_bytes + (op.tcx ? tcx_operand_bytes(dtype) : amp << (2 * kb)));
+            }
         }
         pending.push_back({(int)p->ops.size(), op.kind, kb});
         p->ops.push_back(std::move(op));
@@ -902,7 +931,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     bool small = !opts.launch_per_pass && n <= kSmallMaxQubits && !(opts.local_qubits > 0 && opts.local_qubits < n) &&
                  !p->ops.empty();
     for (const PlanOp& op : p->ops)
-        small = small && ((op.kind == OP_DENSE_SMALL && op.k <= 4) || (op.kind == OP_DENSE_TILE && op.k == 5) ||
+        small = small && !op.tcx && ((op.kind == OP_DENSE_SMALL && op.k <= 4) || (op.kind == OP_DENSE_TILE && op.k == 5) ||
                           (op.kind == OP_DIAG && op.k <= 6) || op.kind == OP_PHASE);
     const size_t off_small = align(off_cg + sizeof(ComposeGate) * cgates.size());
     const size_t total = off_small + (small ? align(small_program_bytes(dtype, (int)p->ops.size())) : 0) + 1024;
@@ -949,6 +978,8 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
                 e = launch_tc_prepare(U, pd.kb, op.precision, op.lines, base + op.dev_off, s,
                                       op.has_epi ? reinterpret_cast<const double*>(base + op.epi_off + op.epi.off_rowphase)
                                                  : nullptr);
+            } else if (op.tcx) {
+                e = launch_tcx_prepare(dtype, U, pd.kb, base + op.dev_off, s);
             } else if (pd.kind == OP_DENSE_TILE && !(small && pd.kb == 5)) {
                 e = launch_convert_matrix(dtype, U, base + op.dev_off, 2 * (int64_t)D * D, s);
             } else {
@@ -1280,7 +1311,8 @@ int qsim_plan_execute_from_basis(qsim_h h, qsim_plan_h p, uint64_t x, int64_t co
     if (count > nops) { set_error("pass range out of bounds"); return QSIM_EINVAL; }
     // a first tensor-core block (any precision but BF16x6; block pairs and 7-qubit blocks too) generates |x>
     // as its input and writes every amplitude
-    if (count > 0 && ((p->ops[0].kind == OP_TC && p->ops[0].precision != QSIM_PREC_BF16X6) || p->ops[0].kind == OP_TC_PAIR))
+    if (count > 0 && ((p->ops[0].kind == OP_TC && p->ops[0].precision != QSIM_PREC_BF16X6) || p->ops[0].kind == OP_TC_PAIR ||
+                      p->ops[0].tcx))
         return enqueue_ops(h, p, 0, (size_t)count, &x);
     // a resident plan sets |x> itself, in the same launch
     if (p->small && count == nops) return enqueue_ops(h, p, 0, (size_t)count, &x);

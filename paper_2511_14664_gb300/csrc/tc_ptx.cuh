@@ -32,6 +32,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t phase) {
 
 // Wait for the mbarrier phase with a 2-second limit; false on expiry.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t phase) {
+    if (mbar_try_wait(addr, phase)) return true;
     const uint64_t t0 = globaltimer();
     while (!mbar_try_wait(addr, phase)) {
         if (globaltimer() - t0 > 2000000000ull) return false;
