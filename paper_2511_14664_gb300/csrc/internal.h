@@ -97,6 +97,31 @@ void phase_pack(const PhaseForm& f, int dtype, std::vector<unsigned char>& out, 
 cudaError_t launch_phase(int dtype, void* psi, int n, const void* dtab, const PhasePacked& pk, cudaStream_t s,
                          const DevInfo& d);
 
+// ---- many gates of a per-gate plan in one pass over the state (k_tilegates.cu) --------------------------------
+struct TileGate {
+    bool ok = false;             // tile_gate_ok: may join a group
+    bool diag = false;
+    int k = 0, nc = 0;
+    int q[2] = {0, 0};           // targets; for a diagonal (k = 1 or 2, nc = 0) all its qubits
+    int ctl[QSIM_MAX_CONTROLS] = {0};
+    uint64_t tmask = 0, all = 0; // targets; targets and controls
+    std::vector<double> mat;     // 2^k x 2^k, or the diagonal's 2^k entries (interleaved)
+};
+struct TileGroup {
+    std::vector<int> members;    // gates, in the order they are applied
+    int pos[12] = {0};           // index bits of the tile
+    int steps = 0, ops = 0;      // steps 0: a single gate, which its own kernel runs
+    std::vector<uint64_t> prog;
+};
+constexpr int kTileMinQubits = 17;  // narrower plans run resident (k_small.cu)
+// Dense gates on 1 or 2 targets with any controls, diagonals on at most 2 qubits in all.
+bool tile_gate_ok(bool diag, int k, int nc);
+// The groups a list of gates is applied in (each gate once; gates that share a qubit keep their order unless both are
+// diagonal). n >= 12.
+std::vector<TileGroup> tile_groups(int dtype, int n, const std::vector<TileGate>& gates);
+// One pass of a group with a program (steps > 0).
+cudaError_t launch_tile_gates(int dtype, void* psi, int n, const TileGroup& grp, cudaStream_t s, const DevInfo& d);
+
 // ---- tensor-core fused block (k_tc.cu) ----------------------------------------------------------------------
 // Launch parameters of a phase epilogue (a phase form applied to the block's output): byte offsets of the
 // device tables and the counts.
