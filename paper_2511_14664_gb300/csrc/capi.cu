@@ -109,6 +109,10 @@ int check_device_error(qsim_state* h) {
     return QSIM_OK;
 }
 
+int check_passed_error(qsim_state* h) {
+    return *h->red.herr() ? check_device_error(h) : QSIM_OK;
+}
+
 // Apply one gate through the plain per-gate kernels (shared by qsim_apply_gate and plan execution).
 int apply_gate_plain(qsim_state* h, const int* targets, int k, const int* controls, int nc, const double* m) {
     cudaError_t e;
@@ -199,11 +203,12 @@ int qsim_create(int n, int dtype, void* dev_buf, size_t buf_bytes, void* stream,
     ok = ok && cudaMalloc(&h->red.seg, sizeof(double) * std::max<uint64_t>(2 * nseg, 2 * nseg10)) == cudaSuccess;
     ok = ok && cudaMalloc(&h->red.scan, sizeof(double) * (nseg + 8192)) == cudaSuccess;
     ok = ok && cudaMalloc(&h->red.result, sizeof(double) * 256) == cudaSuccess;
-    ok = ok && cudaMallocHost(&h->red.hresult, sizeof(double) * 256) == cudaSuccess;
+    ok = ok && cudaMallocHost(&h->red.hresult, sizeof(double) * (256 + kHostValues)) == cudaSuccess;
     ok = ok && cudaMalloc(&h->dmat, kDevMatBytes) == cudaSuccess;
     ok = ok && cudaMalloc(&h->dmat64, sizeof(double) * 2 * 16384) == cudaSuccess;  // a 7-qubit block
     ok = ok && cudaMalloc(&h->derr, sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMemset(h->derr, 0, sizeof(unsigned)) == cudaSuccess;
+    h->red.derr = h->derr;
     if (!ok) {
         cudaGetLastError();
         qsim_destroy(h);
@@ -347,7 +352,7 @@ int qsim_norm(qsim_h h, double* out) {
     if (!out) { set_error("NULL output"); return QSIM_EINVAL; }
     cudaError_t e = run_norm(h->dtype, h->psi, h->n, h->red, h->stream, h->dev, out);
     if (e != cudaSuccess) return cuda_fail(e, "norm");
-    return check_device_error(h);
+    return check_passed_error(h);
 }
 
 int qsim_probs(qsim_h h, const int* qubits, int nq, double* out) {
@@ -361,7 +366,7 @@ int qsim_probs(qsim_h h, const int* qubits, int nq, double* out) {
     }
     cudaError_t e = run_probs(h->dtype, h->psi, h->n, qubits, nq, h->red, h->stream, h->dev, out);
     if (e != cudaSuccess) return cuda_fail(e, "probs");
-    return check_device_error(h);
+    return check_passed_error(h);
 }
 
 int qsim_expect_pauli(qsim_h h, const char* paulis, double* out) {
@@ -374,7 +379,7 @@ int qsim_expect_pauli(qsim_h h, const char* paulis, double* out) {
     if (paulis[h->n] != '\0') { set_error("Pauli string longer than n"); return QSIM_EINVAL; }
     cudaError_t e = run_pauli(h->dtype, h->psi, h->n, paulis, h->red, h->stream, h->dev, out);
     if (e != cudaSuccess) return cuda_fail(e, "expect_pauli");
-    return check_device_error(h);
+    return check_passed_error(h);
 }
 
 int qsim_expect_z(qsim_h h, double* zi, double* zz) {
@@ -383,14 +388,15 @@ int qsim_expect_z(qsim_h h, double* zi, double* zz) {
     std::vector<double> zz_dummy(1);
     cudaError_t e = run_zstats(h->dtype, h->psi, h->n, h->red, h->stream, h->dev, zi, zz ? zz : zz_dummy.data());
     if (e != cudaSuccess) return cuda_fail(e, "expect_z");
-    return check_device_error(h);
+    return check_passed_error(h);
 }
 
-static int sample_common(qsim_h h, int64_t shots, uint64_t* out, const double* u_host, uint64_t seed,
-                         int seg_ready_bits = 0) {
-    if (!out) { set_error("NULL output"); return QSIM_EINVAL; }
+// With zi (and zz): the <Z> statistics first, whose segment sums the sampler then uses; one synchronisation for both.
+static int sample_common(qsim_h h, int64_t shots, uint64_t* out, const double* u_host, uint64_t seed, double* zi = nullptr,
+                         double* zz = nullptr) {
+    if (!out && shots > 0) { set_error("NULL output"); return QSIM_EINVAL; }
     if (shots < 0 || shots > (1ll << 31)) { set_error("shots outside 0..2^31"); return QSIM_EINVAL; }
-    if (shots == 0) return QSIM_OK;
+    if (shots == 0 && !zi) return QSIM_OK;
     if ((size_t)shots > h->samples_cap) {
         cudaFree(h->dsamples);
         cudaFree(h->du);
@@ -405,15 +411,24 @@ static int sample_common(qsim_h h, int64_t shots, uint64_t* out, const double* u
         }
         h->samples_cap = (size_t)shots;
     }
-    cudaError_t e;
-    if (u_host) e = cudaMemcpyAsync(h->du, u_host, sizeof(double) * shots, cudaMemcpyHostToDevice, h->stream);
-    else e = launch_uniforms(seed, shots, h->du, h->stream);
-    if (e == cudaSuccess)
-        e = run_sample(h->dtype, h->psi, h->n, h->du, shots, h->dsamples, h->red, h->stream, h->dev, seg_ready_bits);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, h->dsamples, sizeof(uint64_t) * shots, cudaMemcpyDeviceToHost, h->stream);
+    cudaError_t e = cudaSuccess;
+    if (zi) e = enqueue_zstats_host(h->dtype, h->psi, h->n, h->red, h->stream, h->dev);
+    const bool direct = shots <= kHostValues;  // written straight to pinned host memory
+    uint64_t* dst = direct ? reinterpret_cast<uint64_t*>(h->red.hvalues()) : h->dsamples;
+    if (e == cudaSuccess && shots > 0) {
+        if (u_host) e = cudaMemcpyAsync(h->du, u_host, sizeof(double) * shots, cudaMemcpyHostToDevice, h->stream);
+        else e = launch_uniforms(seed, shots, h->du, h->stream);
+        if (e == cudaSuccess)
+            e = run_sample(h->dtype, h->psi, h->n, h->du, shots, dst, h->red, h->stream, h->dev, zi ? zstats_segment_bits(h->n) : 0);
+        if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(out, dst, sizeof(uint64_t) * shots, cudaMemcpyDeviceToHost, h->stream);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "sample");
-    return check_device_error(h);
+    if (e != cudaSuccess) return cuda_fail(e, zi ? "expect_z_and_sample" : "sample");
+    const int rc = check_passed_error(h);
+    if (rc) return rc;
+    if (zi) read_zstats(h->red, h->n, zi, zz);
+    if (direct && shots > 0) std::memcpy(out, dst, sizeof(uint64_t) * shots);
+    return QSIM_OK;
 }
 
 int qsim_sample(qsim_h h, uint64_t seed, int64_t shots, uint64_t* out) {
@@ -425,12 +440,8 @@ int qsim_expect_z_and_sample(qsim_h h, double* zi, double* zz, uint64_t seed, in
     QSIM_CHECK_HANDLE(h);
     if (!zi || (!zz && h->n > 1) || (!out && shots > 0)) { set_error("NULL output"); return QSIM_EINVAL; }
     if (shots < 0 || shots > (1ll << 31)) { set_error("shots outside 0..2^31"); return QSIM_EINVAL; }
-    std::vector<double> zz_dummy(1);
-    cudaError_t e = run_zstats(h->dtype, h->psi, h->n, h->red, h->stream, h->dev, zi, zz ? zz : zz_dummy.data());
-    if (e != cudaSuccess) return cuda_fail(e, "expect_z_and_sample");
-    const int rc = check_device_error(h);
-    if (rc) return rc;
-    return sample_common(h, shots, out, nullptr, seed, zstats_segment_bits(h->n));
+    double zz_dummy[1];
+    return sample_common(h, shots, out, nullptr, seed, zi, zz ? zz : zz_dummy);
 }
 
 int qsim_sample_uniforms(qsim_h h, const double* u, int64_t shots, uint64_t* out) {
@@ -452,7 +463,7 @@ int qsim_inner(qsim_h a, qsim_h b, double* out) {
     }
     cudaError_t e = run_inner(a->dtype, a->psi, b->psi, a->n, a->red, a->stream, a->dev, out);
     if (e != cudaSuccess) return cuda_fail(e, "inner");
-    return check_device_error(a);
+    return check_passed_error(a);
 }
 
 }  // extern "C"

@@ -37,6 +37,8 @@ bool is_unitary(const double* m, int k, double tol);
 int validate_qubits(int n, const int* targets, int k, const int* controls, int nc, int kmax);
 std::vector<int> nonunit_patterns(const double* diag, int k);
 int check_device_error(qsim_state* h);
+// The same from the copy of the error word that a readout's kernels left beside its result.
+int check_passed_error(qsim_state* h);
 int apply_gate_plain(qsim_state* h, const int* targets, int k, const int* controls, int nc, const double* m);
 
 // Greedy fusion (plan.cu): starting from the earliest unplaced gate, collect every later gate that is not

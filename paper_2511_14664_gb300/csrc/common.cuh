@@ -78,6 +78,14 @@ __device__ __forceinline__ ff ff_add(ff a, ff b) {
     return ff_renorm(s, e);
 }
 
+// The sum without renormalisation (8 operations against 11): lo may grow to a few units of the last place of hi, which
+// costs nothing over the few levels of a tree; ff_renorm at its end.
+__device__ __forceinline__ ff ff_add_lazy(ff a, ff b) {
+    float s, e;
+    two_sum(a.hi, b.hi, s, e);
+    return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+
 __device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
 
 // Exact x*y as hi + lo.
@@ -89,6 +97,30 @@ __device__ __forceinline__ ff two_prod(float x, float y) {
 
 // |z|^2 = re^2 + im^2 as a float-float (exact products, compensated sum).
 __device__ __forceinline__ ff ff_abs2(float re, float im) { return ff_add(two_prod(re, re), two_prod(im, im)); }
+
+// |z|^2 without renormalisation.
+__device__ __forceinline__ ff ff_abs2_lazy(float re, float im) { return ff_add_lazy(two_prod(re, re), two_prod(im, im)); }
+
+// x^2 of a double as a float-float (relative error about 2^-50, not renormalised), by integer and FP32 operations:
+// FP64 arithmetic and conversions run at two a cycle and SM. x = hi + lo + rest exactly, the leading 24, the next 24 and
+// the last 5 bits of its significand. Magnitudes below 2^-126 count as zero, above 2^127 as infinity (their squares are
+// outside the float range in any case); NaN stays NaN.
+__device__ __forceinline__ ff ff_square(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+    const uint32_t e = (h >> 20) & 0x7FFu, sign = h & 0x80000000u;
+    uint32_t hb = ((__funnelshift_l(l, h, 3) & 0x7FFFFFFFu) ^ 0x40000000u) | sign;  // the exponent's lower 8 bits, less 896
+    float one = __uint_as_float((hb & 0x7F800000u) | sign);                        // +- 2^(e - 1023)
+    if (e - 897u > 253u) {  // outside the float range
+        hb = e < 897u ? 0u : (0x7F800000u | (e == 0x7FFu && ((h & 0xFFFFFu) | l) ? 0x400000u : 0u));
+        one = 0.f;
+    }
+    const float hi = __uint_as_float(hb), h2 = __fadd_rn(hi, hi);
+    const float lo = __fmul_rn(__fmul_rn((float)(l & 0x1FFFFFE0u), 0x1p-52f), one);
+    const float rest = __fmul_rn(__fmul_rn((float)(l & 0x1Fu), 0x1p-52f), one);
+    const float p = __fmul_rn(hi, hi), t = __fmul_rn(h2, lo), s = __fadd_rn(p, t);
+    const float e0 = __fmaf_rn(hi, hi, -p), e1 = __fsub_rn(t, __fsub_rn(s, p)), e2 = __fmaf_rn(h2, lo, -t);
+    return {s, __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, __fmaf_rn(lo, lo, __fmul_rn(h2, rest))))};
+}
 
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 

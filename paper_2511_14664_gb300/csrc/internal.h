@@ -210,8 +210,12 @@ struct ReduceScratch {
     double* seg = nullptr;       // 2 * 2^(n-10) doubles: segment sums (doubles, then float-float pairs)
     double* scan = nullptr;      // max(1, 2^(n-12)) + 4096 doubles
     double* result = nullptr;    // 256 doubles (device)
-    double* hresult = nullptr;   // 256 doubles (pinned host)
+    double* hresult = nullptr;   // pinned host: 256 doubles of results (the last one the device error word), then kHostValues
+    const unsigned* derr = nullptr;  // device error word, passed to the host with the results
+    unsigned* herr() const { return hresult ? reinterpret_cast<unsigned*>(hresult + 255) : nullptr; }
+    double* hvalues() const { return hresult + 256; }
 };
+constexpr int kHostValues = 1 << 12;  // marginals or samples that kernels write straight to the host
 constexpr int64_t kPartialDoubles = 1 << 21;
 constexpr int kSegBits = 12;
 
@@ -223,6 +227,9 @@ cudaError_t run_pauli(int dtype, const void* psi, int n, const char* paulis, Red
                       const DevInfo& d, double* out);
 cudaError_t run_zstats(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d,
                        double* zi, double* zz);
+// The same in two halves: the kernels, and, once the stream has been synchronised, the values.
+cudaError_t enqueue_zstats_host(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d);
+void read_zstats(const ReduceScratch& r, int n, double* zi, double* zz);
 // The same values written to device arrays zi_dev[n], zz_dev[n - 1] on `s` (no host synchronisation);
 // normalise: divided by the squared norm (the values of the normalised state).
 cudaError_t run_zstats_device(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s,

@@ -72,8 +72,17 @@ __device__ dd block_sum_acc(typename Acc<R>::A v, dd* sm) {
     return r;
 }
 
-// partials layout: quantity q, block b -> partials[2 * (q * nblocks + b)] (hi, lo).
-__global__ void __launch_bounds__(256) k_final_dd(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
+// The device error word next to a result the host is about to read (ReduceScratch::herr), so that checking it takes no
+// copy of its own.
+__device__ __forceinline__ void pass_error(const unsigned* derr, unsigned* herr) {
+    if (derr && herr) *herr = *derr;
+}
+
+// partials layout: quantity q, block b -> partials[2 * (q * nblocks + b)] (hi, lo). `out` is device memory or pinned
+// host memory (written directly: a copy after the kernel would cost as much as the kernel).
+constexpr int kFinalThreads = 64;  // FP64 is scarce: two warps' trees, not eight
+__global__ void __launch_bounds__(kFinalThreads) k_final_dd(const double* __restrict__ partials, int nblocks, double* __restrict__ out,
+                                                            const unsigned* derr, unsigned* herr) {
     __shared__ dd sm[32];
     const int q = blockIdx.x;
     dd acc = {0.0, 0.0};
@@ -85,56 +94,63 @@ __global__ void __launch_bounds__(256) k_final_dd(const double* __restrict__ par
     if (threadIdx.x == 0) {
         out[2 * q] = acc.hi;
         out[2 * q + 1] = acc.lo;
+        if (q == 0) pass_error(derr, herr);
     }
 }
 
-// Amplitudes 2i and 2i+1 as float-float |a|^2 values (one 16-byte load for complex64).
+// |a|^2 of one amplitude, not renormalised.
+__device__ __forceinline__ ff abs2_lazy(float2 v) { return ff_abs2_lazy(v.x, v.y); }
+__device__ __forceinline__ ff abs2_lazy(double2 v) { return ff_add_lazy(ff_square(v.x), ff_square(v.y)); }
+
+// Amplitudes 2i and 2i+1 as float-float |a|^2 values, not renormalised (one 16-byte load for complex64).
 template <typename R>
 __device__ __forceinline__ void load_p2(const typename Amp<R>::T* psi, uint64_t i, ff& p0, ff& p1) {
     if constexpr (sizeof(R) == 4) {
         const float4 v = reinterpret_cast<const float4*>(psi)[i];
-        p0 = ff_abs2(v.x, v.y);
-        p1 = ff_abs2(v.z, v.w);
+        p0 = ff_abs2_lazy(v.x, v.y);
+        p1 = ff_abs2_lazy(v.z, v.w);
     } else {
-        const double2 a = psi[2 * i], b = psi[2 * i + 1];
-        const dd qa = Acc<double>::abs2(a.x, a.y), qb = Acc<double>::abs2(b.x, b.y);
-        const float ha = (float)qa.hi, hb = (float)qb.hi;
-        p0 = {ha, (float)(qa.hi - (double)ha + qa.lo)};
-        p1 = {hb, (float)(qb.hi - (double)hb + qb.lo)};
+        p0 = abs2_lazy(psi[2 * i]);
+        p1 = abs2_lazy(psi[2 * i + 1]);
     }
 }
 
-// Sum of N float-float values as a pairwise tree (depth log2 N instead of a serial chain of N adds).
+// Sum of N float-float values as a pairwise tree (depth log2 N instead of a serial chain of N adds), renormalised.
 template <int N>
 __device__ __forceinline__ ff ff_tree_sum(ff (&q)[N]) {
 #pragma unroll
     for (int w = N / 2; w >= 1; w >>= 1) {
 #pragma unroll
-        for (int i = 0; i < w; ++i) q[i] = ff_add(q[i], q[i + w]);
+        for (int i = 0; i < w; ++i) q[i] = ff_add_lazy(q[i], q[i + w]);
     }
-    return q[0];
+    return ff_renorm(q[0].hi, q[0].lo);
 }
 
 // ============================================================================================================
 // Norm and overlap
 // ============================================================================================================
-// sum |a|^2 over npairs amplitude pairs. Each block reads one contiguous slice of the state (so the blocks
-// in flight spread over the whole vector rather than sweeping it as one narrow window), eight independent
-// 16-byte loads in flight per thread, summed as a tree.
+// sum |a|^2 over npairs amplitude pairs: chunks of kNormU x kWideThreads pairs, dealt to the blocks in turn (573 us at 28
+// qubits when each block took one contiguous slice, 344 like this), summed as a tree.
+constexpr int kBlocksPerSm = 2, kWideThreads = 512;  // every block sum ends in FP64: few blocks, many threads
+constexpr int kNormU = 4;
 template <typename R>
-__global__ void __launch_bounds__(256) k_norm_pairs(const typename Amp<R>::T* __restrict__ psi, uint64_t npairs,
-                                                    double* partials) {
+__global__ void __launch_bounds__(kWideThreads, kBlocksPerSm) k_norm_pairs(const typename Amp<R>::T* __restrict__ psi, uint64_t npairs,
+                                                                          double* partials) {
     __shared__ dd sm[32];
     ff acc = {0.f, 0.f};
-    const uint64_t per = (npairs + gridDim.x - 1) / gridDim.x;
-    const uint64_t lo = (uint64_t)blockIdx.x * per, hi = min(npairs, lo + per);
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += 4 * blockDim.x) {
-        ff q[8];
+    constexpr uint64_t kChunk = (uint64_t)kNormU * kWideThreads;
+    for (uint64_t c = blockIdx.x * kChunk; c < npairs; c += gridDim.x * kChunk) {
+        ff q[2 * kNormU];
+        if (c + kChunk <= npairs) {  // (a bound on each load would keep the loads from being issued together)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint64_t k = i + u * blockDim.x;
-            if (k < hi) load_p2<R>(psi, k, q[2 * u], q[2 * u + 1]);
-            else q[2 * u] = q[2 * u + 1] = ff{0.f, 0.f};
+            for (int u = 0; u < kNormU; ++u) load_p2<R>(psi, c + u * kWideThreads + threadIdx.x, q[2 * u], q[2 * u + 1]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kNormU; ++u) {
+                const uint64_t k = c + u * kWideThreads + threadIdx.x;
+                if (k < npairs) load_p2<R>(psi, k, q[2 * u], q[2 * u + 1]);
+                else q[2 * u] = q[2 * u + 1] = ff{0.f, 0.f};
+            }
         }
         acc = ff_add(acc, ff_tree_sum(q));
     }
@@ -175,20 +191,102 @@ __global__ void __launch_bounds__(256) k_inner_partial(const typename Amp<R>::T*
 // With f != 0, x and x^f are visited together (x has the top flip bit h clear), so every amplitude is read
 // once: their two terms are s(x) w + s(x^f) conj(w), w = conj(psi_{x^f}) psi_x.
 // ============================================================================================================
+//
+// Since s(x^f) = s(x) times the parity of f & (Y|Z mask), the pair's terms are 2 s(x) Re w in every pair (even parity) or
+// 2i s(x) Im w in every pair (odd): one real sum. Signs: an index is a block's base, an unrolled step and a thread on
+// disjoint bits, so its parity is the XOR of three, of which only the base's changes in the loop.
+__device__ __forceinline__ float sgn(float v, uint32_t s) { return __uint_as_float(__float_as_uint(v) ^ (s << 31)); }
+__device__ __forceinline__ ff sgn(ff v, uint32_t s) { return {sgn(v.hi, s), sgn(v.lo, s)}; }
+__device__ __forceinline__ uint32_t parity(uint64_t v) { return (uint32_t)__popcll(v) & 1u; }
+
+constexpr int kPauliU = 4;   // vectors in flight per thread
+// fmask = 0, complex64, N >= 2 * kPauliU * kWideThreads: signed sum of |a|^2.
+__global__ void __launch_bounds__(kWideThreads) k_pauli_z(const float4* __restrict__ psi, uint64_t npairs, uint64_t smask,
+                                                         double* partials) {
+    __shared__ dd sm[32];
+    const uint64_t pm = smask >> 1;  // signs of the pair index; bit 0 of smask: the sign of the odd amplitude
+    const uint32_t odd = (uint32_t)smask & 1u, pt = parity(threadIdx.x & pm);
+    ff acc = {0.f, 0.f};
+    constexpr uint64_t kChunk = (uint64_t)kPauliU * kWideThreads;
+    for (uint64_t c = blockIdx.x * kChunk; c < npairs; c += gridDim.x * kChunk) {
+        ff q[kPauliU];
+#pragma unroll
+        for (int u = 0; u < kPauliU; ++u) {
+            const float4 v = psi[c + u * kWideThreads + threadIdx.x];
+            q[u] = ff_add_lazy(ff_abs2_lazy(v.x, v.y), sgn(ff_abs2_lazy(v.z, v.w), odd));
+            q[u] = sgn(q[u], parity((uint64_t)(u * kWideThreads) & pm));
+        }
+        acc = ff_add(acc, sgn(ff_tree_sum(q), pt ^ parity(c & pm)));
+    }
+    const dd r = block_sum_acc<float>(acc, sm);
+    if (threadIdx.x == 0) {
+        partials[2 * blockIdx.x] = r.hi;
+        partials[2 * blockIdx.x + 1] = r.lo;
+    }
+}
+
+// fmask != 0 with top flip bit h >= 1, complex64, N >= 4 * kPauliU * kWideThreads: vectors i and i ^ (f >> 1) of two
+// amplitudes meet (bit h - 1 of i clear); IM: the terms are Im w, else Re w.
+template <bool IM>
+__global__ void __launch_bounds__(kWideThreads) k_pauli_pairs(const float4* __restrict__ psi, uint64_t nitems, uint64_t fmask,
+                                                             uint64_t smask, int h, double* partials) {
+    __shared__ dd sm[32];
+    const uint64_t pf = fmask >> 1;
+    const bool flip0 = fmask & 1;
+    // smask over the item index (the pair index with bit h - 1, which is clear, taken out)
+    const uint64_t ps = smask >> 1, low = (1ull << (h - 1)) - 1, pm = (ps & low) | ((ps >> 1) & ~low);
+    const uint32_t odd = (uint32_t)smask & 1u, pt = parity(threadIdx.x & pm);
+    ff acc = {0.f, 0.f};
+    constexpr uint64_t kChunk = (uint64_t)kPauliU * kWideThreads;
+    for (uint64_t c = blockIdx.x * kChunk; c < nitems; c += gridDim.x * kChunk) {
+        float4 A[kPauliU], B[kPauliU];
+#pragma unroll
+        for (int u = 0; u < kPauliU; ++u) {
+            const uint64_t i = insert_zero(c + u * kWideThreads + threadIdx.x, h - 1);
+            A[u] = psi[i];
+            B[u] = psi[i ^ pf];
+        }
+        ff q[kPauliU];
+#pragma unroll
+        for (int u = 0; u < kPauliU; ++u) {
+            const float4 a = A[u];
+            float4 b = B[u];
+            if (flip0) b = make_float4(b.z, b.w, b.x, b.y);
+            ff w0, w1;  // conj(b) a of the even and the odd amplitude
+            if constexpr (IM) {
+                w0 = ff_add_lazy(two_prod(b.x, a.y), ff_neg(two_prod(b.y, a.x)));
+                w1 = ff_add_lazy(two_prod(b.z, a.w), ff_neg(two_prod(b.w, a.z)));
+            } else {
+                w0 = ff_add_lazy(two_prod(b.x, a.x), two_prod(b.y, a.y));
+                w1 = ff_add_lazy(two_prod(b.z, a.z), two_prod(b.w, a.w));
+            }
+            q[u] = sgn(ff_add_lazy(w0, sgn(w1, odd)), parity((uint64_t)(u * kWideThreads) & pm));
+        }
+        acc = ff_add(acc, sgn(ff_tree_sum(q), pt ^ parity(c & pm)));
+    }
+    acc = ff_add(acc, acc);  // the pair's two terms
+    const dd r = block_sum_acc<float>(acc, sm);
+    if (threadIdx.x == 0) {
+        partials[2 * blockIdx.x] = r.hi;
+        partials[2 * blockIdx.x + 1] = r.lo;
+    }
+}
+
+// Any string, width and type. The sum is the real part (odd = 0) or the imaginary part (odd = 1) of the expectation.
 template <typename R>
 __global__ void __launch_bounds__(256) k_pauli_partial(const typename Amp<R>::T* __restrict__ psi, int n, uint64_t fmask,
-                                                       uint64_t smask, int h, double* partials) {
+                                                       uint64_t smask, int h, int odd, double* partials) {
     __shared__ dd sm[32];
     using A = typename Acc<R>::A;
-    A sre = Acc<R>::zero(), sim = Acc<R>::zero();
+    A sum = Acc<R>::zero();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     if (fmask == 0) {
         const uint64_t N = 1ull << n;
         for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += stride) {
             const auto a = psi[x];
             A p = Acc<R>::abs2(a.x, a.y);
-            if (__popcll(x & smask) & 1) p = Acc<R>::neg(p);
-            sre = Acc<R>::add(sre, p);
+            if (parity(x & smask)) p = Acc<R>::neg(p);
+            sum = Acc<R>::add(sum, p);
         }
     } else {
         const uint64_t G = 1ull << (n - 1);
@@ -196,27 +294,17 @@ __global__ void __launch_bounds__(256) k_pauli_partial(const typename Amp<R>::T*
             const uint64_t x = insert_zero(g, h), y = x ^ fmask;
             const auto a = psi[x];
             const auto b = psi[y];
-            // w = conj(b) a
-            A wr = Acc<R>::add(Acc<R>::prod(b.x, a.x), Acc<R>::prod(b.y, a.y));
-            A wi = Acc<R>::add(Acc<R>::prod(b.x, a.y), Acc<R>::neg(Acc<R>::prod(b.y, a.x)));
-            const bool sx = __popcll(x & smask) & 1, sy = __popcll(y & smask) & 1;
-            // s(x) w + s(y) conj(w): real = (s(x)+s(y)) wr, imag = (s(x)-s(y)) wi
-            if (sx == sy) {
-                A t = Acc<R>::add(wr, wr);
-                sre = Acc<R>::add(sre, sx ? Acc<R>::neg(t) : t);
-            } else {
-                A t = Acc<R>::add(wi, wi);
-                sim = Acc<R>::add(sim, sx ? Acc<R>::neg(t) : t);
-            }
+            A w = odd ? Acc<R>::add(Acc<R>::prod(b.x, a.y), Acc<R>::neg(Acc<R>::prod(b.y, a.x)))
+                      : Acc<R>::add(Acc<R>::prod(b.x, a.x), Acc<R>::prod(b.y, a.y));
+            if (parity(x & smask)) w = Acc<R>::neg(w);
+            sum = Acc<R>::add(sum, w);
         }
+        sum = Acc<R>::add(sum, sum);
     }
-    const dd r0 = block_sum_acc<R>(sre, sm);
-    const dd r1 = block_sum_acc<R>(sim, sm);
+    const dd r = block_sum_acc<R>(sum, sm);
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = r0.hi;
-        partials[2 * blockIdx.x + 1] = r0.lo;
-        partials[2 * (gridDim.x + blockIdx.x)] = r1.hi;
-        partials[2 * (gridDim.x + blockIdx.x) + 1] = r1.lo;
+        partials[2 * blockIdx.x] = r.hi;
+        partials[2 * blockIdx.x + 1] = r.lo;
     }
 }
 
@@ -294,7 +382,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_probs_warp(cons
                             v[NB * hh + j] = ff_add(v[NB * hh + j], p[j]);
                             v[16 + NB * hh + j] = ff_add(v[16 + NB * hh + j], q[j]);
                         } else {
-                            v[NB * hh + j] = ff_add(v[NB * hh + j], ff_add(p[j], q[j]));
+                            v[NB * hh + j] = ff_add(v[NB * hh + j], ff_add_lazy(p[j], q[j]));
                         }
                     }
                 }
@@ -350,14 +438,27 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_probs_warp(cons
     }
 }
 
+// The S partials of a bin, in double-double: one thread per bin, or one warp for many partials (a single thread's chain of
+// 512 took 0.12 ms).
 __global__ void __launch_bounds__(256) k_probs_warp_final(const double* __restrict__ partials,
                                                           const __grid_constant__ ProbsWArgs a,
                                                           double* __restrict__ out) {
     const uint64_t NL = 1ull << a.nlow, nbins = NL << a.nhigh;
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nbins; p += (uint64_t)gridDim.x * blockDim.x) {
-        dd acc = {0.0, 0.0};
-        for (uint64_t sc = 0; sc < a.S; ++sc) acc = dd_add(acc, dd{partials[p * a.S + sc], 0.0});
-        out[probs_bin(a, p % NL, p / NL)] = acc.hi + acc.lo;
+    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    if (a.S < 32) {
+        for (uint64_t p = t; p < nbins; p += stride) {
+            dd acc = {0.0, 0.0};
+            for (uint64_t sc = 0; sc < a.S; ++sc) acc = dd_add(acc, dd{partials[p * a.S + sc], 0.0});
+            out[probs_bin(a, p % NL, p / NL)] = acc.hi + acc.lo;
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (uint64_t p = t >> 5; p < nbins; p += stride >> 5) {
+            dd acc = {0.0, 0.0};
+            for (uint64_t sc = lane; sc < a.S; sc += 32) acc = dd_add(acc, dd{partials[p * a.S + sc], 0.0});
+            acc = warp_sum_dd(acc);
+            if (lane == 0) out[probs_bin(a, p % NL, p / NL)] = acc.hi + acc.lo;
+        }
     }
 }
 
@@ -365,7 +466,8 @@ __global__ void __launch_bounds__(256) k_probs_warp_final(const double* __restri
 template <typename R>
 __global__ void __launch_bounds__(256) k_probs_small(const typename Amp<R>::T* __restrict__ psi, int n,
                                                      const __grid_constant__ ProbsArgs a, const int* __restrict__ qpos,
-                                                     double* out) {
+                                                     double* out, const unsigned* derr, unsigned* herr) {
+    if (threadIdx.x == 0) pass_error(derr, herr);
     // qpos: the nq marginal positions (user order) followed by the n-nq other positions, ascending.
     const int nq = a.nq;
     const int NB = 1 << nq, nr = n - nq;
@@ -385,14 +487,8 @@ __global__ void __launch_bounds__(256) k_probs_small(const typename Amp<R>::T* _
 
 template <typename R>
 __device__ __forceinline__ ff load_p(const typename Amp<R>::T* psi, uint64_t i) {
-    const auto v = psi[i];
-    if constexpr (sizeof(R) == 4) {
-        return ff_abs2(v.x, v.y);
-    } else {
-        const dd p = Acc<double>::abs2(v.x, v.y);
-        const float hi = (float)p.hi;
-        return {hi, (float)(p.hi - (double)hi + p.lo)};
-    }
+    const ff p = abs2_lazy(psi[i]);
+    return ff_renorm(p.hi, p.lo);
 }
 
 // ---- <Z> statistics with one warp per 1024-amplitude segment -------------------------------------------------
@@ -405,7 +501,7 @@ __device__ __forceinline__ ff load_p(const typename Amp<R>::T* psi, uint64_t i) 
 constexpr int kZW = 21;
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_zstats_warp(const typename Amp<R>::T* __restrict__ psi, uint64_t nseg,
+__global__ void __launch_bounds__(256, 2) k_zstats_warp(const typename Amp<R>::T* __restrict__ psi, uint64_t nseg,
                                                      double* __restrict__ W, float2* __restrict__ Wf,
                                                      double* __restrict__ partials) {
     const int lane = threadIdx.x & 31;
@@ -425,7 +521,7 @@ __global__ void __launch_bounds__(256) k_zstats_warp(const typename Amp<R>::T* _
             for (int j = 0; j < 8; ++j) load_p2<R>(psi, s * 512 + lane + 32 * (8 * hh + j), P[j], Q[j]);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                pj[8 * hh + j] = ff_add(P[j], Q[j]);
+                pj[8 * hh + j] = ff_add_lazy(P[j], Q[j]);
                 qj[8 * hh + j] = Q[j];
                 V[8 * hh + j] = ff_add(V[8 * hh + j], pj[8 * hh + j]);
             }
@@ -525,7 +621,8 @@ __global__ void __launch_bounds__(256) k_zstats_hi(const float2* __restrict__ Wf
 
 // n < 12: one CTA; quantity q: 0 -> T, 1..n -> S_{q-1}, n+1..2n-1 -> X_{q-n-1}.
 template <typename R>
-__global__ void __launch_bounds__(256) k_zstats_small(const typename Amp<R>::T* __restrict__ psi, int n, double* out) {
+__global__ void __launch_bounds__(256) k_zstats_small(const typename Amp<R>::T* __restrict__ psi, int n, double* out,
+                                                      const unsigned* derr, unsigned* herr) {
     __shared__ double p[4096];
     const int N = 1 << n;
     for (int x = threadIdx.x; x < N; x += blockDim.x) {
@@ -544,16 +641,18 @@ __global__ void __launch_bounds__(256) k_zstats_small(const typename Amp<R>::T* 
         }
         out[2 * q] = acc.hi;
         out[2 * q + 1] = acc.lo;
+        if (q == 0) pass_error(derr, herr);
     }
 }
 
 // ============================================================================================================
-// Sampling: W[s] segment sums (2^SB amplitudes each), chunk sums of 1024 segments, inclusive scan of the
-// chunk sums; then one warp per uniform walks chunk -> segment -> amplitude.
+// Sampling: W[s] segment sums (2^SB amplitudes each), made inclusive prefix sums within chunks of 1024 segments, and an
+// inclusive scan of the chunk sums; then one warp per uniform finds chunk -> segment -> amplitude, 32 candidates at a
+// time (1000 samples of 20 qubits: 130 -> 35 us; walking the 1024 segments and amplitudes in steps of 32 took most).
 // ============================================================================================================
 // W[s] = sum of |a|^2 over segment s (2^SB amplitudes), one warp per segment, 16-byte loads eight at a time.
 template <typename R>
-__global__ void __launch_bounds__(256) k_segsum(const typename Amp<R>::T* __restrict__ psi, int SB, uint64_t nseg,
+__global__ void __launch_bounds__(256, 3) k_segsum(const typename Amp<R>::T* __restrict__ psi, int SB, uint64_t nseg,
                                                 double* __restrict__ W) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -568,52 +667,22 @@ __global__ void __launch_bounds__(256) k_segsum(const typename Amp<R>::T* __rest
     const uint64_t pairs = 1ull << (SB - 1);
     for (uint64_t s = warp0; s < nseg; s += nwarps) {
         ff acc = {0.f, 0.f};
-        for (uint64_t j = lane; j < pairs; j += 8 * 32) {
-            ff q[16];
+        if (pairs % 256 == 0) {  // (a bound on each load would keep the loads from being issued together)
+            for (uint64_t j = lane; j < pairs; j += 8 * 32) {
+                ff q[16];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const uint64_t k = j + 32 * u;
-                if (k < pairs) load_p2<R>(psi, s * pairs + k, q[2 * u], q[2 * u + 1]);
-                else q[2 * u] = q[2 * u + 1] = ff{0.f, 0.f};
+                for (int u = 0; u < 8; ++u) load_p2<R>(psi, s * pairs + j + 32 * u, q[2 * u], q[2 * u + 1]);
+                acc = ff_add(acc, ff_tree_sum(q));
             }
-            acc = ff_add(acc, ff_tree_sum(q));
+        } else {
+            for (uint64_t j = lane; j < pairs; j += 32) {
+                ff q[2];
+                load_p2<R>(psi, s * pairs + j, q[0], q[1]);
+                acc = ff_add(acc, ff_tree_sum(q));
+            }
         }
         const ff tot = warp_sum_ff(acc);
         if (lane == 0) W[s] = (double)tot.hi + (double)tot.lo;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_chunksum(const double* __restrict__ W, uint64_t nseg, double* __restrict__ C) {
-    __shared__ dd sm[32];
-    const uint64_t c = blockIdx.x;
-    dd acc = {0.0, 0.0};
-    for (uint64_t i = c * 1024 + threadIdx.x; i < min(nseg, (c + 1) * 1024); i += blockDim.x)
-        acc = dd_add(acc, dd{W[i], 0.0});
-    acc = block_sum_dd(acc, sm);
-    if (threadIdx.x == 0) C[c] = acc.hi + acc.lo;
-}
-
-// Inclusive scan of C[0..m) in place, one CTA of 1024 threads (double-double). Thread t owns the
-// contiguous run [t * per, (t + 1) * per), per = ceil(m / 1024).
-__global__ void __launch_bounds__(1024) k_scan_small(double* __restrict__ C, int m) {
-    __shared__ dd sh[1024];
-    const int t = threadIdx.x;
-    const int per = (m + 1023) / 1024;
-    const int i0 = t * per, i1 = min(m, i0 + per);
-    dd run = {0.0, 0.0};
-    for (int i = i0; i < i1; ++i) run = dd_add(run, dd{C[i], 0.0});
-    sh[t] = run;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const dd v = t >= off ? sh[t - off] : dd{0.0, 0.0};
-        __syncthreads();
-        sh[t] = dd_add(sh[t], v);
-        __syncthreads();
-    }
-    dd acc = t > 0 ? sh[t - 1] : dd{0.0, 0.0};
-    for (int i = i0; i < i1; ++i) {
-        acc = dd_add(acc, dd{C[i], 0.0});
-        C[i] = acc.hi + acc.lo;
     }
 }
 
@@ -637,60 +706,145 @@ __device__ __forceinline__ ff warp_incl_scan_ff(ff v) {
     return v;
 }
 
+__device__ __forceinline__ dd warp_incl_scan_dd(dd v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const dd u = {__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
+        if (lane >= o) v = dd_add(v, u);
+    }
+    return v;
+}
+
+// Chunk c (1024 segments, four a thread): W becomes its inclusive prefix sums, C[c] its sum (double-double).
+__global__ void __launch_bounds__(256) k_chunkscan(double* __restrict__ W, uint64_t nseg, double* __restrict__ C) {
+    __shared__ dd sm[32];
+    __shared__ double wsum[8];
+    const uint64_t c = blockIdx.x, i0 = c * 1024 + 4 * threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double w[4];
+    dd acc = {0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        w[j] = i0 + j < nseg ? W[i0 + j] : 0.0;
+        acc = dd_add(acc, dd{w[j], 0.0});
+    }
+    w[1] += w[0];
+    w[2] += w[1];
+    w[3] += w[2];
+    double pre = warp_incl_scan_d(w[3]);
+    if (lane == 31) wsum[warp] = pre;
+    acc = block_sum_dd(acc, sm);  // (synchronises)
+    if (threadIdx.x == 0) C[c] = acc.hi + acc.lo;
+    pre -= w[3];
+    for (int k = 0; k < warp; ++k) pre += wsum[k];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (i0 + j < nseg) W[i0 + j] = pre + w[j];
+}
+
+// Inclusive scan of C[0..m) in place, one CTA of up to 1024 threads (double-double). Thread t owns the contiguous run
+// [t * per, (t + 1) * per), per = ceil(m / threads).
+__global__ void __launch_bounds__(1024) k_scan_small(double* __restrict__ C, int m) {
+    __shared__ dd tot[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (m + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int i0 = t * per, i1 = min(m, i0 + per);
+    dd run = {0.0, 0.0};
+    for (int i = i0; i < i1; ++i) run = dd_add(run, dd{C[i], 0.0});
+    const dd incl = warp_incl_scan_dd(run);
+    if (lane == 31) tot[warp] = incl;
+    __syncthreads();
+    dd acc = {__shfl_up_sync(0xffffffffu, incl.hi, 1), __shfl_up_sync(0xffffffffu, incl.lo, 1)};  // exclusive
+    if (lane == 0) acc = {0.0, 0.0};
+    if (warp > 0) {
+        dd base = tot[0];
+        for (int k = 1; k < warp; ++k) base = dd_add(base, tot[k]);
+        acc = dd_add(base, acc);
+    }
+    for (int i = i0; i < i1; ++i) {
+        acc = dd_add(acc, dd{C[i], 0.0});
+        C[i] = acc.hi + acc.lo;
+    }
+}
+
+// First index in [0, count) of the ascending array P with P[i] > r, by 32-way steps of the whole warp; count if none.
+__device__ __forceinline__ int warp_first_above(const double* __restrict__ P, int count, double r) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = count;  // the answer lies in [lo, lo + len]
+    while (len > 0) {
+        const int step = (len + 31) >> 5;                       // lane l looks at the last element of its step
+        const int at = lo + min(len, (lane + 1) * step) - 1;
+        const unsigned hit = __ballot_sync(0xffffffffu, P[at] > r);
+        if (!hit) return lo + len;
+        const int l = __ffs(hit) - 1;
+        const int first = lo + l * step, last = lo + min(len, (l + 1) * step) - 1;  // P[last] > r
+        lo = first;
+        len = last - first;                                     // the answer is `last` if none before it is above
+    }
+    return lo;
+}
+
+// One warp per uniform: chunk, segment (prefix sums within the chunk), then the amplitude: lanes own runs of
+// 2^SB / 32 amplitudes each, then the run's amplitudes 32 at a time.
 template <typename R>
 __global__ void __launch_bounds__(256) k_sample(const typename Amp<R>::T* __restrict__ psi, int SB, uint64_t nseg,
                                                 const double* __restrict__ W, const double* __restrict__ C,
                                                 int nchunk, const double* __restrict__ u, int64_t shots,
-                                                uint64_t* __restrict__ out) {
+                                                uint64_t* __restrict__ out, const unsigned* derr, unsigned* herr) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    if (blockIdx.x == 0 && threadIdx.x == 0) pass_error(derr, herr);
     const double total = C[nchunk - 1];
     for (int64_t i = warp0; i < shots; i += nwarps) {
         const double target = u[i] * total;
-        // chunk: first c with C[c] > target
-        int lo = 0, hi = nchunk;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (C[mid] > target) hi = mid; else lo = mid + 1;
-        }
-        int c = lo < nchunk ? lo : nchunk - 1;
+        const int c = min(warp_first_above(C, nchunk, target), nchunk - 1);
         double r = target - (c > 0 ? C[c - 1] : 0.0);
-        // segment inside the chunk
-        const uint64_t s0 = (uint64_t)c * 1024, s1 = min(nseg, s0 + 1024);
-        double run = 0.0;
-        uint64_t seg = ~0ull, last_nz = s0;
-        for (uint64_t sb = s0; sb < s1 && seg == ~0ull; sb += 32) {
-            const uint64_t s = sb + lane;
-            const double w = s < s1 ? W[s] : 0.0;
-            const double pre = warp_incl_scan_d(w);
-            const unsigned hit = __ballot_sync(0xffffffffu, s < s1 && run + pre > r);
-            const unsigned nz = __ballot_sync(0xffffffffu, w > 0.0);
-            if (nz) last_nz = sb + 31 - __clz(nz);
-            if (hit) {
-                const int l = __ffs(hit) - 1;
-                seg = sb + l;
-                const double before = __shfl_sync(0xffffffffu, pre - w, l);
-                r -= run + before;
+        const uint64_t s0 = (uint64_t)c * 1024;
+        const int ns = (int)(min(nseg, s0 + 1024) - s0);
+        int k = warp_first_above(W + s0, ns, r);
+        if (k == ns) {  // rounding: the last segment that adds to the chunk's sum
+            const double last = W[s0 + ns - 1];
+            for (k = ns - 1; k > 0 && W[s0 + k - 1] == last; --k) {}
+            r = last;
+        }
+        if (k > 0) r -= W[s0 + k - 1];
+        const uint64_t seg = s0 + (uint64_t)k, a0 = seg << SB;
+        // each lane's run
+        const int run = SB > 5 ? 1 << (SB - 5) : 1, runs = SB > 5 ? 32 : 1 << SB;
+        ff sum = {0.f, 0.f};
+        if (lane < runs) {
+            if (run % 8 == 0) {
+                for (int j = 0; j < run; j += 8) {
+                    ff q[8];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) load_p2<R>(psi, ((a0 + (uint64_t)lane * run + j) >> 1) + v, q[2 * v], q[2 * v + 1]);
+                    sum = ff_add(sum, ff_tree_sum(q));
+                }
             } else {
-                run += __shfl_sync(0xffffffffu, pre, 31);
+                for (int j = 0; j < run; ++j) sum = ff_add(sum, load_p<R>(psi, a0 + (uint64_t)lane * run + j));
             }
         }
-        if (seg == ~0ull) { seg = last_nz; r = W[seg]; }
-        // amplitude inside the segment
-        const uint64_t a0 = seg << SB, a1 = a0 + (1ull << SB);
-        ff frun = {0.f, 0.f};
-        uint64_t x = ~0ull, lastx = a0;
-        for (uint64_t xb = a0; xb < a1 && x == ~0ull; xb += 32) {
-            const uint64_t xi = xb + lane;
-            const ff p = xi < a1 ? load_p<R>(psi, xi) : ff{0.f, 0.f};
+        const ff incl = warp_incl_scan_ff(sum);
+        const unsigned hit = __ballot_sync(0xffffffffu, ((double)incl.hi + (double)incl.lo) > r);
+        const unsigned nz = __ballot_sync(0xffffffffu, sum.hi > 0.f);
+        const int l = hit ? __ffs(hit) - 1 : (nz ? 31 - __clz(nz) : 0);
+        ff before = {__shfl_sync(0xffffffffu, incl.hi, (l + 31) & 31), __shfl_sync(0xffffffffu, incl.lo, (l + 31) & 31)};
+        if (l == 0) before = {0.f, 0.f};
+        // the run's amplitudes
+        const uint64_t b0 = a0 + (uint64_t)l * run;
+        uint64_t x = ~0ull, lastx = b0;
+        for (int xb = 0; xb < run && x == ~0ull; xb += 32) {
+            const int xi = xb + lane;
+            const ff p = xi < run ? load_p<R>(psi, b0 + xi) : ff{0.f, 0.f};
             const ff pre = warp_incl_scan_ff(p);
-            const ff tot = ff_add(frun, pre);
-            const unsigned hit = __ballot_sync(0xffffffffu, xi < a1 && ((double)tot.hi + (double)tot.lo) > r);
-            const unsigned nz = __ballot_sync(0xffffffffu, p.hi > 0.f);
-            if (nz) lastx = xb + 31 - __clz(nz);
-            if (hit) x = xb + (__ffs(hit) - 1);
-            else frun = ff_add(frun, ff{__shfl_sync(0xffffffffu, pre.hi, 31), __shfl_sync(0xffffffffu, pre.lo, 31)});
+            const ff tot = ff_add(before, pre);
+            const unsigned h2 = __ballot_sync(0xffffffffu, xi < run && p.hi > 0.f && ((double)tot.hi + (double)tot.lo) > r);
+            const unsigned n2 = __ballot_sync(0xffffffffu, p.hi > 0.f);
+            if (n2) lastx = b0 + xb + 31 - __clz(n2);
+            if (h2) x = b0 + xb + (__ffs(h2) - 1);
+            else before = ff_add(before, ff{__shfl_sync(0xffffffffu, pre.hi, 31), __shfl_sync(0xffffffffu, pre.lo, 31)});
         }
         if (x == ~0ull) x = lastx;
         if (lane == 0) out[i] = x;
@@ -711,27 +865,24 @@ __global__ void k_uniforms(uint64_t seed, int64_t count, double* __restrict__ ou
 // ============================================================================================================
 // Host drivers
 // ============================================================================================================
-static cudaError_t fetch(ReduceScratch& r, int nvals, cudaStream_t s) {
-    cudaError_t e = cudaMemcpyAsync(r.hresult, r.result, sizeof(double) * nvals, cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return e;
-    return cudaStreamSynchronize(s);
+// The kernels wrote the result (and the error word) to the pinned host buffer.
+static cudaError_t fetch(cudaStream_t s) {
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : cudaStreamSynchronize(s);
 }
 
-static int reduce_blocks(const DevInfo& d, uint64_t N, int nq) {
-    int64_t b = std::min<int64_t>((int64_t)d.num_sms * 8, (int64_t)((N + 255) / 256));
-    b = std::min<int64_t>(b, kPartialDoubles / (2 * std::max(1, nq)));
-    return (int)std::max<int64_t>(1, b);
+static int reduce_blocks(const DevInfo& d, uint64_t N, int threads, int per_sm) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)d.num_sms * per_sm, (int64_t)((N + threads - 1) / threads)));
 }
 
 cudaError_t run_norm(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d, double* out) {
     const uint64_t N = 1ull << n;
-    const int nb = reduce_blocks(d, N / 2, 1);
-    if (dtype == QSIM_C64) k_norm_pairs<float><<<nb, 256, 0, s>>>((const float2*)psi, N / 2, r.partials);
-    else k_norm_pairs<double><<<nb, 256, 0, s>>>((const double2*)psi, N / 2, r.partials);
-    k_final_dd<<<1, 256, 0, s>>>(r.partials, nb, r.result);
-    cudaError_t e = cudaGetLastError();
+    const int nb = reduce_blocks(d, N / 2, 4 * kWideThreads, kBlocksPerSm);
+    if (dtype == QSIM_C64) k_norm_pairs<float><<<nb, kWideThreads, 0, s>>>((const float2*)psi, N / 2, r.partials);
+    else k_norm_pairs<double><<<nb, kWideThreads, 0, s>>>((const double2*)psi, N / 2, r.partials);
+    k_final_dd<<<1, kFinalThreads, 0, s>>>(r.partials, nb, r.hresult, r.derr, r.herr());
+    const cudaError_t e = fetch(s);
     if (e != cudaSuccess) return e;
-    if ((e = fetch(r, 2, s)) != cudaSuccess) return e;
     *out = r.hresult[0] + r.hresult[1];
     return cudaSuccess;
 }
@@ -739,13 +890,12 @@ cudaError_t run_norm(int dtype, const void* psi, int n, ReduceScratch& r, cudaSt
 cudaError_t run_inner(int dtype, const void* a, const void* b, int n, ReduceScratch& r, cudaStream_t s,
                       const DevInfo& d, double* out) {
     const uint64_t N = 1ull << n;
-    const int nb = reduce_blocks(d, N, 2);
+    const int nb = reduce_blocks(d, N, 256, 8);
     if (dtype == QSIM_C64) k_inner_partial<float><<<nb, 256, 0, s>>>((const float2*)a, (const float2*)b, N, r.partials);
     else k_inner_partial<double><<<nb, 256, 0, s>>>((const double2*)a, (const double2*)b, N, r.partials);
-    k_final_dd<<<2, 256, 0, s>>>(r.partials, nb, r.result);
-    cudaError_t e = cudaGetLastError();
+    k_final_dd<<<2, kFinalThreads, 0, s>>>(r.partials, nb, r.hresult, r.derr, r.herr());
+    const cudaError_t e = fetch(s);
     if (e != cudaSuccess) return e;
-    if ((e = fetch(r, 4, s)) != cudaSuccess) return e;
     out[0] = r.hresult[0] + r.hresult[1];
     out[1] = r.hresult[2] + r.hresult[3];
     return cudaSuccess;
@@ -762,15 +912,27 @@ cudaError_t run_pauli(int dtype, const void* psi, int n, const char* paulis, Red
         if (c == 'Y') ++ny;
     }
     const int h = f ? 63 - __builtin_clzll(f) : 0;
-    const uint64_t work = f ? (1ull << (n - 1)) : (1ull << n);
-    const int nb = reduce_blocks(d, work, 2);
-    if (dtype == QSIM_C64) k_pauli_partial<float><<<nb, 256, 0, s>>>((const float2*)psi, n, f, sm, h, r.partials);
-    else k_pauli_partial<double><<<nb, 256, 0, s>>>((const double2*)psi, n, f, sm, h, r.partials);
-    k_final_dd<<<2, 256, 0, s>>>(r.partials, nb, r.result);
-    cudaError_t e = cudaGetLastError();
+    const bool odd = __builtin_popcountll(f & sm) & 1;  // the sum is imaginary
+    // whole chunks of vectors for the wide kernels (items: vectors, or pairs of vectors)
+    const uint64_t items = f ? (n >= 2 ? 1ull << (n - 2) : 0) : (n >= 1 ? 1ull << (n - 1) : 0);
+    const bool wide = dtype == QSIM_C64 && items >= (uint64_t)kPauliU * kWideThreads && (f == 0 || h >= 1);
+    int nb;
+    if (wide) {
+        nb = reduce_blocks(d, items, kPauliU * kWideThreads, kBlocksPerSm);
+        const float4* p = (const float4*)psi;
+        if (!f) k_pauli_z<<<nb, kWideThreads, 0, s>>>(p, items, sm, r.partials);
+        else if (odd) k_pauli_pairs<true><<<nb, kWideThreads, 0, s>>>(p, items, f, sm, h, r.partials);
+        else k_pauli_pairs<false><<<nb, kWideThreads, 0, s>>>(p, items, f, sm, h, r.partials);
+    } else {
+        nb = reduce_blocks(d, f ? (1ull << (n - 1)) : (1ull << n), 256, 8);
+        if (dtype == QSIM_C64) k_pauli_partial<float><<<nb, 256, 0, s>>>((const float2*)psi, n, f, sm, h, odd, r.partials);
+        else k_pauli_partial<double><<<nb, 256, 0, s>>>((const double2*)psi, n, f, sm, h, odd, r.partials);
+    }
+    k_final_dd<<<1, kFinalThreads, 0, s>>>(r.partials, nb, r.hresult, r.derr, r.herr());
+    const cudaError_t e = fetch(s);
     if (e != cudaSuccess) return e;
-    if ((e = fetch(r, 4, s)) != cudaSuccess) return e;
-    const double sr = r.hresult[0] + r.hresult[1], si = r.hresult[2] + r.hresult[3];
+    const double v = r.hresult[0] + r.hresult[1];
+    const double sr = odd ? 0.0 : v, si = odd ? v : 0.0;
     // multiply by i^{ny}
     switch (ny & 3) {
         case 0: out[0] = sr; out[1] = si; break;
@@ -781,8 +943,10 @@ cudaError_t run_pauli(int dtype, const void* psi, int n, const char* paulis, Red
     return cudaSuccess;
 }
 
+__global__ void k_pass_error(const unsigned* derr, unsigned* herr) { pass_error(derr, herr); }
+
 // n >= 12: k_probs_warp (see above); the 2^nq results go to r.scan (nq <= 12) or to a temporary device
-// buffer of 8 x 2^nq bytes from the stream-ordered allocator, then one copy to the host.
+// buffer of 8 x 2^nq bytes from the stream-ordered allocator, then one copy to the host (nq <= 12: its pinned buffer).
 static cudaError_t run_probs_warp(int dtype, const void* psi, int n, const int* qubits, int nq, ReduceScratch& r,
                                   cudaStream_t s, const DevInfo& d, double* out) {
     ProbsWArgs a;
@@ -816,6 +980,7 @@ static cudaError_t run_probs_warp(int dtype, const void* psi, int n, const int* 
     double* dout = r.scan;
     cudaError_t e = cudaSuccess;
     const bool tmp = nq > kSegBits;
+    static_assert(kHostValues >= 1 << kSegBits, "");
     if (tmp && (e = cudaMallocAsync(reinterpret_cast<void**>(&dout), bytes, s)) != cudaSuccess) return e;
     const bool m0 = (a.lowmask & 1u) != 0;
     auto launch = [&](auto kern, auto typed_psi) {
@@ -831,13 +996,22 @@ static cudaError_t run_probs_warp(int dtype, const void* psi, int n, const int* 
     if (dtype == QSIM_C64) e = m0 ? launch(k_probs_warp<float, true>, p32) : launch(k_probs_warp<float, false>, p32);
     else e = m0 ? launch(k_probs_warp<double, true>, p64) : launch(k_probs_warp<double, false>, p64);
     if (e == cudaSuccess && S > 1) {
-        k_probs_warp_final<<<(unsigned)std::min<uint64_t>(((1ull << nq) + 255) / 256, 4096), 256, 0, s>>>(r.partials, a, dout);
+        k_probs_warp_final<<<(unsigned)std::min<uint64_t>((((S < 32 ? 1ull : 32ull) << nq) + 255) / 256, 4096), 256, 0, s>>>(r.partials, a, dout);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, bytes, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) {
+        k_pass_error<<<1, 1, 0, s>>>(r.derr, r.herr());
+        e = cudaGetLastError();
+    }
+    // (written in the caller's bin order, too scattered for direct writes to the host)
+    if (e == cudaSuccess) e = cudaMemcpyAsync(tmp ? out : r.hvalues(), dout, bytes, cudaMemcpyDeviceToHost, s);
     const cudaError_t ef = tmp ? cudaFreeAsync(dout, s) : cudaSuccess;
     const cudaError_t es = cudaStreamSynchronize(s);
-    return e != cudaSuccess ? e : (ef != cudaSuccess ? ef : es);
+    if (e != cudaSuccess) return e;
+    if (ef != cudaSuccess) return ef;
+    if (es != cudaSuccess) return es;
+    if (!tmp) std::memcpy(out, r.hvalues(), bytes);
+    return cudaSuccess;
 }
 
 cudaError_t run_probs(int dtype, const void* psi, int n, const int* qubits, int nq, ReduceScratch& r,
@@ -854,12 +1028,11 @@ cudaError_t run_probs(int dtype, const void* psi, int n, const int* qubits, int 
             if (std::find(qubits, qubits + nq, q) == qubits + nq) qpos.push_back(q);
         int* dq = reinterpret_cast<int*>(r.partials + kPartialDoubles - 64);
         if ((e = cudaMemcpyAsync(dq, qpos.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
-        if (dtype == QSIM_C64) k_probs_small<float><<<1, 256, 0, s>>>((const float2*)psi, n, a, dq, r.partials);
-        else k_probs_small<double><<<1, 256, 0, s>>>((const double2*)psi, n, a, dq, r.partials);
+        if (dtype == QSIM_C64) k_probs_small<float><<<1, 256, 0, s>>>((const float2*)psi, n, a, dq, r.hvalues(), r.derr, r.herr());
+        else k_probs_small<double><<<1, 256, 0, s>>>((const double2*)psi, n, a, dq, r.hvalues(), r.derr, r.herr());
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        std::vector<double> h(2 * (size_t)NB);  // up to 2 x 2^11 values: more than the pinned result buffer
-        if ((e = cudaMemcpyAsync(h.data(), r.partials, sizeof(double) * 2 * NB, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+        const double* h = r.hvalues();  // up to 2 x 2^11 values
         for (int m = 0; m < NB; ++m) out[m] = h[2 * m] + h[2 * m + 1];
         return cudaSuccess;
     }
@@ -868,32 +1041,32 @@ cudaError_t run_probs(int dtype, const void* psi, int n, const int* qubits, int 
 
 int zstats_segment_bits(int n) { return n < kSegBits ? 0 : 10; }
 
-// The <Z> kernels: r.result receives, as (hi, lo) pairs, T, S_0..S_{n-1}, X_0..X_{n-2} for n < 12 (one CTA),
+// The <Z> kernels: out receives, as (hi, lo) pairs, T, S_0..S_{n-1}, X_0..X_{n-2} for n < 12 (one CTA),
 // else the kZW warp-segment quantities (T, S_0..S_9, X_0..X_9) followed by S_10..S_{n-1}, X_10..X_{n-2}.
 static cudaError_t enqueue_zstats(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s,
-                                  const DevInfo& d) {
+                                  const DevInfo& d, double* out, unsigned* herr) {
     if (n < kSegBits) {
-        if (dtype == QSIM_C64) k_zstats_small<float><<<1, 256, 0, s>>>((const float2*)psi, n, r.result);
-        else k_zstats_small<double><<<1, 256, 0, s>>>((const double2*)psi, n, r.result);
+        if (dtype == QSIM_C64) k_zstats_small<float><<<1, 256, 0, s>>>((const float2*)psi, n, out, r.derr, herr);
+        else k_zstats_small<double><<<1, 256, 0, s>>>((const double2*)psi, n, out, r.derr, herr);
         return cudaGetLastError();
     }
     // warp segments of 1024 amplitudes (n >= 12 here): bits 0..9 per thread, bits >= 10 from W
     const uint64_t nseg = 1ull << (n - 10);
-    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)d.num_sms * 8, (int64_t)((nseg + 7) / 8)));
+    // as many CTAs as run at once: each ends in FP64 sums of its 21 quantities
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)d.num_sms * kBlocksPerSm, (int64_t)((nseg + 7) / 8)));
     double* W = r.seg;                                   // 2^(n-10) doubles
     float2* Wf = reinterpret_cast<float2*>(r.seg + nseg);  // then the same sums as float-float
     if (dtype == QSIM_C64) k_zstats_warp<float><<<nb, 256, 0, s>>>((const float2*)psi, nseg, W, Wf, r.partials);
     else k_zstats_warp<double><<<nb, 256, 0, s>>>((const double2*)psi, nseg, W, Wf, r.partials);
-    k_final_dd<<<kZW, 256, 0, s>>>(r.partials, nb, r.result);
+    k_final_dd<<<kZW, kFinalThreads, 0, s>>>(r.partials, nb, out, r.derr, herr);
     const int nh = n - 10;
     // after k_final_dd above has consumed the warp partials (same stream), the buffer takes the high bits'
     const unsigned P = (unsigned)std::min<uint64_t>(32, nseg);
     k_zstats_hi<<<dim3(P, 2 * nh - 1), 256, 0, s>>>(Wf, nseg, nh, r.partials);
-    k_final_dd<<<2 * nh - 1, 256, 0, s>>>(r.partials, (int)P, r.result + 2 * kZW);
+    k_final_dd<<<2 * nh - 1, kFinalThreads, 0, s>>>(r.partials, (int)P, out + 2 * kZW, nullptr, nullptr);
     return cudaGetLastError();
 }
 
-static int zstats_result_values(int n) { return n < kSegBits ? 4 * n : 2 * kZW + 2 * (2 * (n - 10) - 1); }
 
 // <Z_i> = T - 2 S_i and <Z_i Z_{i+1}> = T - 2 X_i from the quantities enqueue_zstats leaves (h: (hi, lo) pairs).
 __host__ __device__ inline double zstats_value(const double* h, int q) { return h[2 * q] + h[2 * q + 1]; }
@@ -918,19 +1091,27 @@ __global__ void k_zstats_finish(const double* __restrict__ h, int n, int normali
     }
 }
 
-cudaError_t run_zstats(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d,
-                       double* zi, double* zz) {
-    cudaError_t e = enqueue_zstats(dtype, psi, n, r, s, d);
-    if (e != cudaSuccess) return e;
-    if ((e = fetch(r, zstats_result_values(n), s)) != cudaSuccess) return e;
+cudaError_t enqueue_zstats_host(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d) {
+    return enqueue_zstats(dtype, psi, n, r, s, d, r.hresult, r.herr());
+}
+
+void read_zstats(const ReduceScratch& r, int n, double* zi, double* zz) {
     for (int i = 0; i < n; ++i) zi[i] = zstats_zi(r.hresult, n, i);
     for (int i = 0; i + 1 < n; ++i) zz[i] = zstats_zz(r.hresult, n, i);
+}
+
+cudaError_t run_zstats(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s, const DevInfo& d,
+                       double* zi, double* zz) {
+    cudaError_t e = enqueue_zstats_host(dtype, psi, n, r, s, d);
+    if (e != cudaSuccess) return e;
+    if ((e = fetch(s)) != cudaSuccess) return e;
+    read_zstats(r, n, zi, zz);
     return cudaSuccess;
 }
 
 cudaError_t run_zstats_device(int dtype, const void* psi, int n, ReduceScratch& r, cudaStream_t s,
                               const DevInfo& d, double* zi_dev, double* zz_dev, bool normalise) {
-    cudaError_t e = enqueue_zstats(dtype, psi, n, r, s, d);
+    cudaError_t e = enqueue_zstats(dtype, psi, n, r, s, d, r.result, nullptr);
     if (e != cudaSuccess) return e;
     k_zstats_finish<<<1, 64, 0, s>>>(r.result, n, normalise ? 1 : 0, zi_dev, zz_dev);
     return cudaGetLastError();
@@ -956,11 +1137,11 @@ cudaError_t run_sample(int dtype, const void* psi, int n, const double* u_dev, i
         if (dtype == QSIM_C64) k_segsum<float><<<nb, 256, 0, s>>>((const float2*)psi, SB, nseg, W);
         else k_segsum<double><<<nb, 256, 0, s>>>((const double2*)psi, SB, nseg, W);
     }
-    k_chunksum<<<nchunk, 256, 0, s>>>(W, nseg, C);
-    k_scan_small<<<1, 1024, 0, s>>>(C, nchunk);
+    k_chunkscan<<<nchunk, 256, 0, s>>>(W, nseg, C);
+    k_scan_small<<<1, std::min(1024, (nchunk + 31) & ~31), 0, s>>>(C, nchunk);
     const int sb = (int)std::max<int64_t>(1, std::min<int64_t>((shots * 32 + 255) / 256, (int64_t)d.num_sms * 8));
-    if (dtype == QSIM_C64) k_sample<float><<<sb, 256, 0, s>>>((const float2*)psi, SB, nseg, W, C, nchunk, u_dev, shots, out_dev);
-    else k_sample<double><<<sb, 256, 0, s>>>((const double2*)psi, SB, nseg, W, C, nchunk, u_dev, shots, out_dev);
+    if (dtype == QSIM_C64) k_sample<float><<<sb, 256, 0, s>>>((const float2*)psi, SB, nseg, W, C, nchunk, u_dev, shots, out_dev, r.derr, r.herr());
+    else k_sample<double><<<sb, 256, 0, s>>>((const double2*)psi, SB, nseg, W, C, nchunk, u_dev, shots, out_dev, r.derr, r.herr());
     return cudaGetLastError();
 }
 
