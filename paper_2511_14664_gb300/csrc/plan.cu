@@ -622,7 +622,9 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     // Estimated cost of a grouping in passes: a 7-qubit tensor-core block streams the state like any pass
     // but takes about 1.2 times as long (3.1-3.2 against 2.6 ms at 30 qubits); a phase pass counts 1, or 0.15
     // when it follows a dense block of at most 6 qubits (it becomes that block's epilogue, which only a
-    // tensor-core precision has).
+    // tensor-core precision has). Up to 20 qubits a pass is the time of one tile, 10.1-10.7 us at 7 qubits and 5.7-6.5 at
+    // 6 (11.5 and 9.0 at 21), unless several plans run side by side (launch_per_pass).
+    const double cost7 = n <= 20 && !opts.launch_per_pass ? 1.7 : 1.2;
     auto cost = [&](const std::vector<std::vector<int>>& bl) {
         double cs = 0.0;
         bool prev_dense6 = false;
@@ -632,7 +634,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
             for (int gi : b) { Q |= gmask[gi]; wide = wide && gwide[gi]; diag = diag && gdiag[gi]; }
             const int k = popcnt(Q);
             if (wide && k > 6) cs += (prev_dense6 && opts.precision != QSIM_PREC_SIMT) ? 0.15 : 1.0;
-            else cs += (tc7 && k == 7 && !wide) ? 1.2 : 1.0;
+            else cs += (tc7 && k == 7 && !wide) ? cost7 : 1.0;
             prev_dense6 = !diag && k <= 6;
         }
         return cs;
@@ -666,7 +668,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     } else {
         std::vector<uint64_t> key = {0 /* a plan */, (uint64_t)n, (uint64_t)kmax, narrow, (uint64_t)use_wide,
                                      (uint64_t)opts.plan_effort, (uint64_t)(opts.precision != QSIM_PREC_SIMT),
-                                     (uint64_t)tc7, (uint64_t)G};
+                                     (uint64_t)tc7, (uint64_t)G, (uint64_t)(opts.launch_per_pass != 0)};
         key.reserve(key.size() + 2 * (size_t)G);
         for (int i = 0; i < G; ++i) {
             key.push_back(gmask[i]);
