@@ -5,7 +5,8 @@
 // U = G_g ... G_1 is built column by column: start from the identity and apply every gate to all 2^kb
 // columns at once, exactly like applying it to 2^kb small state vectors. The columns evolve independently,
 // so a block's columns may be spread over several CTAs (grid y): each CTA holds W of them and ping-pongs
-// them between two shared-memory buffers (W = 2^kb up to kb = 6, 2 x 64 KiB; W = 32 for kb = 7, 2 x 64 KiB).
+// them between two shared-memory buffers (W at most 2^kb up to kb = 6, 2 x 64 KiB, and 32 for kb = 7, 2 x 64 KiB; down
+// to 4 when there are few blocks).
 #include <algorithm>
 
 #include "common.cuh"
@@ -66,7 +67,10 @@ cudaError_t launch_compose(const ComposeBlock* dblocks, int nblocks, const Compo
                            const double* dpool, double* dout, int max_kb, cudaStream_t s) {
     if (nblocks == 0) return cudaSuccess;
     if (max_kb < 1 || max_kb > 7) return cudaErrorInvalidValue;
-    const int Dm = 1 << max_kb, cols_max = max_kb <= 6 ? Dm : 32;
+    // a few blocks are spread over the SMs by columns (7 blocks of 138 gates in all, one CTA a block: 50 us)
+    const int Dm = 1 << max_kb;
+    int cols_max = max_kb <= 6 ? Dm : 32;
+    while (cols_max > 4 && (long long)nblocks * (Dm / cols_max) < 128) cols_max /= 2;
     const size_t smem = 2 * sizeof(double2) * (size_t)Dm * (size_t)cols_max;
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_compose), (int)smem);
     if (e != cudaSuccess) return e;

@@ -92,6 +92,7 @@ struct qsim_plan {
     bool pooled = false;    // dbuf came from the library's memory pool
     bool small = false;     // a whole-plan execution is one resident launch (k_small.cu)
     size_t small_off = 0;   // its program in the plan buffer
+    std::vector<std::vector<unsigned char>> staging;  // host sources of uploads that may still be in flight
     std::vector<qsim::TileGroup> tiles;  // a whole per-gate execution: groups of ops, many gates a pass (k_tilegates.cu)
 };
 
@@ -541,8 +542,10 @@ int qsim_plan_cache_clear(void) {
     return QSIM_OK;
 }
 
-int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts_in, void* stream_v,
-                     qsim_plan_h* out, qsim_plan_info* info) {
+// wait: return only when the plan's device data is complete (it may then run on any stream); otherwise the caller runs
+// it on the same stream and synchronises that before it destroys the plan.
+static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts_in, void* stream_v, bool wait,
+                       qsim_plan_h* out, qsim_plan_info* info) {
     set_error("%s", "");
     const auto t0 = std::chrono::steady_clock::now();
     if (!c || !out) { set_error("NULL argument"); return QSIM_EINVAL; }
@@ -990,22 +993,26 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     p->dbuf_bytes = total;
     char* base = static_cast<char*>(p->dbuf);
     int rc = QSIM_OK;
+    // Every source of an upload is kept until the stream has been synchronised: once, at the end.
+    auto upload = [&](size_t off, std::vector<unsigned char>&& src) {
+        p->staging.push_back(std::move(src));
+        return cudaMemcpyAsync(base + off, p->staging.back().data(), p->staging.back().size(), cudaMemcpyHostToDevice, s);
+    };
     // phase tables first: the row phases of an epilogue go into its block's operand below
     for (size_t oi = 0; rc == QSIM_OK && oi < p->ops.size(); ++oi) {
         PlanOp& op = p->ops[oi];
         if (op.kind != OP_PHASE && !(op.kind == OP_TC && op.has_epi)) continue;
-        e = cudaMemcpyAsync(base + (op.kind == OP_PHASE ? op.dev_off : op.epi_off), op.blob.data(), op.blob.size(),
-                            cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // pageable host source
+        e = upload(op.kind == OP_PHASE ? op.dev_off : op.epi_off, std::move(op.blob));
         if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
-        op.blob.clear();
-        op.blob.shrink_to_fit();
+        op.blob = {};
     }
     if (rc == QSIM_OK && !cblocks.empty()) {
-        e = cudaMemcpyAsync(base + off_pool, pool.data(), sizeof(double) * pool.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(base + off_cb, cblocks.data(), sizeof(ComposeBlock) * cblocks.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(base + off_cg, cgates.data(), sizeof(ComposeGate) * cgates.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host vectors are pageable temporaries
+        // gate matrices and descriptors lie one after another: one copy
+        std::vector<unsigned char> up(off_cg + sizeof(ComposeGate) * cgates.size() - off_pool);
+        std::memcpy(up.data(), pool.data(), sizeof(double) * pool.size());
+        std::memcpy(up.data() + (off_cb - off_pool), cblocks.data(), sizeof(ComposeBlock) * cblocks.size());
+        std::memcpy(up.data() + (off_cg - off_pool), cgates.data(), sizeof(ComposeGate) * cgates.size());
+        e = upload(off_pool, std::move(up));
         if (e == cudaSuccess)
             e = launch_compose(reinterpret_cast<ComposeBlock*>(base + off_cb), (int)cblocks.size(),
                                reinterpret_cast<ComposeGate*>(base + off_cg), reinterpret_cast<double*>(base + off_pool),
@@ -1063,7 +1070,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
             const double* U2 = reinterpret_cast<double*>(base + off_out) + 2 * cblocks[op.compose_idx2].out_off;
             e = launch_tc_pair_prepare(U1, U2, base + op.dev_off, s);
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess && !fetch.empty()) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess && one_copy)
             for (const auto& fo : fetch) {
                 PlanOp& op = p->ops[fo.first];
@@ -1085,15 +1092,12 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     for (size_t di = 0; rc == QSIM_OK && di < direct.size(); ++di) {
         PlanOp& op = p->ops[direct[di]];
         const size_t cnt = (size_t)2 << (2 * op.k);
-        std::vector<float> f;
-        if (dtype == QSIM_C64) {
-            f.resize(cnt);
-            for (size_t i = 0; i < cnt; ++i) f[i] = (float)op.mat[i];
-            e = cudaMemcpyAsync(base + op.dev_off, f.data(), cnt * sizeof(float), cudaMemcpyHostToDevice, s);
-        } else {
-            e = cudaMemcpyAsync(base + op.dev_off, op.mat.data(), cnt * sizeof(double), cudaMemcpyHostToDevice, s);
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // pageable host sources
+        std::vector<unsigned char> up(cnt * (dtype == QSIM_C64 ? sizeof(float) : sizeof(double)));
+        if (dtype == QSIM_C64)
+            for (size_t i = 0; i < cnt; ++i) reinterpret_cast<float*>(up.data())[i] = (float)op.mat[i];
+        else
+            std::memcpy(up.data(), op.mat.data(), up.size());
+        e = upload(op.dev_off, std::move(up));
         if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
         op.mat.clear();
         op.mat.shrink_to_fit();
@@ -1113,12 +1117,16 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
         }
         std::vector<unsigned char> prog(small_program_bytes(dtype, (int)p->ops.size()));
         if (small_program_build(dtype, sd, prog.data())) {
-            e = cudaMemcpyAsync(base + off_small, prog.data(), prog.size(), cudaMemcpyHostToDevice, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // pageable host source
+            e = upload(off_small, std::move(prog));
             if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
             p->small = true;
             p->small_off = off_small;
         }
+    }
+    if (rc == QSIM_OK && wait) {
+        e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
+        p->staging.clear();
     }
     if (rc) { cudaStreamSynchronize(s); plan_buffer_free(p->dbuf, p->pooled); delete p; return rc; }
     }  // !dry
@@ -1193,6 +1201,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
                 std::vector<int> glob;
                 for (int q = 0; q < n; ++q) if ((bring >> q) & 1) glob.push_back(phys[q]);
                 if (cand.size() < glob.size()) {
+                    if (!dry) cudaStreamSynchronize(s);
                     plan_buffer_free(p->dbuf, p->pooled);
                     delete p;
                     set_error("local_qubits = %d leaves too few idle local qubits for a %d-qubit pass", L, (int)op_qubits(op).size());
@@ -1232,6 +1241,7 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
                 for (const auto& pr : *inv) std::swap(chk[pr.first], chk[pr.second]);
             for (int q = 0; q < n; ++q)
                 if (chk[q] != q) {
+                    if (!dry) cudaStreamSynchronize(s);
                     plan_buffer_free(p->dbuf, p->pooled);
                     delete p;
                     set_error("internal error: qubit order restore");
@@ -1274,6 +1284,11 @@ int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts
     if (info) *info = I;
     *out = p;
     return QSIM_OK;
+}
+
+int qsim_plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* opts, void* stream, qsim_plan_h* out,
+                     qsim_plan_info* info) {
+    return plan_create(c, dtype, opts, stream, true, out, info);
 }
 
 int qsim_plan_execute(qsim_h h, qsim_plan_h p) {
@@ -1388,11 +1403,13 @@ int qsim_run(qsim_h h, const qsim_circuit* c, const qsim_run_opts* opts, qsim_pl
     if (opts) o = *opts;
     o.use_graph = 0;
     qsim_plan_h p = nullptr;
-    int rc = qsim_plan_create(c, h->dtype, &o, h->stream, &p, info);
+    int rc = plan_create(c, h->dtype, &o, h->stream, false, &p, info);
     if (rc) return rc;
     rc = qsim_plan_execute(h, p);
-    cudaStreamSynchronize(h->stream);
-    qsim_plan_destroy(p);
+    cudaStreamSynchronize(h->stream);  // the only stream that the plan's work and buffer were on
+    if (p->pooled) cudaFreeAsync(p->dbuf, h->stream);
+    else cudaFree(p->dbuf);
+    delete p;
     return rc;
 }
 

@@ -98,8 +98,8 @@ SIGNATURES = {
     "qsim_get_state": ([_vp, _vp, _i], _i),
     "qsim_synchronize": ([_vp], _i),
     "qsim_inject_device_error": ([_vp, ctypes.c_uint], _i),
-    "qsim_apply_gate": ([_vp, _P(_i), _i, _P(_i), _i, _P(ctypes.c_double)], _i),
-    "qsim_apply_fused": ([_vp, _P(_i), _i, _P(ctypes.c_double), _i], _i),
+    "qsim_apply_gate": ([_vp, _P(_i), _i, _P(_i), _i, _vp], _i),
+    "qsim_apply_fused": ([_vp, _P(_i), _i, _vp, _i], _i),
     "qsim_swap_qubits": ([_vp, _P(_i), _P(_i), _i], _i),
     "qsim_plan_create": ([_P(Circuit), _i, _P(RunOpts), _vp, _P(_vp), _P(PlanInfo)], _i),
     "qsim_plan_execute": ([_vp, _vp], _i),
@@ -163,9 +163,13 @@ def _check(rc: int) -> None:
         raise QsimError(rc, lib().qsim_last_error().decode())
 
 
+_INT_ARRAYS = [ctypes.c_int * max(1, n) for n in range(2 * MAX_TARGETS + 1)]  # made once: a single-gate call is microseconds
+
+
 def _ints(xs: Iterable[int]):
     xs = [int(x) for x in xs]
-    return (ctypes.c_int * max(1, len(xs)))(*xs), len(xs)
+    n = len(xs)
+    return (_INT_ARRAYS[n] if n < len(_INT_ARRAYS) else ctypes.c_int * n)(*xs), n
 
 
 def _mat(U) -> np.ndarray:
@@ -245,13 +249,15 @@ class State:
         t, k = _ints(targets)
         c, nc = _ints(controls)
         m = _mat(U)
-        _check(lib().qsim_apply_gate(self.h, t, k, c, nc, _dptr(m)))
+        rc = lib().qsim_apply_gate(self.h, t, k, c, nc, m.ctypes.data)
+        if rc:
+            _check(rc)
         return self
 
     def apply_fused(self, targets: Sequence[int], U, precision: int = PREC_SIMT):
         t, k = _ints(targets)
         m = _mat(U)
-        _check(lib().qsim_apply_fused(self.h, t, k, _dptr(m), int(precision)))
+        _check(lib().qsim_apply_fused(self.h, t, k, m.ctypes.data, int(precision)))
         return self
 
     def swap_qubits(self, a: Sequence[int], b: Sequence[int]):
@@ -337,7 +343,41 @@ def _pack_gates(gs):
     G = len(gs)
     rec = np.zeros(max(1, G), dtype=_GATE_NP)
     pools = []
-    if G:
+    if 0 < G <= 1024:
+        # few gates: one pass that sorts them by width (the array operations below cost more than this loop)
+        groups = {}
+        for i, g in enumerate(gs):
+            t, c = g.targets, g.controls
+            key = (len(t), len(c))
+            e = groups.get(key)
+            if e is None:
+                if key[0] > MAX_TARGETS or key[1] > MAX_CONTROLS:
+                    raise ValueError("a gate has more than %d targets or controls" % MAX_TARGETS)
+                e = groups[key] = ([], [], [], [], [], {})
+            m = g.matrix
+            at = e[5].get(id(m))
+            if at is None:  # one copy per distinct matrix object
+                at = e[5][id(m)] = len(e[4])
+                e[4].append(m)
+            e[0].append(i)
+            e[1].extend(t)
+            e[2].extend(c)
+            e[3].append(at)
+        for (k, nc), (idx, t, c, at, mats, _) in groups.items():
+            M = np.ascontiguousarray(np.array(mats, dtype=np.complex128))
+            if M.shape[1:] != (1 << k, 1 << k):
+                raise ValueError("a %d-qubit gate needs a %dx%d matrix" % (k, 1 << k, 1 << k))
+            pools.append(M)
+            r = np.zeros(len(idx), dtype=_GATE_NP)
+            r["k"] = k
+            r["nc"] = nc
+            if k:
+                r["targets"][:, :k] = np.array(t, dtype=np.int32).reshape(-1, k)
+            if nc:
+                r["controls"][:, :nc] = np.array(c, dtype=np.int32).reshape(-1, nc)
+            r["matrix"] = M.ctypes.data + np.array(at, dtype=np.uint64) * np.uint64(M[0].nbytes)
+            rec[idx] = r
+    elif G:
         tg = [g.targets for g in gs]
         ct = [g.controls for g in gs]
         mt = [g.matrix for g in gs]
