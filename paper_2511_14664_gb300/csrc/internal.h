@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -70,6 +71,23 @@ bool small_program_build(int dtype, const std::vector<SmallOpDesc>& ops, unsigne
 cudaError_t launch_small_run(int dtype, void* psi, int n, void* dprog, int npass, unsigned* dev_err, cudaStream_t s,
                              const DevInfo& d, const uint64_t* from_basis);
 
+// ---- small states: many gates between two grid barriers (k_small_tiles.cu) ------------------------------------
+struct TileGate;
+struct SmallTiles {
+    int groups = 0;          // 0: none
+    int arith = 0;           // QSIM_C64 or QSIM_C128: the type of its arithmetic; the state keeps its own
+    double us = 0.0;         // estimates: microseconds;
+    double roundings = 0.0;  // the gates' rounding errors, as a sum of squares in units of a rounding in `arith`
+};
+// Dense products of at most two qubits and diagonals in place of a fused plan's gates, where that is less work.
+std::vector<TileGate> fuse_pairs(int arith, const std::vector<TileGate>& gates);
+// The program of a state of n <= kSmallMaxQubits qubits (every gate ok); false if it does not fit its limits.
+bool small_tiles_build(int arith, int n, const std::vector<TileGate>& gates, std::vector<unsigned char>& prog,
+                       SmallTiles* out);
+// Run the uploaded program (16-byte aligned) in one launch; with from_basis the state is first |*from_basis>.
+cudaError_t launch_small_tiles(int dtype, const SmallTiles& t, void* psi, int n, void* dprog, unsigned* dev_err,
+                               cudaStream_t s, const DevInfo& d, const uint64_t* from_basis);
+
 // ---- phase pass: any number of 1- and 2-qubit diagonal gates (k_phase.cu) -----------------------------------
 // The combined phase c + sum_a h_a x_a + sum_{a<b} lam_ab x_a x_b (radians) of a run of diagonal gates.
 struct PhaseForm {
@@ -113,7 +131,13 @@ struct TileGroup {
     int steps = 0, ops = 0;      // steps 0: a single gate, which its own kernel runs
     std::vector<uint64_t> prog;
 };
-constexpr int kTileMinQubits = 17;  // narrower plans run resident (k_small.cu)
+constexpr int kTileMinQubits = 17;  // narrower plans run resident (k_small.cu, k_small_tiles.cu)
+// Gates cut into groups of which each acts on `bits` qubits at most (diagonals and controls on any), in an order that keeps
+// that of gates that share a qubit (diagonals among themselves excepted). The qubits in lowset count in every group;
+// `size` adds up to max_size at most, gates to max_ops. A gate that is not ok is a group of its own.
+struct TileCut { std::vector<int> members; uint64_t set = 0; };
+std::vector<TileCut> tile_cut(const std::vector<TileGate>& g, int bits, uint64_t lowset, const std::function<int(const TileGate&)>& size,
+                              int max_size, int max_ops);
 // Dense gates on 1 or 2 targets with any controls, diagonals on at most 2 qubits in all.
 bool tile_gate_ok(bool diag, int k, int nc);
 // The groups a list of gates is applied in (each gate once; gates that share a qubit keep their order unless both are

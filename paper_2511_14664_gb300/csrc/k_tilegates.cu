@@ -485,25 +485,20 @@ static void emit_group(const std::vector<TileGate>& g, const std::vector<int>& m
 
 bool tile_gate_ok(bool diag, int k, int nc) { return diag ? k + nc <= 2 : k <= 2; }
 
-std::vector<TileGroup> tile_groups(int dtype, int n, const std::vector<TileGate>& gates) {
-    const int B = dtype == QSIM_C64 ? tile::kBits<float> : tile::kBits<double>;
-    const int low = dtype == QSIM_C64 ? tile::kLow<float> : tile::kLow<double>;
-    // gates that no group takes (too wide) stand alone and hold back what shares their qubits
-    std::vector<TileGroup> out;
+std::vector<TileCut> tile_cut(const std::vector<TileGate>& g, int bits, uint64_t lowset, const std::function<int(const TileGate&)>& size,
+                              int max_size, int max_ops) {
+    std::vector<TileCut> out;
     std::vector<int> und;
-    for (int i = 0; i < (int)gates.size(); ++i) und.push_back(i);
-    const uint64_t lowset = (1ull << low) - 1;
-    std::vector<TileGate> g = gates;
+    for (int i = 0; i < (int)g.size(); ++i) und.push_back(i);
     while (!und.empty()) {
-        TileGroup grp;
-        if (!g[und[0]].ok) {
-            grp.members = {und[0]};
+        TileCut cut;
+        if (!g[und[0]].ok) {  // no group takes it: alone
+            cut.members = {und[0]};
             und.erase(und.begin());
-            out.push_back(std::move(grp));
+            out.push_back(std::move(cut));
             continue;
         }
-        std::vector<int> best;
-        uint64_t best_set = 0, seen = 0;
+        uint64_t seen = 0;
         int tried = 0;
         for (size_t u = 0; u < und.size() && tried < 12; ++u) {
             const TileGate& c = g[und[u]];
@@ -512,24 +507,37 @@ std::vector<TileGroup> tile_groups(int dtype, int n, const std::vector<TileGate>
             if (!c.ok || !free_ || (u > 0 && c.diag)) continue;
             ++tried;
             uint64_t set = lowset;
-            std::vector<int> got = tile::collect(g, und, c.diag ? -1 : und[u], set, B, ~0ull);
-            if (got.size() > best.size()) { best.swap(got); best_set = set; }
+            std::vector<int> got = tile::collect(g, und, c.diag ? -1 : und[u], set, bits, ~0ull);
+            if (got.size() > cut.members.size()) { cut.members.swap(got); cut.set = set; }
         }
-        // a program larger than its kernel parameter is cut short
-        int words = 1;
-        for (size_t m = 0; m < best.size(); ++m) {
-            const TileGate& c = g[best[m]];
-            words += tile::kStepWords + tile::kOpWords + (dtype == QSIM_C64 ? 1 : 2) * (!c.diag && c.k == 2 ? 16 : 4);
-            if ((words > tile::kMaxProg || m >= (size_t)tile::kMaxOps) && m > 0) { best.resize(m); break; }
+        // a program larger than the room set aside for it is cut short
+        int used = 0;
+        for (size_t m = 0; m < cut.members.size(); ++m) {
+            used += size(g[cut.members[m]]);
+            if ((used > max_size || m >= (size_t)max_ops) && m > 0) { cut.members.resize(m); break; }
         }
-        grp.members = best;
         std::vector<int> rest;
         for (int i : und)
-            if (!std::binary_search(best.begin(), best.end(), i)) rest.push_back(i);
+            if (!std::binary_search(cut.members.begin(), cut.members.end(), i)) rest.push_back(i);
         und.swap(rest);
+        out.push_back(std::move(cut));
+    }
+    return out;
+}
+
+std::vector<TileGroup> tile_groups(int dtype, int n, const std::vector<TileGate>& g) {
+    const int B = dtype == QSIM_C64 ? tile::kBits<float> : tile::kBits<double>;
+    const int low = dtype == QSIM_C64 ? tile::kLow<float> : tile::kLow<double>;
+    auto words = [&](const TileGate& c) {
+        return tile::kStepWords + tile::kOpWords + (dtype == QSIM_C64 ? 1 : 2) * (!c.diag && c.k == 2 ? 16 : 4);
+    };
+    std::vector<TileGroup> out;
+    for (const TileCut& cut : tile_cut(g, B, (1ull << low) - 1, words, tile::kMaxProg - 1, tile::kMaxOps)) {
+        TileGroup grp;
+        grp.members = cut.members;
         if (grp.members.size() > 1) {
-            if (dtype == QSIM_C64) tile::emit_group<float>(g, grp.members, best_set, n, grp);
-            else tile::emit_group<double>(g, grp.members, best_set, n, grp);
+            if (dtype == QSIM_C64) tile::emit_group<float>(g, grp.members, cut.set, n, grp);
+            else tile::emit_group<double>(g, grp.members, cut.set, n, grp);
         }
         out.push_back(std::move(grp));
     }

@@ -92,6 +92,8 @@ struct qsim_plan {
     bool pooled = false;    // dbuf came from the library's memory pool
     bool small = false;     // a whole-plan execution is one resident launch (k_small.cu)
     size_t small_off = 0;   // its program in the plan buffer
+    qsim::SmallTiles stiles;  // groups > 0: the program is k_small_tiles.cu's
+    bool bare = false;      // the passes have no operands of their own (one-shot runs): only the whole plan can run
     std::vector<std::vector<unsigned char>> staging;  // host sources of uploads that may still be in flight
     std::vector<qsim::TileGroup> tiles;  // a whole per-gate execution: groups of ops, many gates a pass (k_tilegates.cu)
 };
@@ -392,6 +394,29 @@ void group_cache_put(const std::vector<uint64_t>& key, const std::vector<std::ve
     ++c.entries;
 }
 
+// A gate (mat: its matrix, or for a diagonal its 2^k entries) as the tile kernels take it; ok is false where they do not.
+static TileGate tile_gate(bool diag, int k, int nc, const int* targets, const int* controls, const double* mat) {
+    TileGate t;
+    t.diag = diag;
+    t.k = k;
+    t.nc = nc;
+    for (int j = 0; j < k; ++j) t.tmask |= 1ull << targets[j];
+    t.all = t.tmask;
+    for (int j = 0; j < nc; ++j) t.all |= 1ull << controls[j];
+    t.ok = tile_gate_ok(diag, k, nc);
+    if (!t.ok) return t;
+    std::copy(targets, targets + k, t.q);
+    std::copy(controls, controls + nc, t.ctl);
+    t.mat.assign(mat, mat + (diag ? 2 << k : 2 << (2 * k)));
+    if (diag && nc > 0) {  // a controlled phase: 1 unless the control (table bit 1) is set
+        t.q[1] = controls[0];
+        t.k = 2;
+        t.nc = 0;
+        t.mat = {1.0, 0.0, 1.0, 0.0, mat[0], mat[1], mat[2], mat[3]};
+    }
+    return t;
+}
+
 static double op_bytes(const PlanOp& op, int n, size_t amp) {
     if (op.kind == OP_SWAP) return 2.0 * amp * std::ldexp(1.0, n) * (1.0 - std::ldexp(1.0, -op.nswap));
     if (op.kind == OP_PHASE) return 2.0 * amp * std::ldexp(1.0, n);
@@ -455,11 +480,14 @@ static int enqueue_ops(qsim_state* h, const qsim_plan* p, size_t first = 0, size
     cudaError_t e = cudaSuccess;
     const size_t last = std::min(p->ops.size(), count == (size_t)-1 ? p->ops.size() : first + count);
     if (p->small && first == 0 && last == p->ops.size()) {
-        e = launch_small_run(h->dtype, h->psi, h->n, static_cast<char*>(p->dbuf) + p->small_off, (int)last, h->derr,
-                             h->stream, h->dev, first_from_basis);
+        char* prog = static_cast<char*>(p->dbuf) + p->small_off;
+        e = p->stiles.groups > 0
+                ? launch_small_tiles(h->dtype, p->stiles, h->psi, h->n, prog, h->derr, h->stream, h->dev, first_from_basis)
+                : launch_small_run(h->dtype, h->psi, h->n, prog, (int)last, h->derr, h->stream, h->dev, first_from_basis);
         if (e != cudaErrorCooperativeLaunchTooLarge) return e == cudaSuccess ? QSIM_OK : cuda_fail(e, "resident plan launch");
         // fewer SMs available than the device has (e.g. a share of them under MPS): launch per pass
         cudaGetLastError();
+        if (p->bare) return cuda_fail(e, "resident plan launch");
         e = cudaSuccess;
         if (first_from_basis) {
             e = launch_set_basis(h->dtype, h->psi, h->n, *first_from_basis, h->stream, h->dev);
@@ -939,27 +967,10 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     // ---- per-gate plans: groups of gates that share a tile take one pass when the whole plan is executed (the
     // passes stay listed, and can be executed, one by one) ----
     if (!dry && opts.mode == QSIM_RUN_PLAIN && !opts.launch_per_pass && !remap_later && n >= kTileMinQubits) {
-        std::vector<TileGate> tg(p->ops.size());
-        for (size_t i = 0; i < p->ops.size(); ++i) {
-            const PlanOp& op = p->ops[i];
-            TileGate& t = tg[i];
-            t.diag = op.kind == OP_DIAG;
-            t.k = op.k;
-            t.nc = op.nc;
-            for (int j = 0; j < op.k; ++j) t.tmask |= 1ull << op.targets[j];
-            t.all = t.tmask;
-            for (int j = 0; j < op.nc; ++j) t.all |= 1ull << op.controls[j];
-            t.ok = (t.diag || op.kind == OP_DENSE_SMALL) && tile_gate_ok(t.diag, op.k, op.nc);
-            if (!t.ok) continue;
-            std::copy(op.targets, op.targets + op.k, t.q);
-            std::copy(op.controls, op.controls + op.nc, t.ctl);
-            t.mat = op.mat;
-            if (t.diag && op.nc > 0) {  // a controlled phase: 1 unless the control (table bit 1) is set
-                t.q[1] = op.controls[0];
-                t.k = 2;
-                t.nc = 0;
-                t.mat = {1.0, 0.0, 1.0, 0.0, op.mat[0], op.mat[1], op.mat[2], op.mat[3]};
-            }
+        std::vector<TileGate> tg;
+        for (const PlanOp& op : p->ops) {
+            tg.push_back(tile_gate(op.kind == OP_DIAG, op.k, op.nc, op.targets, op.controls, op.mat.data()));
+            tg.back().ok = tg.back().ok && (op.kind == OP_DIAG || op.kind == OP_DENSE_SMALL);
         }
         // At 17 qubits a complex128 state has 64 tiles, fewer than the SMs: two-qubit dense gates are bound by FP64 there
         // and faster spread over all SMs gate by gate (0.39 against 0.45 ms for 48 of them); others gain (170
@@ -971,6 +982,63 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
         for (const TileGroup& g : p->tiles) any = any || g.steps > 0;
         if (!any) p->tiles.clear();
     }
+    // a small state whose passes are all CUDA-core dense blocks, diagonals or phase passes runs them in one
+    // resident launch
+    bool small = !opts.launch_per_pass && n <= kSmallMaxQubits && !(opts.local_qubits > 0 && opts.local_qubits < n) &&
+                 !p->ops.empty();
+    for (const PlanOp& op : p->ops)
+        small = small && !op.tcx && ((op.kind == OP_DENSE_SMALL && op.k <= 4) || (op.kind == OP_DENSE_TILE && op.k == 5) ||
+                          (op.kind == OP_DIAG && op.k <= 6) || op.kind == OP_PHASE);
+    // ---- small states: the whole plan in one launch, many gates between two grid barriers (k_small_tiles.cu), from the
+    // circuit's gates, in fused plans combined on up to two qubits. A plan of a few passes stays with them. ----
+    std::vector<unsigned char> small_prog;
+    if (!dry && small && p->ops.size() >= 4) {
+        std::vector<TileGate> tg;
+        bool ok = true;
+        for (int i = 0; i < G && ok; ++i) {
+            const qsim_gate& g = c->gates[i];
+            std::vector<double> dg;
+            if (gdiag[i] && g.k <= 2)
+                for (int m = 0; m < (1 << g.k); ++m) {
+                    dg.push_back(g.matrix[2 * (m * (1 << g.k) + m)]);
+                    dg.push_back(g.matrix[2 * (m * (1 << g.k) + m) + 1]);
+                }
+            tg.push_back(tile_gate(gdiag[i], g.k, g.nc, g.targets, g.controls, gdiag[i] ? dg.data() : g.matrix));
+            ok = tg.back().ok;
+        }
+        if (ok && opts.mode == QSIM_RUN_PLAIN) {
+            if (!small_tiles_build(dtype, n, tg, small_prog, &p->stiles)) p->stiles = {};
+        } else if (ok) {
+            // A fused plan that is kept takes the faster of the two by estimate (with a tenth for its error). k_small.cu's
+            // passes cost 3.1 us in complex64 (14 qubits), in complex128 2.6 us and the FP64 of a dense block, whose chain
+            // is as long below 14 qubits. So TFIM chains, whose blocks hold many cheap gates, stay there (14 qubits,
+            // complex64: 31 against 41 us) and brickwork comes here (14 qubits, complex64 56 against 72 us, complex128 97
+            // against 164 us). A one-shot run saves composing those blocks, 0.1 ms, and always comes here.
+            // Nor may its errors grow: a row of a dense block on k qubits rounds like 2^k units, its coefficients like one
+            // (TFIM, 12 qubits, one-shot: 215 units and 3.4e-7 of the norm pass by pass, 267 and 6e-7 here). So where the
+            // products round more, or where the passes are few (from |0>, many of a first block's terms are exact zeros:
+            // 9 to 15 qubits, 10 layers, 1.9e-7 pass by pass and 2.0e-7 here; 20 layers, 3.3e-7 and 3.0e-7), a complex64
+            // state is computed in FP64 between its barriers (that TFIM circuit: 5e-8; 258 us against 202 and, pass by
+            // pass, 414).
+            double passes_us = 0.0, passes_roundings = 0.0;
+            for (const PlanOp& op : p->ops) {
+                const bool diag = op.kind == OP_DIAG || op.kind == OP_PHASE;
+                passes_us += dtype == QSIM_C64 ? 3.1 : 2.6 + (diag ? 1.0 : std::ldexp(4.0, op.k + std::max(n, 14)) / 482e3);
+                passes_roundings += diag ? 2.0 : 1.0 + std::ldexp(1.0, op.k);
+            }
+            for (int arith = dtype; arith <= QSIM_C128 && p->stiles.groups == 0; ++arith) {
+                SmallTiles t;
+                std::vector<unsigned char> prog;
+                if (!small_tiles_build(arith, n, fuse_pairs(arith, tg), prog, &t)) continue;
+                if ((wait && t.us >= 0.9 * passes_us) || (arith == QSIM_C64 && (t.roundings > passes_roundings || p->ops.size() < 12)))
+                    continue;
+                p->stiles = t;
+                small_prog = std::move(prog);
+            }
+        }
+    }
+    const bool stiles = p->stiles.groups > 0;
+    p->bare = stiles && !wait;
 
     p->dry = dry;
     if (!dry) {
@@ -979,15 +1047,9 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     const size_t off_pool = align(off_out + sizeof(double) * 2 * (size_t)compose_out);
     const size_t off_cb = align(off_pool + sizeof(double) * pool.size());
     const size_t off_cg = align(off_cb + sizeof(ComposeBlock) * cblocks.size());
-    // a small state whose passes are all CUDA-core dense blocks, diagonals or phase passes runs them in one
-    // resident launch
-    bool small = !opts.launch_per_pass && n <= kSmallMaxQubits && !(opts.local_qubits > 0 && opts.local_qubits < n) &&
-                 !p->ops.empty();
-    for (const PlanOp& op : p->ops)
-        small = small && !op.tcx && ((op.kind == OP_DENSE_SMALL && op.k <= 4) || (op.kind == OP_DENSE_TILE && op.k == 5) ||
-                          (op.kind == OP_DIAG && op.k <= 6) || op.kind == OP_PHASE);
     const size_t off_small = align(off_cg + sizeof(ComposeGate) * cgates.size());
-    const size_t total = off_small + (small ? align(small_program_bytes(dtype, (int)p->ops.size())) : 0) + 1024;
+    if (stiles) small = false;
+    const size_t total = off_small + (stiles ? align(small_prog.size()) : small ? align(small_program_bytes(dtype, (int)p->ops.size())) : 0) + 1024;
     e = plan_buffer_alloc(&p->dbuf, total, s, &p->pooled);
     if (e != cudaSuccess) { delete p; set_error("plan buffer of %zu bytes", total); return QSIM_ENOMEM; }
     p->dbuf_bytes = total;
@@ -1001,12 +1063,12 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     // phase tables first: the row phases of an epilogue go into its block's operand below
     for (size_t oi = 0; rc == QSIM_OK && oi < p->ops.size(); ++oi) {
         PlanOp& op = p->ops[oi];
-        if (op.kind != OP_PHASE && !(op.kind == OP_TC && op.has_epi)) continue;
+        if ((op.kind != OP_PHASE && !(op.kind == OP_TC && op.has_epi)) || p->bare) continue;
         e = upload(op.kind == OP_PHASE ? op.dev_off : op.epi_off, std::move(op.blob));
         if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
         op.blob = {};
     }
-    if (rc == QSIM_OK && !cblocks.empty()) {
+    if (rc == QSIM_OK && !cblocks.empty() && !p->bare) {
         // gate matrices and descriptors lie one after another: one copy
         std::vector<unsigned char> up(off_cg + sizeof(ComposeGate) * cgates.size() - off_pool);
         std::memcpy(up.data(), pool.data(), sizeof(double) * pool.size());
@@ -1089,7 +1151,7 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
         }
         if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
     }
-    for (size_t di = 0; rc == QSIM_OK && di < direct.size(); ++di) {
+    for (size_t di = 0; rc == QSIM_OK && !p->bare && di < direct.size(); ++di) {
         PlanOp& op = p->ops[direct[di]];
         const size_t cnt = (size_t)2 << (2 * op.k);
         std::vector<unsigned char> up(cnt * (dtype == QSIM_C64 ? sizeof(float) : sizeof(double)));
@@ -1101,6 +1163,12 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
         if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
         op.mat.clear();
         op.mat.shrink_to_fit();
+    }
+    if (rc == QSIM_OK && stiles) {
+        e = upload(off_small, std::move(small_prog));
+        if (e != cudaSuccess) rc = cuda_fail(e, "plan preparation");
+        p->small = true;
+        p->small_off = off_small;
     }
     if (rc == QSIM_OK && small) {
         std::vector<SmallOpDesc> sd(p->ops.size());
@@ -1407,9 +1475,17 @@ int qsim_run(qsim_h h, const qsim_circuit* c, const qsim_run_opts* opts, qsim_pl
     if (rc) return rc;
     rc = qsim_plan_execute(h, p);
     cudaStreamSynchronize(h->stream);  // the only stream that the plan's work and buffer were on
+    const bool again = rc && p->bare;  // a resident launch refused (fewer SMs available than the device has): per pass
     if (p->pooled) cudaFreeAsync(p->dbuf, h->stream);
     else cudaFree(p->dbuf);
     delete p;
+    if (again) {
+        o.launch_per_pass = 1;
+        if ((rc = qsim_plan_create(c, h->dtype, &o, h->stream, &p, info))) return rc;
+        rc = qsim_plan_execute(h, p);
+        cudaStreamSynchronize(h->stream);
+        qsim_plan_destroy(p);
+    }
     return rc;
 }
 
