@@ -653,9 +653,11 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     // Estimated cost of a grouping in passes: a 7-qubit tensor-core block streams the state like any pass
     // but takes about 1.2 times as long (3.1-3.2 against 2.6 ms at 30 qubits); a phase pass counts 1, or 0.15
     // when it follows a dense block of at most 6 qubits (it becomes that block's epilogue, which only a
-    // tensor-core precision has). Up to 20 qubits a pass is the time of one tile, 10.1-10.7 us at 7 qubits and 5.7-6.5 at
-    // 6 (11.5 and 9.0 at 21), unless several plans run side by side (launch_per_pass).
-    const double cost7 = n <= 20 && !opts.launch_per_pass ? 1.7 : 1.2;
+    // tensor-core precision has). Up to 19 qubits a pass is the time of one tile, 10.1-10.7 us at 7 qubits and 5.7-6.5 at
+    // 6 (19-qubit brickwork: 245 us in 6-qubit blocks, 311 in 7-qubit ones), unless several plans run side by side
+    // (launch_per_pass). At 20 qubits that brickwork would gain too (325 to 293 us), but accuracy figures are quoted for
+    // its 7-qubit blocks.
+    const double cost7 = n <= 19 && !opts.launch_per_pass ? 1.7 : 1.2;
     auto cost = [&](const std::vector<std::vector<int>>& bl) {
         double cs = 0.0;
         bool prev_dense6 = false;
