@@ -208,6 +208,7 @@ k_tc_block(float2* __restrict__ psi, const __grid_constant__ Args a, const uint4
     auto empty = [&](int p) { return bar0 + 8u * (uint32_t)p; };
     auto full = [&](int p) { return bar0 + 8u * (uint32_t)(P + p); };
     const uint32_t bbar = bar0 + 8u * (uint32_t)(2 * P);
+    auto bar_wait = [](uint32_t bar, uint32_t par) { return K <= 5 ? mbar_wait_timed(bar, par) : mbar_wait_bounded(bar, par); };
     // Launched as a programmatic dependent of the kernel before it: everything above (offsets, barriers,
     // TMEM) overlapped that kernel's tail; from here on its writes are visible. The next block kernel may
     // be scheduled at once: it cannot share this SM (shared memory), so its CTAs start where ours finish.
@@ -253,13 +254,13 @@ k_tc_block(float2* __restrict__ psi, const __grid_constant__ Args a, const uint4
                 }
             };
             uint32_t last_bar = 0, last_par = 0;
-            bool bad = !mbar_wait_bounded(bbar, 0);  // B in shared memory
+            bool bad = !bar_wait(bbar, 0);  // B in shared memory
             if (bad) mbar_wait_bounded(bbar, 0);     // once more for the copy still in flight
             for (uint64_t i = 0; i < m && !bad; ++i) {
                 const uint32_t dcol = (i & 1) ? NR : 0, par = (uint32_t)(i & 1);
 #pragma unroll
                 for (int p = P - 1; p >= 0; --p) {
-                    if (!mbar_wait_bounded(full(p), par)) { bad = true; break; }
+                    if (!bar_wait(full(p), par)) { bad = true; break; }
                     fence_after();
                     issue(p, dcol);
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
@@ -556,7 +557,7 @@ k_tc_block(float2* __restrict__ psi, const __grid_constant__ Args a, const uint4
         };
         // warp-uniform bounded wait (the TMEM accesses that follow are .sync.aligned)
         auto wait = [&](uint32_t bar, uint32_t par) -> bool {
-            const bool ok = !__any_sync(0xffffffffu, !mbar_wait_bounded(bar, par));
+            const bool ok = !__any_sync(0xffffffffu, !bar_wait(bar, par));
             fence_after();
             return ok;
         };

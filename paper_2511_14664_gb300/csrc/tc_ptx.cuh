@@ -31,13 +31,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t phase) {
 }
 
 // Wait for the mbarrier phase with a 2-second limit; false on expiry.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t phase) {
-    if (mbar_try_wait(addr, phase)) return true;
+__device__ __forceinline__ bool mbar_wait_timed(uint32_t addr, uint32_t phase) {
     const uint64_t t0 = globaltimer();
     while (!mbar_try_wait(addr, phase)) {
         if (globaltimer() - t0 > 2000000000ull) return false;
     }
     return true;
+}
+
+// The same where the phase has often completed already: a test before the timer is read (30-qubit brickwork in 7-qubit
+// blocks 154 -> 151 ms, 24-qubit 2172 -> 2142 us). In 5-qubit blocks, whose warps mostly wait, it measured 1 to 2 %
+// slower.
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t phase) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(addr), "r"(phase)
+        : "memory");
+    return done != 0 || mbar_wait_timed(addr, phase);
 }
 
 __device__ __forceinline__ uint32_t tf32_rna(float x) {
