@@ -15,11 +15,12 @@
 // With a tensor-core precision, circuits of at least batch_tc_min_n qubits (default 20) leave the persistent
 // launch: one cluster streams a state at a fraction of the GPU's bandwidth (about 0.44 TB/s for a 16-CTA
 // cluster on a 24-qubit state, where the whole GPU does 6.5), so each becomes a fused tensor-core plan
-// (6-qubit blocks, or up to 7 with FP16X3) enqueued after the launch, its first block generating |0>, its <Z>
-// values reduced on the device into the same output arrays. These plans run on eight worker streams forked
-// from the caller's stream and joined back, so that one circuit's pipeline fill and drain overlap another's
-// passes (the narrower circuits' kernels on a half or a quarter of the SMs, side by side). The whole enqueue
-// is one CUDA graph when replayed.
+// (6-qubit blocks, or up to 7 with FP16X3), its first block generating |0>, its <Z> values reduced on the device
+// into the same output arrays. These plans run on eight worker streams forked from the caller's stream before the
+// persistent launch and joined back after it: their kernels take the SMs that launch leaves (64 chains of 10 to 24
+// qubits: 12.9 ms with the plans after the launch, 11.5 ms beside it), and one circuit's pipeline fill and drain
+// overlap another's passes (the narrower circuits' kernels on a half or a quarter of the SMs, side by side). States
+// and results lie apart. The whole enqueue is one CUDA graph when replayed.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -51,8 +52,8 @@ constexpr int kThreads = 256;
 constexpr int kKmax = 4;
 constexpr int kSmallMax = 13;  // largest width kept in shared memory (2^13 x 8 B = 64 KiB)
 constexpr size_t kWideStreams = 8;  // worker streams for the circuits run as tensor-core plans
-constexpr int kHalfGridBelow = 24;     // wide circuits narrower than this run their plans on half the SMs,
-constexpr int kQuarterGridBelow = 22;  // and narrower than this on a quarter of them
+constexpr int kHalfGridBelow = 25;     // wide circuits narrower than this run their plans on half the SMs,
+constexpr int kQuarterGridBelow = 23;  // and narrower than this on a quarter of them
 
 struct Pass {
     int k;
@@ -969,10 +970,10 @@ int qsim_batch_plan_create(const qsim_circuit* cs, int count, const qsim_run_opt
 }
 
 // Wide circuit w (its plan) on worker stream k: the plan from |0> (its first block generates the basis
-// state), then its <Z> values. Below 24 qubits (fewer than 7 tiles of a tensor-core pass per SM) the plan's
-// kernels take half the SMs, below 22 a quarter: each CTA then has more tiles to pipeline, and other worker
-// streams' kernels run on the rest (256-chain batch on 8 worker streams: 45.5 ms, against 49.2 ms with every
-// kernel on all SMs and 4 streams; half the SMs below 24 alone 46.8 ms).
+// state), then its <Z> values. Below 25 qubits (at most 14 tiles of a tensor-core pass per SM) the plan's
+// kernels take half the SMs, below 23 a quarter: each CTA then has more tiles to pipeline, and other worker
+// streams' kernels run on the rest (256 chains of 10 to 24 qubits on 8 worker streams: 42.7 ms, against 43.7 ms
+// with half below 24 and a quarter below 22, and 49.2 ms with every kernel on all SMs and 4 streams).
 static int enqueue_wide(qsim_batch_h b, qsim_plan_h plan, size_t w, int k, void* dev_ws) {
     qsim_state st;
     st.n = b->wide_n[w];
@@ -993,14 +994,16 @@ static int enqueue_wide(qsim_batch_h b, qsim_plan_h plan, size_t w, int k, void*
 
 static int batch_enqueue(qsim_batch_h b, void* dev_ws, cudaStream_t s) {
     b->args.ws = static_cast<float2*>(dev_ws);
+    const bool wide = !b->wide_plans.empty();
+    cudaError_t e = wide ? cudaEventRecord(b->fork_ev, s) : cudaSuccess;
+    if (e != cudaSuccess) return cuda_fail(e, "batch fork");
     if (b->nlarge + b->nsmall > 0) {
         const int rc = batch_launch(b, s);
         if (rc) return rc;
     }
-    if (b->wide_plans.empty()) return QSIM_OK;
+    if (!wide) return QSIM_OK;
     // wide circuits on the worker streams (fork from s, join back into s): each plan from |0> (its first
     // block generates the basis state), then its <Z> values
-    cudaError_t e = cudaEventRecord(b->fork_ev, s);
     for (size_t k = 0; e == cudaSuccess && k < b->wstreams.size(); ++k) e = cudaStreamWaitEvent(b->wstreams[k], b->fork_ev, 0);
     if (e != cudaSuccess) return cuda_fail(e, "batch fork");
     int rc = QSIM_OK;
