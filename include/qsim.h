@@ -113,8 +113,7 @@ typedef struct {
        executed (QSIM_EINVAL). */
     int32_t dry_run;
     /* Batches only (qsim_batch_plan_create): with a tensor-core precision, circuits of at least this many
-       qubits run as fused tensor-core plans (6-qubit blocks, or up to 7 with QSIM_PREC_FP16X3; every pass on
-       the whole GPU) inside the same
+       qubits run as fused tensor-core plans (6-qubit blocks, or up to 7 with QSIM_PREC_FP16X3) inside the same
        enqueue, instead of on one cluster of the persistent launch (0 = 20; at least 13). Ignored for
        QSIM_PREC_SIMT. */
     int32_t batch_tc_min_n;
@@ -448,11 +447,13 @@ int qsim_fp64_peak(double seconds, double* tflops, double* ms);
  * state in the caller's workspace, passes separated by cluster barriers), then one CTA per smaller circuit
  * with the whole state in shared memory. With opts->precision a tensor-core precision, circuits of at
  * least opts->batch_tc_min_n qubits (default 20) are planned as fused tensor-core plans instead (k = 6
- * blocks, or up to 7 with QSIM_PREC_FP16X3; their state in the workspace) and enqueued after the persistent
+ * blocks, or up to 7 with QSIM_PREC_FP16X3; their state in the workspace) that run beside the persistent
  * launch, with their <Z> values reduced on the device: one cluster streams a wide state at a fraction of the
- * GPU's bandwidth, a plan's passes use all of it (below 24 qubits a half, below 22 a quarter of the SMs, so
- * that several run side by side). Those plans run on eight streams the batch owns, forked from the caller's stream
- * and joined back into it, so all work of an execution is ordered before later work on that stream. For circuit i, <Z_q> lands at zi[zi_off(i) + q] (q < n_i) and
+ * GPU's bandwidth, a plan's passes use all of it (below 25 qubits a half, below 23 a quarter of the SMs, so
+ * that several run side by side). With opts->max_fused = 0 the other circuits of at least 19 qubits are planned
+ * too (where that is estimated faster), as blocks of 5 qubits in the states' own precision (QSIM_PREC_SIMT). Those plans run on eight streams the
+ * batch owns, forked from the caller's stream and joined back into it, so all work of an execution is ordered
+ * before later work on that stream. For circuit i, <Z_q> lands at zi[zi_off(i) + q] (q < n_i) and
  * <Z_q Z_{q+1}> at zz[zz_off(i) + q] (q < n_i - 1), the offsets being the running sums of n_i and n_i - 1
  * in input order; sums are compensated (float-float per thread, double-double across threads), and the
  * values are those of the normalised state (divided by the computed squared norm, which FP32 arithmetic

@@ -16,7 +16,8 @@
 // launch: one cluster streams a state at a fraction of the GPU's bandwidth (about 0.44 TB/s for a 16-CTA
 // cluster on a 24-qubit state, where the whole GPU does 6.5), so each becomes a fused tensor-core plan
 // (6-qubit blocks, or up to 7 with FP16X3), its first block generating |0>, its <Z> values reduced on the device
-// into the same output arrays. These plans run on eight worker streams forked from the caller's stream before the
+// into the same output arrays. So do, as plans of 5-qubit blocks in their own precision, the other circuits of
+// at least kOwnPlanMinN qubits, unless the caller asks for a fusion width or the tensor-core plans hide them. These plans run on eight worker streams forked from the caller's stream before the
 // persistent launch and joined back after it: their kernels take the SMs that launch leaves (64 chains of 10 to 24
 // qubits: 12.9 ms with the plans after the launch, 11.5 ms beside it), and one circuit's pipeline fill and drain
 // overlap another's passes (the narrower circuits' kernels on a half or a quarter of the SMs, side by side). States
@@ -52,6 +53,11 @@ constexpr int kThreads = 256;
 constexpr int kKmax = 4;
 constexpr int kSmallMax = 13;  // largest width kept in shared memory (2^13 x 8 B = 64 KiB)
 constexpr size_t kWideStreams = 8;  // worker streams for the circuits run as tensor-core plans
+// Circuits of at least this many qubits run as plans of 5-qubit blocks in their own precision (k_tcx.cu) where no
+// tensor-core precision takes them. 16-step chains, one / nine / forty of a width, in clusters of the persistent launch
+// and as plans: 18 qubits 0.47 / 0.76 / 2.24 ms and 0.21 / 0.69 / 2.34; 19 qubits 0.99 / 1.67 / 4.97 and 0.23 / 1.04 /
+// 3.70; one of 24 qubits 33.7 and 2.57. 64 chains of 10 to 24 qubits: 75 and 26 ms.
+constexpr int kOwnPlanMinN = 19;
 constexpr int kHalfGridBelow = 25;     // wide circuits narrower than this run their plans on half the SMs,
 constexpr int kQuarterGridBelow = 23;  // and narrower than this on a quarter of them
 
@@ -586,10 +592,27 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream_v);
     // circuits this wide run as tensor-core plans (6-qubit blocks need n >= 13); 0 = the tuned threshold
     batch::tune_cache_autoload();
-    const int tc_min_n = opts.precision == QSIM_PREC_SIMT ? 1000
+    const int tc_min_n = opts.precision == QSIM_PREC_SIMT ? QSIM_MAX_QUBITS + 1
                          : (opts.batch_tc_min_n > 0 ? std::max(13, opts.batch_tc_min_n) : batch::tuned_tc_min_n(opts.precision));
+    // others this wide run as plans in the state's own precision, unless a fusion width is asked for
+    int own_min_n = opts.max_fused == 0 ? batch::kOwnPlanMinN : QSIM_MAX_QUBITS + 1;
+    // With enough tensor-core circuits beside it the persistent launch is hidden, and plans of its circuits would only
+    // take SMs from theirs (256 chains of 10 to 24 qubits, FP16X3: 42.7 ms with the 19-qubit ones in clusters, 44.6 as
+    // plans; 29 of 11 to 21 qubits: 1.15 and 0.71 ms). Estimates in microseconds: 40 gates a tensor-core pass at 4.6 TB/s;
+    // 12 gates a cluster's pass of 20 us at 19 qubits, nine clusters.
+    double beside = 0.0, longest = 0.0, all = 0.0;
+    for (int ci = 0; ci < count; ++ci) {
+        const double g = (double)cs[ci].num_gates;
+        if (cs[ci].n >= tc_min_n) beside += g / 40.0 * std::ldexp(16.0, cs[ci].n) / 4.6e6;
+        else if (cs[ci].n >= own_min_n) {
+            const double us = g / 12.0 * std::ldexp(20.0, cs[ci].n - 19);
+            longest = std::max(longest, us);
+            all += us;
+        }
+    }
+    if (beside > std::max(longest, all / 9.0)) own_min_n = QSIM_MAX_QUBITS + 1;
     std::vector<char> wide(count, 0);
-    for (int ci = 0; ci < count; ++ci) wide[ci] = cs[ci].n >= tc_min_n;
+    for (int ci = 0; ci < count; ++ci) wide[ci] = cs[ci].n >= std::min(tc_min_n, own_min_n);
 
     // ---- plan every circuit ---------------------------------------------------------------------------
     std::vector<ComposeBlock> cblocks;
@@ -890,9 +913,10 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
         const int prc = !ok ? QSIM_ENOMEM : parallel_for(nw, nth, device, [&](int w, int my_slot) -> int {
             qsim_run_opts po{};
             po.mode = QSIM_RUN_FUSED;
+            const bool own = cs[wides[w]].n < tc_min_n;
             // FP16X3: 7-qubit blocks where the planner finds them cheaper (nearest-neighbour chains)
-            po.max_fused = opts.precision == QSIM_PREC_FP16X3 ? 7 : 6;
-            po.precision = opts.precision;
+            po.max_fused = own ? 5 : (opts.precision == QSIM_PREC_FP16X3 ? 7 : 6);
+            po.precision = own ? QSIM_PREC_SIMT : opts.precision;
             po.tc_min_k = 5;
             po.launch_per_pass = 1;  // plans run concurrently on worker streams inside a captured graph
             const int r = qsim_plan_create(&cs[wides[w]], QSIM_C64, &po, pst[my_slot], &wph[w], &wpi[w]);

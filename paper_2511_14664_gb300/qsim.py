@@ -580,7 +580,8 @@ def fp64_peak(seconds: float = 1.0):
 class Batch:
     """Many independent circuits (each from |0...0>, complex64) in one persistent launch; returns the
     per-circuit <Z_q> and <Z_q Z_{q+1}>. With a tensor-core precision, circuits of at least tc_min_n qubits
-    (0 = 20) run as fused tensor-core plans in the same enqueue."""
+    (0 = 20) run as fused tensor-core plans in the same enqueue; with max_fused = 0 the others of at least 19
+    qubits run as plans in their own precision."""
 
     def __init__(self, circuits, max_fused: int = 0, stream=None, precision: int = 0, tc_min_n: int = 0):
         import torch
