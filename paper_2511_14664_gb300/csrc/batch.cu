@@ -61,10 +61,12 @@ constexpr int kOwnPlanMinN = 19;
 constexpr int kHalfGridBelow = 25;     // wide circuits narrower than this run their plans on half the SMs,
 constexpr int kQuarterGridBelow = 23;  // and narrower than this on a quarter of them
 
-struct Pass {
-    int k;
-    int targets[kKmax];  // ascending; bit j of the matrix index <-> targets[j]
+struct alignas(16) Pass {
     int64_t mat_off;     // complex entries into the matrix pool
+    int k;
+    int pad;
+    int targets[kKmax];  // ascending; bit j of the matrix index <-> targets[j]
+    uint32_t off[1 << kKmax];  // index bits of each matrix index
 };
 struct Circ {
     int n;
@@ -86,83 +88,163 @@ struct Args {
 
 struct Shared {
     float2 state[1 << kSmallMax];
-    float2 U[1 << (2 * kKmax)];
-    uint64_t off[1 << kKmax];  // gather offsets of the current pass
+    alignas(16) float2 U[2][1 << (2 * kKmax)];
+    alignas(16) Pass pass[3];
     ff seg[8][24];
     double segT, segS11;
     dd red[64];
     int claim;
 };
 
-// ---- dense pass: groups g0, g0 + stride, ... of psi (global or shared memory) ---------------------------
+// ---- dense pass of psi (global or shared memory) by `stride` threads, of which this is g0 (the 32 lanes of a warp are
+// neighbours). A thread takes two groups whose amplitudes are adjacent where there are enough groups, else one, else
+// 2^sl lanes share a group's rows (16-CTA cluster, 14 qubits: 1024 groups of 16 for 4096 threads). Every amplitude is
+// the same chain of FMAs whichever way. Bound: the FP32 pipe, with the loads and stores of the state at 60 and 29 bytes
+// a cycle and SM beside it in clusters; latency where a pass has few groups. Measured, 16-step chains, against one or
+// two groups a thread with the groups of a narrow state on the first CTAs, a load of each matrix before its pass and
+// <Z> of a narrow state by one thread a value: one of 10, 14, 16 qubits 245 -> 86, 185 -> 125, 215 -> 157 us; 400 of
+// 10, 13, 14, 16 qubits 508 -> 247, 602 -> 544, 7160 -> 4920, 8498 -> 6358 us; of 18 qubits level (one 467 us, 400
+// 20.7 -> 20.8 ms). 512 threads a CTA were up to 1.8 times slower.
 template <int K>
-__device__ __noinline__ void apply_dense(float2* psi, int n, const int* tg, const float2* U, const uint64_t* off,
-                                        uint64_t g0, uint64_t stride) {
-    constexpr int D = 1 << K;
-    const uint64_t G = 1ull << (n - K);
-    if (tg[0] >= 1 && G >= 2) {
-        // qubit 0 is not a target: groups 2h and 2h+1 are adjacent amplitudes, one 16-byte vector each
-        for (uint64_t h = g0; h < G / 2; h += stride) {
-            const uint64_t base = insert_zeros(2 * h, tg, K);
-            float4 v[D];
+__device__ __forceinline__ uint32_t insert_zeros32(uint32_t v, const int* pos) {  // states of at most 26 qubits
 #pragma unroll
-            for (int m = 0; m < D; ++m) v[m] = *reinterpret_cast<const float4*>(psi + base + off[m]);
-#pragma unroll
-            for (int r = 0; r < D; ++r) {
-                float r0 = 0.f, i0 = 0.f, r1 = 0.f, i1 = 0.f;
-#pragma unroll
-                for (int c = 0; c < D; ++c) {
-                    const float2 u = U[r * D + c];
-                    r0 = __fmaf_rn(u.x, v[c].x, r0); r0 = __fmaf_rn(-u.y, v[c].y, r0);
-                    i0 = __fmaf_rn(u.x, v[c].y, i0); i0 = __fmaf_rn(u.y, v[c].x, i0);
-                    r1 = __fmaf_rn(u.x, v[c].z, r1); r1 = __fmaf_rn(-u.y, v[c].w, r1);
-                    i1 = __fmaf_rn(u.x, v[c].w, i1); i1 = __fmaf_rn(u.y, v[c].z, i1);
-                }
-                *reinterpret_cast<float4*>(psi + base + off[r]) = make_float4(r0, i0, r1, i1);
-            }
-        }
-        return;
+    for (int j = 0; j < K; ++j) {
+        const uint32_t low = v & ((1u << pos[j]) - 1);
+        v = ((v - low) << 1) | low;
     }
-    for (uint64_t g = g0; g < G; g += stride) {
-        const uint64_t base = insert_zeros(g, tg, K);
+    return v;
+}
+
+template <int K>
+__device__ __forceinline__ float2 dense_row(const float2* u, const float2 (&v)[1 << K]) {
+    float re = 0.f, im = 0.f;
+#pragma unroll
+    for (int c = 0; c < (1 << K); ++c) {
+        re = __fmaf_rn(u[c].x, v[c].x, re);
+        re = __fmaf_rn(-u[c].y, v[c].y, re);
+        im = __fmaf_rn(u[c].x, v[c].y, im);
+        im = __fmaf_rn(u[c].y, v[c].x, im);
+    }
+    return make_float2(re, im);
+}
+
+template <int K>
+__device__ __noinline__ void apply_pairs(float2* psi, int n, const int* tg, const float2* U, const uint32_t* off,
+                                        uint32_t g0, uint32_t stride) {
+    constexpr int D = 1 << K;
+    const uint32_t G = 1u << (n - K);
+    for (uint32_t h = g0; h < G / 2; h += stride) {
+        const uint32_t base = insert_zeros32<K>(2 * h, tg);
+        float4 v[D];
+#pragma unroll
+        for (int m = 0; m < D; ++m) v[m] = *reinterpret_cast<const float4*>(psi + (base + off[m]));
+#pragma unroll
+        for (int r = 0; r < D; ++r) {
+            float r0 = 0.f, i0 = 0.f, r1 = 0.f, i1 = 0.f;
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+                const float2 u = U[r * D + c];
+                r0 = __fmaf_rn(u.x, v[c].x, r0); r0 = __fmaf_rn(-u.y, v[c].y, r0);
+                i0 = __fmaf_rn(u.x, v[c].y, i0); i0 = __fmaf_rn(u.y, v[c].x, i0);
+                r1 = __fmaf_rn(u.x, v[c].z, r1); r1 = __fmaf_rn(-u.y, v[c].w, r1);
+                i1 = __fmaf_rn(u.x, v[c].w, i1); i1 = __fmaf_rn(u.y, v[c].z, i1);
+            }
+            *reinterpret_cast<float4*>(psi + (base + off[r])) = make_float4(r0, i0, r1, i1);
+        }
+    }
+}
+
+template <int K>
+__device__ __noinline__ void apply_groups(float2* psi, int n, const int* tg, const float2* U, const uint32_t* off,
+                                         uint32_t g0, uint32_t stride) {
+    constexpr int D = 1 << K;
+    for (uint32_t g = g0; g < (1u << (n - K)); g += stride) {
+        const uint32_t base = insert_zeros32<K>(g, tg);
         float2 v[D];
 #pragma unroll
         for (int m = 0; m < D; ++m) v[m] = psi[base + off[m]];
 #pragma unroll
-        for (int r = 0; r < D; ++r) {
-            float re = 0.f, im = 0.f;
+        for (int r = 0; r < D; ++r) psi[base + off[r]] = dense_row<K>(U + r * D, v);
+    }
+}
+
+// One task a thread: (groups << sl) <= stride.
+template <int K>
+__device__ __noinline__ void apply_split(float2* psi, int n, const int* tg, const float2* U, const uint32_t* off,
+                                        uint32_t g0, int sl) {
+    constexpr int D = 1 << K;
+    const uint32_t g = g0 >> sl;
+    const bool act = g < (1u << (n - K));
+    const uint32_t base = act ? insert_zeros32<K>(g, tg) : 0;
+    float2 v[D];
+    if (act) {
 #pragma unroll
-            for (int c = 0; c < D; ++c) {
-                const float2 u = U[r * D + c];
-                re = __fmaf_rn(u.x, v[c].x, re);
-                re = __fmaf_rn(-u.y, v[c].y, re);
-                im = __fmaf_rn(u.x, v[c].y, im);
-                im = __fmaf_rn(u.y, v[c].x, im);
-            }
-            psi[base + off[r]] = make_float2(re, im);
-        }
+        for (int m = 0; m < D; ++m) v[m] = psi[base + off[m]];
+    }
+    __syncwarp();  // the lanes of a group are in one warp: every load before any store
+    if (act)
+        for (int r = (int)(g0 & ((1u << sl) - 1)); r < D; r += 1 << sl) psi[base + off[r]] = dense_row<K>(U + r * D, v);
+}
+
+template <int K>
+__device__ __forceinline__ void apply_dense(float2* psi, int n, const int* tg, const float2* U, const uint32_t* off,
+                                           uint32_t g0, uint32_t stride) {
+    const uint32_t G = 1u << (n - K);
+    if (tg[0] >= 1 && G / 2 >= stride) {  // qubit 0 is not a target: groups 2h and 2h + 1 are adjacent
+        apply_pairs<K>(psi, n, tg, U, off, g0, stride);
+    } else if (G >= stride) {
+        apply_groups<K>(psi, n, tg, U, off, g0, stride);
+    } else {
+        int sl = 1;
+        while (sl < K && (G << (sl + 1)) <= stride) ++sl;
+        apply_split<K>(psi, n, tg, U, off, g0, sl);
     }
 }
 
-__device__ __noinline__ void apply_pass(float2* psi, int n, const Pass& P, const float2* U, const uint64_t* off,
-                                       uint64_t g0, uint64_t stride) {
+__device__ __noinline__ void apply_pass(float2* psi, int n, const Pass& P, const float2* U, uint32_t g0, uint32_t stride) {
     switch (P.k) {
-        case 1: apply_dense<1>(psi, n, P.targets, U, off, g0, stride); break;
-        case 2: apply_dense<2>(psi, n, P.targets, U, off, g0, stride); break;
-        case 3: apply_dense<3>(psi, n, P.targets, U, off, g0, stride); break;
-        default: apply_dense<4>(psi, n, P.targets, U, off, g0, stride); break;
+        case 1: apply_dense<1>(psi, n, P.targets, U, P.off, g0, stride); break;
+        case 2: apply_dense<2>(psi, n, P.targets, U, P.off, g0, stride); break;
+        case 3: apply_dense<3>(psi, n, P.targets, U, P.off, g0, stride); break;
+        default: apply_dense<4>(psi, n, P.targets, U, P.off, g0, stride); break;
     }
 }
 
-// Load a pass's matrix and gather offsets into shared memory (the caller synchronises afterwards).
-__device__ __forceinline__ void load_pass(const Args& a, const Pass& P, Shared& sh) {
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// A circuit's passes, a barrier of the cluster or of the CTA after each. While pass p runs, the matrix of pass p + 1 and the description of pass
+// p + 2 are copied into shared memory, so that no pass waits for them.
+__device__ __forceinline__ void run_passes(const float2* mats, const Pass* ps, int npass, int n, float2* psi, uint32_t g0,
+                                          uint32_t stride, Shared& sh, bool cluster) {
+    constexpr int kChunks = sizeof(Pass) / 16;
     const int t = threadIdx.x;
-    const int DD = 1 << (2 * P.k);
-    for (int i = t; i < DD; i += kThreads) sh.U[i] = a.mats[P.mat_off + i];
-    if (t < (1 << P.k)) {
-        uint64_t o = 0;
-        for (int j = 0; j < P.k; ++j) o |= (uint64_t)((t >> j) & 1) << P.targets[j];
-        sh.off[t] = o;
+    auto fetch_pass = [&](int p) {
+        if (p < npass && t < kChunks)
+            copy16_async(reinterpret_cast<char*>(&sh.pass[p % 3]) + 16 * t, reinterpret_cast<const char*>(ps + p) + 16 * t);
+    };
+    auto fetch_matrix = [&](int p) {
+        if (p >= npass) return;
+        const Pass& P = sh.pass[p % 3];
+        if (t < (1 << (2 * P.k - 1))) copy16_async(&sh.U[p & 1][2 * t], mats + P.mat_off + 2 * t);
+    };
+    fetch_pass(0);
+    fetch_pass(1);
+    copy_async_wait();
+    __syncthreads();
+    fetch_matrix(0);
+    copy_async_wait();
+    __syncthreads();
+    for (int p = 0; p < npass; ++p) {
+        fetch_matrix(p + 1);
+        fetch_pass(p + 2);
+        apply_pass(psi, n, sh.pass[p % 3], sh.U[p & 1], g0, stride);
+        copy_async_wait();
+        if (cluster) cg::this_cluster().sync();  // the next pass sees every CTA's stores
+        else __syncthreads();
     }
 }
 
@@ -248,19 +330,29 @@ __device__ void zstats_segments(const float2* psi, int n, uint64_t s0, uint64_t 
     __syncthreads();
 }
 
-// Small widths (n < 12): quantity q = 0 -> T, 1..n -> S_{q-1}, n+1..2n-1 -> X_{q-n-1}, one thread each.
+// Small widths (n < 12): quantity q = 0 -> T, 1..n -> S_{q-1}, n+1..2n-1 -> X_{q-n-1}: lane q of each warp over every
+// eighth amplitude, the warps' sums added in order (11 qubits: 2048 dependent additions by one thread a quantity took
+// 0.3 ms, longer than the passes).
 __device__ __noinline__ void zstats_serial(const float2* psi, int n, Shared& sh) {
-    const int q = threadIdx.x;
+    const int q = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kWarps = kThreads / 32;
+    static_assert(2 * 11 <= 24 && kWarps == 8, "the partials fit sh.seg");
     if (q < 2 * n) {
         ff acc = {0.f, 0.f};
         const int N = 1 << n;
-        for (int x = 0; x < N; ++x) {
+        for (int x = warp; x < N; x += kWarps) {
             bool use;
             if (q == 0) use = true;
             else if (q <= n) use = (x >> (q - 1)) & 1;
             else { const int i = q - n - 1; use = ((x >> i) ^ (x >> (i + 1))) & 1; }
             if (use) acc = ff_add(acc, p_of(psi, x));
         }
+        sh.seg[warp][q] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * n) {
+        ff acc = sh.seg[0][q];
+        for (int w = 1; w < kWarps; ++w) acc = ff_add(acc, sh.seg[w][q]);
         sh.red[q] = dd{(double)acc.hi + (double)acc.lo, 0.0};
     }
     __syncthreads();
@@ -305,16 +397,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(const __grid_constant__ A
         const Circ c = a.circs[idx];
         float2* psi = a.ws + c.state_off;
         const uint64_t N = 1ull << c.n;
-        const uint64_t gid = (uint64_t)rank * kThreads + t, gstride = (uint64_t)CL * kThreads;
+        // warp by warp over the CTAs, so that a pass of few groups is spread over all of them
+        const uint32_t gid = ((t >> 5) * CL + rank) * 32 + (t & 31), gstride = CL * kThreads;
         for (uint64_t i = gid; i < N; i += gstride) psi[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
         cl.sync();
-        for (int p = 0; p < c.npass; ++p) {
-            const Pass P = a.passes[c.first_pass + p];
-            load_pass(a, P, sh);
-            __syncthreads();
-            apply_pass(psi, c.n, P, sh.U, sh.off, gid, gstride);
-            cl.sync();  // release / acquire at cluster scope: the next pass sees every CTA's stores
-        }
+        run_passes(a.mats, a.passes + c.first_pass, c.npass, c.n, psi, gid, gstride, sh, true);
         zstats_segments(psi, c.n, rank, CL, sh);
         cl.sync();
         if (rank == 0 && t < 24 + 2 * (c.n - 12)) {
@@ -337,13 +424,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(const __grid_constant__ A
         float2* psi = sh.state;
         const int N = 1 << c.n;
         for (int i = t; i < N; i += kThreads) psi[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
-        for (int p = 0; p < c.npass; ++p) {
-            const Pass P = a.passes[c.first_pass + p];
-            load_pass(a, P, sh);
-            __syncthreads();
-            apply_pass(psi, c.n, P, sh.U, sh.off, t, kThreads);
-            __syncthreads();
-        }
+        run_passes(a.mats, a.passes + c.first_pass, c.npass, c.n, psi, t, kThreads, sh, false);
         if (c.n >= 12) zstats_segments(psi, c.n, 0, 1, sh);
         else zstats_serial(psi, c.n, sh);
         write_z(sh.red, c.n, a.zi + c.zi_off, a.zz + c.zz_off);
@@ -676,6 +757,8 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
             for (int q = 0; q < n; ++q)
                 if ((Q >> q) & 1) { local[q] = kb; P.targets[kb++] = q; }
             P.k = kb;
+            for (int m = 0; m < 1 << kb; ++m)
+                for (int j = 0; j < kb; ++j) P.off[m] |= (uint32_t)((m >> j) & 1) << P.targets[j];
             P.mat_off = compose_out;
             ComposeBlock cb{kb, (int)cgates.size(), (int)blk.size(), compose_out};
             compose_out += (int64_t)1 << (2 * kb);
