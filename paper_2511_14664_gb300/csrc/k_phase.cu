@@ -10,11 +10,15 @@
 // Phases are 64-bit fixed-point turns (2^64 = one turn): sums wrap around exactly (mod 2 pi) and need no FP64
 // arithmetic, which is scarce on GB300. A range is 1024 consecutive amplitudes: lanes are index bits 0..4
 // (coalesced 256-byte accesses) and each lane's 32 amplitudes differ in bits 5..9. A warp owns a group of
-// 16 consecutive ranges (bits 10..13): it reduces the terms on the group's fixed top bits once, into a
-// constant and a coefficient for each bit below (warp shuffles), and folds in the 4 range bits from small
+// 1 to 16 consecutive ranges (bits 10..13): it reduces the terms on the group's fixed top bits once, into a
+// constant and a coefficient for each bit below, and folds in the range bits from small
 // shared-memory tables per range. Per lane this leaves
 //     phi(lane, m) = s_lane + sum_e nu_e m_e + M(m)   (m = bits 5..9),
 // evaluated as products of unit complex numbers in a depth-5 tree (no per-amplitude sin / cos).
+//
+// Bound: HBM in complex64 from 24 qubits on; in complex128 FP64 (three complex products an amplitude and six sines and
+// cosines a range: about 20 us a range for a warp on an FP64 unit of its own). So a group has 16 ranges only where
+// there are 1024 such groups, and the blocks are narrow enough for one on every SM.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -34,9 +38,14 @@ constexpr int kLaneBits = 5;
 // of 2^nb ranges (block), the rest fixed per group (top). Terms are split by the bit groups they touch.
 constexpr int kBlockBits = 4;
 
+// Ranges of a group (their log2): up to 16 share the top terms, but at least 1024 warps come first. With 16 at every
+// width a 17-qubit pass ran on one SM (622 us in complex128, now 25, and 31 in complex64, now 7), a 22-qubit one on 32
+// of them (627 us, now 160, and 35, now 13); 26 qubits 2505 -> 2471 and 190 -> 177 us (the top terms by one lane a bit).
+static int block_bits(int n) { return std::max(0, std::min(kBlockBits, n - kLowBits - 10)); }
+
 struct Args {
     uint64_t c;
-    int nb;                        // block bits (min(4, n - 10))
+    int nb;                        // block bits (block_bits(n))
     int ntt;                       // terms on two top bits (a single top bit appears as a == b)
     int lt_off[kLowBits + kBlockBits + 1];  // terms (low or block bit j, top bit a): [lt_off[j], lt_off[j+1])
     const uint32_t* tt_ab;         // a | b << 8
@@ -79,12 +88,13 @@ __global__ void __launch_bounds__(256) k_phase(typename Amp<R>::T* __restrict__ 
         }
         s = warp_sum64(s) + a.c;
         __syncwarp();  // the previous group's readers of mu are done
-        for (int j = 0; j < NMU; ++j) {
+        if (lane < NMU) {  // lane j: at most one term a top bit
             uint64_t t = 0;
-            for (int i = a.lt_off[j] + lane; i < a.lt_off[j + 1]; i += 32)
+            const int end = a.lt_off[lane + 1];
+#pragma unroll 4
+            for (int i = a.lt_off[lane]; i < end; ++i)
                 if ((gbase >> a.lt_a[i]) & 1) t += a.lt_l[i];
-            t = warp_sum64(t);
-            if (lane == 0) mu[j] = t;
+            mu[lane] = t;
         }
         __syncwarp();
         const uint64_t lane_c = ll_lane[lane] + s;
@@ -173,7 +183,7 @@ bool phase_form_build(const qsim_gate* const* gates, int count, int n, PhaseForm
 void phase_pack(const PhaseForm& f, int dtype, std::vector<unsigned char>& out, PhasePacked& pk) {
     using namespace phase;
     const int n = (int)f.h.size();
-    const int nb = std::max(0, std::min(kBlockBits, n - kLowBits));
+    const int nb = block_bits(n);
     const int G = kLowBits + nb;  // bits below the top bits
     std::vector<uint32_t> tt_ab, lt_a;
     std::vector<uint64_t> tt_l, lt_l;
@@ -265,7 +275,7 @@ void phase_pack(const PhaseForm& f, int dtype, std::vector<unsigned char>& out, 
 
 cudaError_t launch_phase(int dtype, void* psi, int n, const void* dtab, const PhasePacked& pk, cudaStream_t s,
                          const DevInfo& d) {
-    if (n < phase::kLowBits || pk.nb != std::max(0, std::min(phase::kBlockBits, n - phase::kLowBits)))
+    if (n < phase::kLowBits || pk.nb != phase::block_bits(n))
         return cudaErrorInvalidValue;
     const unsigned char* b = static_cast<const unsigned char*>(dtab);
     phase::Args a;
@@ -280,9 +290,11 @@ cudaError_t launch_phase(int dtype, void* psi, int n, const void* dtab, const Ph
     a.small = reinterpret_cast<const uint64_t*>(b + pk.off_small);
     a.tmid = b + pk.off_tmid;
     const int64_t groups = (int64_t)1 << (n - phase::kLowBits - pk.nb);
-    const unsigned grid = grid_for(groups * 32, 256, d.num_sms, 8);
-    if (dtype == QSIM_C64) phase::k_phase<float><<<grid, 256, 0, s>>>(static_cast<float2*>(psi), n, a);
-    else phase::k_phase<double><<<grid, 256, 0, s>>>(static_cast<double2*>(psi), n, a);
+    int threads = 256;  // a block on every SM first
+    while (threads > 32 && groups * 32 < (int64_t)threads * d.num_sms) threads /= 2;
+    const unsigned grid = grid_for(groups * 32, threads, d.num_sms, 8);
+    if (dtype == QSIM_C64) phase::k_phase<float><<<grid, threads, 0, s>>>(static_cast<float2*>(psi), n, a);
+    else phase::k_phase<double><<<grid, threads, 0, s>>>(static_cast<double2*>(psi), n, a);
     return cudaGetLastError();
 }
 
