@@ -100,6 +100,7 @@ struct PhaseForm {
 struct PhasePacked {
     uint64_t c = 0;
     int nb = 0, ntt = 0;
+    bool lm = false;  // terms join index bits 0..4 and 5..9
     int lt_off[15] = {};
     size_t off_tt_ab = 0, off_tt_l = 0, off_lt_a = 0, off_lt_l = 0, off_small = 0, off_tmid = 0;
 };

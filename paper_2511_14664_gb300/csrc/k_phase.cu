@@ -13,11 +13,13 @@
 // 1 to 16 consecutive ranges (bits 10..13): it reduces the terms on the group's fixed top bits once, into a
 // constant and a coefficient for each bit below, and folds in the range bits from small
 // shared-memory tables per range. Per lane this leaves
-//     phi(lane, m) = s_lane + sum_e nu_e m_e + M(m)   (m = bits 5..9),
-// evaluated as products of unit complex numbers in a depth-5 tree (no per-amplitude sin / cos).
+//     phi(lane, m) = s_lane + sum_e nu_e m_e + M(m)   (m = bits 5..9).
+// Where no term joins a lane bit and a bit 5..9, nu is the same for all lanes: in complex128 lane m then computes the
+// factor of m, and an amplitude takes the product of its lane's factor and that one. Otherwise the factors are products of unit complex
+// numbers in a depth-5 tree. (No per-amplitude sin / cos.)
 //
-// Bound: HBM in complex64 from 24 qubits on; in complex128 FP64 (three complex products an amplitude and six sines and
-// cosines a range: about 20 us a range for a warp on an FP64 unit of its own). So a group has 16 ranges only where
+// Bound: HBM in complex64 from 24 qubits on; in complex128 FP64 (85 % busy at 22 qubits): two complex products an
+// amplitude and two sines and cosines a lane and range, or three and six (22 qubits 93 and 160 us). So a group has 16 ranges only where
 // there are 1024 such groups, and the blocks are narrow enough for one on every SM.
 #include <algorithm>
 #include <cmath>
@@ -52,12 +54,13 @@ struct Args {
     const uint64_t* tt_l;
     const uint32_t* lt_a;          // the top bit
     const uint64_t* lt_l;
-    const uint64_t* small;         // ll_lane[32] | lm[32][5] | sb[16] | mb[16][10]  (see phase_pack)
+    const uint64_t* small;         // ll_lane[32] | lm[32][5] | sb[16] | mb[16][10] | mm[32]  (see phase_pack)
     const void* tmid;              // [32] complex (state precision): exp(i * mid-mid terms of bits 5..9)
 };
-constexpr int kSmallWords = 32 + 32 * 5 + 16 + 16 * kLowBits;
+constexpr int kSmallWords = 32 + 32 * 5 + 16 + 16 * kLowBits + 32;
 
-template <typename R>
+// LM: terms join lane bits and bits 5..9.
+template <typename R, bool LM>
 __global__ void __launch_bounds__(256) k_phase(typename Amp<R>::T* __restrict__ psi, int n, const Args a) {
     using T = typename Amp<R>::T;
     constexpr int M = 1 << (kLowBits - kLaneBits);  // 32 amplitudes per lane, in two halves of 16
@@ -65,14 +68,17 @@ __global__ void __launch_bounds__(256) k_phase(typename Amp<R>::T* __restrict__ 
     constexpr int NMU = kLowBits + kBlockBits;
     __shared__ uint64_t sm[kSmallWords];
     __shared__ uint64_t smu[8][NMU];                // per warp: coefficients of the low and block bits
-    __shared__ T stmid[M];
+    __shared__ T stmid[LM ? M : 1];
+    __shared__ T smid[LM ? 1 : 8][M];               // per warp: the factor of each m
     for (int i = threadIdx.x; i < kSmallWords; i += blockDim.x) sm[i] = a.small[i];
-    if (threadIdx.x < M) stmid[threadIdx.x] = static_cast<const T*>(a.tmid)[threadIdx.x];
+    if constexpr (LM)
+        if (threadIdx.x < M) stmid[threadIdx.x] = static_cast<const T*>(a.tmid)[threadIdx.x];
     __syncthreads();
     const uint64_t* ll_lane = sm;
     const uint64_t* lm = sm + 32;
     const uint64_t* sb = lm + 32 * 5;
     const uint64_t* mb = sb + 16;
+    [[maybe_unused]] const uint64_t* mm = mb + 16 * kLowBits;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint64_t* mu = smu[wib];
     const int gbits = kLowBits + a.nb;
@@ -108,30 +114,50 @@ __global__ void __launch_bounds__(256) k_phase(typename Amp<R>::T* __restrict__ 
 #pragma unroll
             for (int j = 0; j < kLaneBits; ++j)
                 if ((lane >> j) & 1) sl += mu[j] + mbv[j];
-            auto coef = [&](int e) { return mu[kLaneBits + e] + mbv[kLaneBits + e] + lm[lane * (kLowBits - kLaneBits) + e]; };
-            // factors of the first half (m < 16) by a depth-4 tree; the second half adds bit 9's factor
-            T F[H];
-            F[0] = unit_phase(R(0), sl);
+            if constexpr (!LM) {
+                uint64_t pm = mm[lane];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const T B = unit_phase(R(0), coef(e));
+                for (int e = 0; e < 5; ++e)
+                    if ((lane >> e) & 1) pm += mu[kLaneBits + e] + mbv[kLaneBits + e];
+                __syncwarp();  // the previous range's readers are done
+                smid[wib][lane] = unit_phase(R(0), pm);
+                __syncwarp();
+                const T S = unit_phase(R(0), sl);
 #pragma unroll
-                for (int m = 0; m < (1 << e); ++m) F[(1 << e) + m] = cmul(F[m], B);
-            }
-            const T B4 = unit_phase(R(0), coef(4));
-            auto apply_half = [&](auto hc) {
-                constexpr int half = decltype(hc)::value;
-                T v[H];
+                for (int half = 0; half < 2; ++half) {
+                    T v[H];
 #pragma unroll
-                for (int m = 0; m < H; ++m) v[m] = psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane];
+                    for (int m = 0; m < H; ++m) v[m] = psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane];
 #pragma unroll
-                for (int m = 0; m < H; ++m) {
-                    const T f = half ? cmul(cmul(F[m], B4), stmid[H + m]) : cmul(F[m], stmid[m]);
-                    psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane] = cmul(v[m], f);
+                    for (int m = 0; m < H; ++m)
+                        psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane] = cmul(v[m], cmul(S, smid[wib][half * H + m]));
                 }
-            };
-            apply_half(std::integral_constant<int, 0>{});
-            apply_half(std::integral_constant<int, 1>{});
+            } else {
+                auto coef = [&](int e) { return mu[kLaneBits + e] + mbv[kLaneBits + e] + lm[lane * (kLowBits - kLaneBits) + e]; };
+                // factors of the first half (m < 16) by a depth-4 tree; the second half adds bit 9's factor
+                T F[H];
+                F[0] = unit_phase(R(0), sl);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const T B = unit_phase(R(0), coef(e));
+#pragma unroll
+                    for (int m = 0; m < (1 << e); ++m) F[(1 << e) + m] = cmul(F[m], B);
+                }
+                const T B4 = unit_phase(R(0), coef(4));
+                auto apply_half = [&](auto hc) {
+                    constexpr int half = decltype(hc)::value;
+                    T v[H];
+#pragma unroll
+                    for (int m = 0; m < H; ++m) v[m] = psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane];
+#pragma unroll
+                    for (int m = 0; m < H; ++m) {
+                        const T f = half ? cmul(cmul(F[m], B4), stmid[H + m]) : cmul(F[m], stmid[m]);
+                        psi[base + ((uint64_t)(half * H + m) << kLaneBits) + lane] = cmul(v[m], f);
+                    }
+                };
+                apply_half(std::integral_constant<int, 0>{});
+                apply_half(std::integral_constant<int, 1>{});
+            }
         }
     }
 }
@@ -200,6 +226,7 @@ void phase_pack(const PhaseForm& f, int dtype, std::vector<unsigned char>& out, 
     uint64_t* lm = ll_lane + 32;
     uint64_t* sb = lm + 32 * 5;
     uint64_t* mb = sb + 16;
+    uint64_t* mm = mb + 16 * kLowBits;
     double midmid[5][5] = {};
     uint64_t lanelane[5][5] = {};
     for (const auto& p : f.pairs) {
@@ -214,12 +241,20 @@ void phase_pack(const PhaseForm& f, int dtype, std::vector<unsigned char>& out, 
                 if ((bv >> (p.b - kLowBits)) & 1) mb[bv * kLowBits + p.a] += L;
         } else if (p.b < kLaneBits) lanelane[p.a][p.b] += L;              // lane x lane
         else if (p.a < kLaneBits) {                                        // lane x mid
+            pk.lm = true;
             for (int l = 0; l < 32; ++l)
                 if ((l >> p.a) & 1) lm[l * 5 + (p.b - kLaneBits)] += L;
         } else {
             midmid[p.a - kLaneBits][p.b - kLaneBits] += p.lam;             // mid x mid
         }
     }
+    for (int m = 0; m < 32; ++m)  // bits 5..9 among themselves
+        for (int j = 0; j < 5; ++j) {
+            if (!((m >> j) & 1)) continue;
+            mm[m] += hg[kLaneBits + j];
+            for (int k = j + 1; k < 5; ++k)
+                if ((m >> k) & 1) mm[m] += phase_turns(midmid[j][k]);
+        }
     for (int bv = 0; bv < (1 << nb); ++bv)
         for (int k = 0; k < nb; ++k)
             if ((bv >> k) & 1) sb[bv] += hg[kLowBits + k];
@@ -293,8 +328,13 @@ cudaError_t launch_phase(int dtype, void* psi, int n, const void* dtab, const Ph
     int threads = 256;  // a block on every SM first
     while (threads > 32 && groups * 32 < (int64_t)threads * d.num_sms) threads /= 2;
     const unsigned grid = grid_for(groups * 32, threads, d.num_sms, 8);
-    if (dtype == QSIM_C64) phase::k_phase<float><<<grid, threads, 0, s>>>(static_cast<float2*>(psi), n, a);
-    else phase::k_phase<double><<<grid, threads, 0, s>>>(static_cast<double2*>(psi), n, a);
+    if (dtype == QSIM_C64) {
+        // the tree in either case: its arithmetic hides behind HBM (28 qubits 656 us, 708 with a factor a lane and m)
+        phase::k_phase<float, true><<<grid, threads, 0, s>>>(static_cast<float2*>(psi), n, a);
+    } else {
+        auto kern = pk.lm ? phase::k_phase<double, true> : phase::k_phase<double, false>;
+        kern<<<grid, threads, 0, s>>>(static_cast<double2*>(psi), n, a);
+    }
     return cudaGetLastError();
 }
 

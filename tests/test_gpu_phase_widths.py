@@ -18,7 +18,9 @@ def qsim(gpu_lib):
 
 @pytest.mark.parametrize("dtype", [0, 1])
 @pytest.mark.parametrize("n", [10, 11, 14, 17, 18, 20, 21, 22, 23, 24])
-def test_widths(qsim, dtype, n):
+@pytest.mark.parametrize("joined", [True, False])
+def test_widths(qsim, dtype, n, joined):
+    """joined: terms between index bits 0..4 and 5..9."""
     rng = np.random.default_rng(n)
     c = W.Circuit(n)
     phase = np.zeros(1 << n)
@@ -26,6 +28,8 @@ def test_widths(qsim, dtype, n):
     for a, b in [(0, n - 1), (3, 7), (5, 9), (4, 8), (1, 2), (n - 2, n - 1), (6, n - 3)] + \
             [tuple(int(q) for q in rng.permutation(n)[:2]) for _ in range(12)]:
         th = float(rng.uniform(0, 6))
+        if not joined and min(a, b) < 5 <= max(a, b) < 10:
+            continue
         c.append(W.Gate((a,), (b,), W.CP(th), "cp"))
         phase += th * ((x >> a) & (x >> b) & 1)
     p = qsim.Plan(c, dtype, mode=1, max_fused=5, launch_per_pass=True)
