@@ -550,11 +550,13 @@ def run_ours(args):
     if not args.no_variants and "plain" in plans:
         pp = plans["plain"]
         timed_steps(qsim, torch, st, pp, 1, shots, per_pass=False)
-        ms, pms = timed_steps(qsim, torch, st, pp, 1, shots, per_pass=True)
+        ms, _ = timed_steps(qsim, torch, st, pp, 1, shots, per_pass=False)   # groups of gates share a pass
+        by_pass_ms, pms = timed_steps(qsim, torch, st, pp, 1, shots, per_pass=True)  # one pass a gate
         dense = [(i, m) for i, (i2, m) in enumerate(zip(pp.pass_list, pms)) if pp.pass_list[i]["kind"] == "dense_small"]
         dense_bytes = sum(pp.pass_list[i]["algorithmic_bytes"] for i, _ in dense)
         dense_ms = sum(m for _, m in dense)
         plain = {"gates_per_s": G / (ms / 1000.0), "ms_per_step": ms, "passes": len(pp.pass_list),
+                 "ms_per_step_gate_by_gate": by_pass_ms,
                  "per_gate_pass_gbs": dense_bytes / (dense_ms / 1000.0) / 1e9 if dense_ms > 0 else None}
 
     # ---- end to end through the public API with host buffers -----------------------------------------------------
@@ -677,9 +679,9 @@ def _event_time(torch, fn, steps):
 def run_brick14(args):
     """14-qubit random brickwork (20 layers: Haar U(2) on every qubit + CZ on alternating pairs, 410 gates),
     complex128, full output vector. The state is 256 KiB, so every pass is L2-resident and the run is
-    launch-, latency- and FP64-bound: plans of CUDA-core passes run every pass in one resident cooperative
-    launch (grid barriers between passes), and the same plans launched pass by pass from CUDA graphs are timed
-    beside them. Every path's final vector is compared with the per-gate path's (both complex128 on the GPU;
+    launch-, latency- and FP64-bound: plans of CUDA-core passes run in one resident cooperative launch (grid
+    barriers between groups of gates or between passes), and the same plans launched pass by pass from CUDA
+    graphs are timed beside them. Every path's final vector is compared with the per-gate path's (both complex128 on the GPU;
     the test suite pins the per-gate path to the FP64 oracle)."""
     import numpy as np
     import torch
@@ -709,9 +711,14 @@ def run_brick14(args):
         if ref is None:
             ref = psi
         # FP64 arithmetic of the dense passes: every amplitude of a touched group is a 2^k-term complex dot
-        # product (8 2^k real flops); diagonal and phase passes add a few flops per amplitude (not counted)
-        fp64 = sum(8.0 * (1 << q["k"]) * 2.0 ** (n - q["nc"]) for q in p.passes()
-                   if q["kind"] in ("dense_small", "dense_tile"))
+        # product (8 2^k real flops); diagonal and phase passes add a few flops per amplitude (not counted). A
+        # resident plan may apply the gates themselves or products of a few: it is counted gate by gate.
+        if p.info["resident"]:
+            fp64 = sum(8.0 * (1 << len(g.targets)) * 2.0 ** (n - len(g.controls)) for g in c.gates
+                       if np.count_nonzero(g.matrix - np.diag(np.diag(g.matrix))))
+        else:
+            fp64 = sum(8.0 * (1 << q["k"]) * 2.0 ** (n - q["nc"]) for q in p.passes()
+                       if q["kind"] in ("dense_small", "dense_tile"))
         out[name] = {"ms_per_step": ms, "gates_per_s": len(c) / (ms / 1000.0), "passes": p.info["passes"],
                      "resident": bool(p.info["resident"]), "fp64_gflop": fp64 / 1e9,
                      "fp64_tflops": fp64 / (ms / 1000.0) / 1e12,
@@ -745,8 +752,9 @@ def run_brick14(args):
                         roofline={"bound": "alu", "achieved": b["fp64_tflops"], "peak": fp64_peak, "unit": "TFLOP/s",
                                   "frac": b["fp64_tflops"] / fp64_peak, "traffic": None,
                                   "peak_source": "measured: independent FP64 FMA chains on every SM, this run",
-                                  "note": "L2-resident state (no HBM traffic to speak of): the dense passes' FP64 "
-                                          "FMAs against the measured FP64 rate; the rest is barrier and latency",
+                                  "note": "L2-resident state (no HBM traffic to speak of): the FP64 arithmetic of the "
+                                          "dense gates, gate by gate, against the measured FP64 rate; the rest is "
+                                          "barrier and latency",
                                   "hbm_equivalent_gbs": b["achieved_gbs"]},
                         e2e={"value": len(c) / e2e_s, "unit": UNIT,
                              "h2d_bytes_per_step": int(sum(g.matrix.size * 16 + 8 * (len(g.targets) + len(g.controls)) for g in c.gates)),
@@ -847,7 +855,7 @@ def run_tfim_batch(args):
     wide_ms = {("tf32x3 k = 6" if p == 1 else "fp16x3 k <= 7"): round(v[0], 3) for p, v in wide_paths.items()}
     wide_paths[4 if tc_prec == 1 else 1][1].close()
     res = b.results()
-    # the same batch with every circuit in the persistent launch (CUDA cores only)
+    # the same batch in the states' own precision (persistent launch, wide circuits as own-precision plans)
     simt_only = None
     if not args.no_variants:
         bs = qsim.Batch(cs, max_fused=0)
@@ -937,7 +945,7 @@ def run_tfim_batch(args):
                              "d2h_bytes_per_step": 8 * sum(2 * c.n - 1 for c in cs)},
                         tune_s=tune_s, sample_zi0=list(res[0][0][:4]), one_by_one=one_by_one, e2e_breakdown=best,
                         e2e_planned_then_executed=min(staged, key=lambda r: r["total_s"]),
-                        persistent_launch_only=simt_only)
+                        own_precision=simt_only)
     if not args.no_cpu:
         import oracle as oracle_mod
         # oracle on the smallest circuits until the time budget runs out; work ~ gates x 2^n

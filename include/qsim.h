@@ -67,7 +67,8 @@ extern "C" {
 #define QSIM_PREC_FP16X3 4
 
 /* Run modes. */
-#define QSIM_RUN_PLAIN 0 /* one device pass per gate (diagonal gates touch only their non-unit entries) */
+#define QSIM_RUN_PLAIN 0 /* gate by gate: one pass per gate (diagonal gates touch only their non-unit entries); executed
+                            as a whole, gates on common qubits share a read and write of the state */
 #define QSIM_RUN_FUSED 1 /* gates merged into dense or diagonal blocks of at most max_fused qubits */
 
 #define QSIM_MAX_TARGETS 8
@@ -129,10 +130,11 @@ typedef struct {
        two single passes on GB300 (the pass is bound by instruction issue, not memory); for study. */
     int32_t pair_blocks;
     /* Plans of states of at most 16 qubits whose passes are all CUDA-core dense blocks (k <= 5), diagonals
-       (k <= 6) or phase passes run every pass inside ONE cooperative launch, one CTA per SM resident over the plan and a grid
-       barrier between passes (Sec. 2.1: the passes applied in order; at these sizes a pass is a few
-       microseconds of arithmetic, less than a launch costs). Only a whole-plan execution does; a pass range
-       launches per pass. 1 = always one launch per pass (and the CUDA graph of use_graph). */
+       (k <= 6) or phase passes run inside ONE cooperative launch, one CTA per SM resident over the plan and a grid
+       barrier between passes, or between groups of gates on common qubits (Sec. 2.1: applied in order; at these
+       sizes a pass is a few microseconds of arithmetic, less than a launch costs). Only a whole-plan execution
+       does; a pass range launches per pass. 1 = always one launch per pass (and the CUDA graph of use_graph); per-gate
+       plans of wider states then run each gate in a pass of its own too. */
     int32_t launch_per_pass;
 } qsim_run_opts;
 
@@ -451,9 +453,10 @@ int qsim_fp64_peak(double seconds, double* tflops, double* ms);
  * launch, with their <Z> values reduced on the device: one cluster streams a wide state at a fraction of the
  * GPU's bandwidth, a plan's passes use all of it (below 25 qubits a half, below 23 a quarter of the SMs, so
  * that several run side by side). With opts->max_fused = 0 the other circuits of at least 19 qubits are planned
- * too (where that is estimated faster), as blocks of 5 qubits in the states' own precision (QSIM_PREC_SIMT). Those plans run on eight streams the
- * batch owns, forked from the caller's stream and joined back into it, so all work of an execution is ordered
- * before later work on that stream. For circuit i, <Z_q> lands at zi[zi_off(i) + q] (q < n_i) and
+ * too (where that is estimated faster), as blocks of 5 qubits in the states' own precision (QSIM_PREC_SIMT).
+ * Those plans run on eight streams the batch owns, forked from the caller's stream and joined back into it, so
+ * all work of an execution is ordered before later work on that stream. For circuit i, <Z_q> lands at
+ * zi[zi_off(i) + q] (q < n_i) and
  * <Z_q Z_{q+1}> at zz[zz_off(i) + q] (q < n_i - 1), the offsets being the running sums of n_i and n_i - 1
  * in input order; sums are compensated (float-float per thread, double-double across threads), and the
  * values are those of the normalised state (divided by the computed squared norm, which FP32 arithmetic

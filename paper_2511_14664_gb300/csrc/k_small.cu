@@ -1,6 +1,9 @@
 // k_small.cu -- every pass of a small-state plan in ONE cooperative launch (paper Sec. 2.1 "State-Vector
 // Simulation": the gates, or fused blocks, applied one after another to the state vector).
 //
+// This is the path of plans that k_small_tiles.cu, which puts many gates between two barriers, does not take or is
+// estimated slower on (few passes that hold many cheap gates; plan.cu has the rule).
+//
 // For a state of up to 2^16 amplitudes a pass is a few microseconds of arithmetic (at 14 qubits and a
 // complex128 state, a 4-qubit dense block is 2^14 x 64 FP64 FMAs, about 2 us at GB300's FP64 rate spread
 // over every SM), so one launch per pass spends more time starting and draining kernels than computing. Here
