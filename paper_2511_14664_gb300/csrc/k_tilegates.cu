@@ -84,8 +84,14 @@ template <typename T> __device__ __forceinline__ T cscale(T d, T v) {
 template <typename R, int RB, int KIND, bool CTL>
 __device__ __forceinline__ void apply1(typename Amp<R>::T (&v)[NV], const typename Amp<R>::T* c, int rctl) {
     using T = typename Amp<R>::T;
-    const T u0 = c[0], u1 = c[1], u2 = c[2], u3 = c[3];
-    const R a0 = u0.x, a1 = u0.y, b0 = u1.x, b1 = u1.y, c0 = u2.x, c1 = u2.y, d0 = u3.x, d1 = u3.y;
+    R a0, a1, b0, b1, c0, c1, d0, d1;
+    if constexpr (sizeof(R) == 4) {
+        const float4 ab = reinterpret_cast<const float4*>(c)[0], cd = reinterpret_cast<const float4*>(c)[1];
+        a0 = ab.x; a1 = ab.y; b0 = ab.z; b1 = ab.w; c0 = cd.x; c1 = cd.y; d0 = cd.z; d1 = cd.w;
+    } else {
+        const T u0 = c[0], u1 = c[1], u2 = c[2], u3 = c[3];
+        a0 = u0.x; a1 = u0.y; b0 = u1.x; b1 = u1.y; c0 = u2.x; c1 = u2.y; d0 = u3.x; d1 = u3.y;
+    }
 #pragma unroll
     for (int p = 0; p < NV / 2; ++p) {
         const int i = ((p >> RB) << (RB + 1)) | (p & ((1 << RB) - 1)), j = i | (1 << RB);
@@ -109,10 +115,58 @@ __device__ __forceinline__ void apply1(typename Amp<R>::T (&v)[NV], const typena
         }
     }
 }
-// A two-qubit gate on register bits R0 < R1 (matrix bit 0 <-> R0); SWAP exchanges them.
+// A two-qubit gate on register bits R0 < R1 (matrix bit 0 <-> R0); SWAP exchanges them. Without controls complex64 takes
+// two groups of four at a time and reads the matrix two columns at a time: 16 shared-memory loads for 256 FMAs instead
+// of 64 (24 qubits, 96 U(4) gates: 1.75 -> 1.60 ms; 25 qubits, 750 random-circuit gates, where a one-qubit matrix is two
+// loads instead of four: 6.31 -> 5.88 ms).
 template <typename R, int R0, int R1, bool SWAP>
 __device__ __forceinline__ void apply2(typename Amp<R>::T (&v)[NV], const typename Amp<R>::T* c, int rctl) {
     using T = typename Amp<R>::T;
+    if constexpr (!SWAP && sizeof(R) == 4) {
+        if (rctl == 0) {
+#pragma unroll
+            for (int h = 0; h < NV / 8; ++h) {
+                int at[2][4];
+                T x[2][4];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int g = 2 * h + e;
+                    int i = ((g >> R0) << (R0 + 1)) | (g & ((1 << R0) - 1));
+                    i = ((i >> R1) << (R1 + 1)) | (i & ((1 << R1) - 1));
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        at[e][r] = i | ((r & 1) << R0) | ((r >> 1) << R1);
+                        x[e][r] = v[at[e][r]];
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    R re[2] = {0, 0}, im[2] = {0, 0};
+#pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        const float4 u = *reinterpret_cast<const float4*>(c + 4 * r + k);
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            re[e] = fmar(u.x, x[e][k].x, re[e]);
+                            re[e] = fmar(-u.y, x[e][k].y, re[e]);
+                            im[e] = fmar(u.x, x[e][k].y, im[e]);
+                            im[e] = fmar(u.y, x[e][k].x, im[e]);
+                            re[e] = fmar(u.z, x[e][k + 1].x, re[e]);
+                            re[e] = fmar(-u.w, x[e][k + 1].y, re[e]);
+                            im[e] = fmar(u.z, x[e][k + 1].y, im[e]);
+                            im[e] = fmar(u.w, x[e][k + 1].x, im[e]);
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        v[at[e][r]].x = re[e];
+                        v[at[e][r]].y = im[e];
+                    }
+                }
+            }
+            return;
+        }
+    }
 #pragma unroll
     for (int g = 0; g < NV / 4; ++g) {
         int i = ((g >> R0) << (R0 + 1)) | (g & ((1 << R0) - 1));
