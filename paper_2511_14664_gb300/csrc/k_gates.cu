@@ -208,16 +208,25 @@ struct TileArgs {
     uint64_t off[64];
 };
 
-template <typename R, int K>
-__global__ void __launch_bounds__(256)
+// A CTA takes ROWS groups at a time, a thread OUTS rows of the product of one of them: the same FMA chain whichever way.
+// 64 groups (U's rows are read by whole warps) where that leaves a tile for every SM (complex64: for half of them), else
+// 16, 4 or one, so that the arithmetic of a small state is spread. With 64 always, 6-qubit passes took 260 us in
+// complex128 up to 18 qubits and 12 to 14 us in complex64; now 17 us at 14 qubits, 37 at 16, 133 at 18, and 6 to 8 us;
+// 5-qubit passes in complex128 68 us, now 10 to 14, 21 and 68. From 20 qubits on nothing changes.
+template <int K, int ROWS> constexpr int kTileOuts = ROWS == 64 ? (1 << K) / 4 : (ROWS == 16 ? (1 << K) / 16 : 1);
+template <int K, int ROWS> constexpr int kTileThreads = ROWS * (1 << K) / kTileOuts<K, ROWS>;
+template <int K, int ROWS> constexpr int kTilePitch = (1 << K) + (ROWS == 64 ? 0 : 1);  // other lanes, other rows: no conflicts
+
+template <typename R, int K, int ROWS>
+__global__ void __launch_bounds__(kTileThreads<K, ROWS>)
 k_dense_tile(typename Amp<R>::T* __restrict__ psi, uint64_t ngroups, const __grid_constant__ TileArgs a,
              const typename Amp<R>::T* __restrict__ U) {
     using T = typename Amp<R>::T;
-    constexpr int D = 1 << K, ROWS = 64, OUTS = D / 4;
+    constexpr int D = 1 << K, OUTS = kTileOuts<K, ROWS>, LD = kTilePitch<K, ROWS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sU = reinterpret_cast<T*>(smem_raw);  // D x D
-    T* sX = sU + D * D;                      // column-major: sX[c * ROWS + r]
-    for (int i = threadIdx.x; i < D * D; i += blockDim.x) sU[i] = U[i];
+    T* sU = reinterpret_cast<T*>(smem_raw);  // D x D, rows LD apart
+    T* sX = sU + D * LD;                     // column-major: sX[c * ROWS + r]
+    for (int i = threadIdx.x; i < D * D; i += blockDim.x) sU[(i >> K) * LD + (i & (D - 1))] = U[i];
     const int r = threadIdx.x & (ROWS - 1), q = threadIdx.x / ROWS;
     const uint64_t ntiles = (ngroups + ROWS - 1) / ROWS;
     __syncthreads();
@@ -240,7 +249,7 @@ k_dense_tile(typename Amp<R>::T* __restrict__ psi, uint64_t ngroups, const __gri
             const T x = sX[c * ROWS + r];
 #pragma unroll
             for (int j = 0; j < OUTS; ++j) {
-                const T u = sU[(q * OUTS + j) * D + c];
+                const T u = sU[(q * OUTS + j) * LD + c];
                 ar[j] = fmar(u.x, x.x, ar[j]);
                 ar[j] = fmar(-u.y, x.y, ar[j]);
                 ai[j] = fmar(u.x, x.y, ai[j]);
@@ -562,10 +571,24 @@ cudaError_t launch_diag(int dtype, void* psi, int n, int k, const int* targets, 
     return diag_t<double>(psi, n, k, targets, f, diag, touch, s, d);
 }
 
+template <typename R, int K, int ROWS>
+static cudaError_t dense_tile_rows(void* psi, uint64_t ngroups, const TileArgs& a, const void* dmat, cudaStream_t s, const DevInfo& d) {
+    using T = typename Amp<R>::T;
+    constexpr int D = 1 << K;
+    const size_t smem = (size_t)(D * kTilePitch<K, ROWS> + D * ROWS) * sizeof(T);
+    auto kern = k_dense_tile<R, K, ROWS>;
+    cudaError_t e = smem_optin(reinterpret_cast<const void*>(kern), (int)smem);
+    if (e != cudaSuccess) return e;
+    const uint64_t ntiles = (ngroups + ROWS - 1) / ROWS;
+    const int per_sm = smem > 100 * 1024 ? 1 : 3;
+    kern<<<grid_for((int64_t)ntiles, 1, d.num_sms, per_sm), kTileThreads<K, ROWS>, smem, s>>>(
+        reinterpret_cast<T*>(psi), ngroups, a, reinterpret_cast<const T*>(dmat));
+    return cudaGetLastError();
+}
+
 template <typename R, int K>
 static cudaError_t dense_tile_t(void* psi, int n, const int* targets, const Fixed& f, const void* dmat,
                                 cudaStream_t s, const DevInfo& d) {
-    using T = typename Amp<R>::T;
     TileArgs a;
     std::memset(&a, 0, sizeof(a));
     a.nf = f.nf;
@@ -573,15 +596,11 @@ static cudaError_t dense_tile_t(void* psi, int n, const int* targets, const Fixe
     a.cmask = f.cmask;
     constexpr int D = 1 << K;
     for (int m = 0; m < D; ++m) a.off[m] = target_offset(m, K, targets);
-    const size_t smem = (size_t)(D * D + D * 64) * sizeof(T);
-    cudaError_t e = smem_optin(reinterpret_cast<const void*>(k_dense_tile<R, K>), (int)smem);
-    if (e != cudaSuccess) return e;
-    const uint64_t ngroups = 1ull << (n - f.nf);
-    const uint64_t ntiles = (ngroups + 63) / 64;
-    const int per_sm = smem > 100 * 1024 ? 1 : 3;
-    k_dense_tile<R, K><<<grid_for((int64_t)ntiles, 1, d.num_sms, per_sm), 256, smem, s>>>(
-        reinterpret_cast<T*>(psi), ngroups, a, reinterpret_cast<const T*>(dmat));
-    return cudaGetLastError();
+    const uint64_t ngroups = 1ull << (n - f.nf), sms = (uint64_t)std::max(1, d.num_sms);
+    if (ngroups >= (sizeof(R) == 4 ? 32 : 64) * sms) return dense_tile_rows<R, K, 64>(psi, ngroups, a, dmat, s, d);
+    if (ngroups >= 16 * sms) return dense_tile_rows<R, K, 16>(psi, ngroups, a, dmat, s, d);
+    if (ngroups >= 4 * sms) return dense_tile_rows<R, K, 4>(psi, ngroups, a, dmat, s, d);
+    return dense_tile_rows<R, K, 1>(psi, ngroups, a, dmat, s, d);
 }
 
 template <typename R, int K>

@@ -56,7 +56,7 @@ struct PlanOp {
 
 // Where a composed block of k qubits leaves the CUDA cores for k_tcx.cu, by the time of one pass (microseconds, CUDA
 // cores / k_tcx, targets from qubit 6 up): complex128 k = 1 n = 18 / 19 / 20: 8.3 / 11.6, 12.4 / 11.8, 20.6 / 16.5;
-// k = 2 n = 18 / 19: 11.0 / 11.5, 22.6 / 11.8; k = 3 n = 17: 12.4 / 11.4; k = 5 n = 17: 67.7 / 11.5, n = 24: 3457 / 190.
+// k = 2 n = 18 / 19: 11.0 / 11.5, 22.6 / 11.8; k = 3 n = 17: 12.4 / 11.4; k = 5 n = 17: 37.0 / 11.5, n = 24: 3457 / 190.
 // complex64 k = 5 n = 18 / 19: 6.2 / 6.4, 8.2 / 6.5, n = 26: 461 / 246; k = 4 n = 20 / 21 / 24: 21.6 / 8.5, 11.6 / 12.9,
 // 61.5 / 66.2, and with qubit 0 among the targets n = 24: 129 / 79. Below 17 qubits plans run resident (k_small.cu).
 constexpr int kTcxMinQubits = 17;
