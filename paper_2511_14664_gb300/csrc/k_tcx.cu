@@ -83,7 +83,7 @@ template <> struct Cfg<double> {
 };
 template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
 template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
-template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 1; }
+template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 5; }
 template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
 // planes, column offsets, row exponents of the input [2][IN / 4][128] and of tiles in flight
 // [row_slots][128], barriers, the TMEM slot, alignment
@@ -210,15 +210,17 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + bars<R>());
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // barriers: per buffer, A stored (full), accumulators read (freed), MMAs of a plane group retired (done)
+    // barriers: per buffer, A stored (full), accumulators read (freed), MMAs of a plane group retired (done); the
+    // operand loaded (bbar); per quadrant of 32 rows, the row exponents of its input warps written (rowbar)
     auto full = [&](uint32_t b) { return smem_u32(mbar + b); };
     auto freed = [&](uint32_t b) { return smem_u32(mbar + BUF + b); };
     auto done = [&](uint32_t b, int g) { return smem_u32(mbar + (2 + g) * BUF + b); };
-    const uint32_t bbar = smem_u32(mbar + bars<R>() - 1);
+    const uint32_t bbar = smem_u32(mbar + BUF * (2 + GROUPS));
+    auto rowbar = [&](int q) { return smem_u32(mbar + BUF * (2 + GROUPS) + 1 + q); };
     for (int c = tid; c < D; c += threads<R>()) sCol[c] = deposit((uint64_t)c, a.tpos, K);
     if (tid == 0) {
         for (int j = 0; j < bars<R>(); ++j) {
-            const int count = j < BUF ? kIn : (j < 2 * BUF ? kOut : 1);
+            const int count = j < BUF ? kIn : (j < 2 * BUF ? kOut : (j <= BUF * (2 + GROUPS) ? 1 : kIn / 4));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar + j)), "r"(count) : "memory");
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -335,12 +337,16 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             asm volatile("" : "+r"(e) :: "memory");  // before any later load is issued (loads share scoreboards)
             return e;
         };
-        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow.
-        auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) {
+        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow. The
+        // quadrant's warps meet at an mbarrier, whose wait ends when one of them has given up (no warp waits at a named
+        // barrier: it has no limit).
+        auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) -> bool {
             constexpr int EB = DBL ? 20 : 23;  // exponent position in a real's upper word
             uint32_t* const ex = sE + (i & 1) * (kIn / 4 * 128) + r;
             ex[(warp >> 2) * 128] = e;
-            asm volatile("bar.sync %0, %1;" :: "r"(1 + quad), "n"(kIn * 8) : "memory");  // the warps of the quadrant
+            __syncwarp();
+            if (lane == 0) mbar_arrive(rowbar(quad));
+            if (!wait(rowbar(quad), i & 1)) return false;
 #pragma unroll
             for (int k = 0; k < kIn / 4; ++k) e = max(e, ex[k * 128]);
             uint32_t E = max(e >> EB, kLowE<R>);
@@ -383,6 +389,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 #pragma unroll
                 for (int j = 0; j < W; ++j) X[j] = (uint32_t)__float2int_rn(__uint_as_float(X[j]) * up) + 0x80808080u;
             }
+            return true;
         };
         // Digit plane s of the tile: byte S-1-s of every real, less 128, as FP16 pairs (re, im).
         auto store_plane = [&](const uint32_t (&X)[W], int s, uint32_t b) {
@@ -404,7 +411,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         };
         // Tile i: fixed point, then its planes as the planes of tile i - BUF retire.
         auto put = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) -> bool {
-            convert(X, i, e);
+            if (!convert(X, i, e)) return false;
 #pragma unroll
             for (int g = 0; g < GROUPS; ++g) {
                 if (i >= BUF && !wait(done(buf(i), g), par(i - BUF))) return false;
