@@ -134,8 +134,8 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
     uint32_t* sP2 = reinterpret_cast<uint32_t*>(sDepHi + 16);     // [64] T1 column c: B2 byte offset part | xor part << 16
     uint32_t* sStN2 = sP2 + 64;                                   // [128] staging word part of R2 column n2
     uint32_t* sFj = sStN2 + 128;                                  // [16] f of tile bits 9..12
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sFj + 16);       // full1[2] done1[2] full2 done2[2] bops
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 8);
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sFj + 16);       // full1[2] done1[2] full2 done2[2] bops data
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 9);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto fswz = [&](uint32_t hi9) {  // f of tile bits 4..12 (given shifted down by 4)
@@ -170,8 +170,8 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
         sStN2[c] = t ^ fswz(t >> 4);
     }
     if (tid == 0) {
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t cnt = (j < 2 || j == 4) ? kDataWarps : 1;  // full1[0..1], full2: one arrival per data warp
+        for (int j = 0; j < 9; ++j) {
+            const uint32_t cnt = (j < 2 || j == 4 || j == 8) ? kDataWarps : 1;  // full1[0..1], full2, data: one arrival per data warp
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar + j)), "r"(cnt) : "memory");
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -189,7 +189,7 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
     auto done1 = [&](int s) { return bar0 + 8u * (uint32_t)(2 + s); };
     const uint32_t full2 = bar0 + 8u * 4;
     auto done2 = [&](int s) { return bar0 + 8u * (uint32_t)(5 + s); };
-    const uint32_t bbar = bar0 + 8u * 7;
+    const uint32_t bbar = bar0 + 8u * 7, dbar = bar0 + 8u * 8;
     // a programmatic dependent of the kernel before it: its writes are visible from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -298,7 +298,13 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
             fence_after();
             return ok;
         };
-        auto data_sync = [&]() { asm volatile("bar.sync 1, %0;" :: "r"(kDataThreads) : "memory"); };
+        // The data warps meet at an mbarrier, whose wait ends when one of them has given up (a named barrier has no limit).
+        uint32_t met = 0;
+        auto data_sync = [&]() -> bool {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dbar);
+            return wait(dbar, met++ & 1);
+        };
         float2 X[kCPT];
         auto load = [&](uint64_t t) {
             const uint64_t b = insert_zeros(t, a.spos, kTileBits) + rowoff1;
@@ -365,7 +371,7 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
                 asm volatile("st.shared.v2.f32 [%0], {%1, %2};" :: "r"(sB2 + 8u * word), "f"(re * kOut), "f"(im * kOut)
                              : "memory");
             }
-            data_sync();
+            if (!data_sync()) return false;
             const uint64_t b = insert_zeros(t, a.spos, kTileBits) + deplo;
 #pragma unroll 8
             for (int jj = 0; jj < 16; ++jj) {
@@ -374,8 +380,7 @@ k_tc_pair(float2* __restrict__ psi, const __grid_constant__ PairArgs a, const ui
                 asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(y.x), "=f"(y.y) : "r"(sB2 + 8u * word) : "memory");
                 psi[b + sDepHi[jj]] = y;
             }
-            data_sync();  // the staging buffer is the next tile's B2
-            return true;
+            return data_sync();  // the staging buffer is the next tile's B2
         };
         // Tile j lives in TMEM slot j & 1. Per iteration: finish MMA 1 of tile j (p2), fill tile j + 2's A1
         // while MMA 2 of tile j runs, store tile j (p3), then release slot j & 1 to tile j + 2.
@@ -484,7 +489,7 @@ cudaError_t launch_tc_pair(void* psi, int n, const int* t1, const int* t2, const
     if ((reinterpret_cast<uintptr_t>(dops) & 15) != 0) return cudaErrorInvalidValue;
     if (from_basis) { a.from_basis = 1; a.basis = *from_basis; }
     // operands, tables and barriers; at least 120 KiB, so that one CTA (one TMEM owner) runs per SM
-    const size_t smem = std::max<size_t>((size_t)tcp::kOffTab + (64 + 512 + 16) * 8 + (64 + 128 + 16) * 4 + 8 * 8 + 16 + 1024,
+    const size_t smem = std::max<size_t>((size_t)tcp::kOffTab + (64 + 512 + 16) * 8 + (64 + 128 + 16) * 4 + 8 * 9 + 8 + 16 + 1024,
                                          120 * 1024);
     cudaError_t e = cudaFuncSetAttribute(tcp::k_tc_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

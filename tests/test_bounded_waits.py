@@ -10,7 +10,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_14664_gb300", "csrc")
 
 
-@pytest.mark.parametrize("name", ["k_tcx.cu"])
+@pytest.mark.parametrize("name", ["k_tcx.cu", "k_tc_pair.cu", "k_tc.cu", "k_tc7.cu"])
 def test_no_named_barrier_beside_bounded_waits(name):
     text = open(os.path.join(CSRC, name)).read()
     assert "mbar_wait_bounded" in text
