@@ -50,8 +50,15 @@ extern "C" {
 
 /* Arithmetic used for fused dense blocks (Sec. 2.1: fusion trades flops for arithmetic intensity). */
 #define QSIM_PREC_SIMT 0   /* the state's own precision: CUDA-core FMA, or, for fused blocks of
-                              up to 5 qubits where it is faster, exact integer products on the
-                              tensor cores, whose error is no larger */
+                              up to 5 qubits where it is faster (from 17 qubits on), sums of
+                              exact integer products on the tensor cores. Those work relative to
+                              the largest amplitude of a row (the amplitudes that a block joins,
+                              in a block of fewer than 5 qubits those of up to 32 that lie beside
+                              them): in norm the error is below that of FMA, and amplitude by
+                              amplitude below 2^-16 (complex64) or 2^-43 (complex128) of
+                              sum_c |U_rc| |x_c|, of which a chain of FMAs may lose 2^-18 or 2^-47.
+                              Rows of too wide a range for that are taken by FMA, so that small
+                              amplitudes keep their digits */
 #define QSIM_PREC_TF32X3 1 /* tensor cores: 3 TF32 products (hi*hi + hi*lo + lo*hi), FP32 accumulation */
 #define QSIM_PREC_BF16X3 2 /* tensor cores: 2-way BF16 split, 3 products, FP32 accumulation. REDUCED
                               accuracy (~16 significant bits per product, not complex64 level): ~1e-8

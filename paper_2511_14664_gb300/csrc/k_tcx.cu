@@ -16,10 +16,24 @@
 //     (2^-28) of the row's scale.
 //   * y = 2^(E') sum_d D_d 2^(-8d): in complex128 summed in a 64-bit integer and rounded once, in complex64 by
 //     three FMAs.
-// The errors are those of the fixed-point steps, 2^-55 (2^-31) of the row's scale, and of the final rounding:
-// smaller than the accumulated roundings of 64 FMAs (against 64 bits, 23-qubit brickwork of depth 10: 1.6e-15,
-// by FMAs 1.8e-15; 26-qubit random pairs in complex64: 2.3e-7, by FMAs 1.0e-6). A row with an infinity or NaN
-// gives NaN.
+// The errors are those of the fixed-point steps, of the positions left out and of the final rounding, all relative to the
+// row's largest amplitude: at most 2^-25 (2^-52) of the power of two above it, in rms 2^-27 (2^-54) in the emulated
+// digit arithmetic; smaller than the accumulated roundings of 64 FMAs (against 64 bits, 23-qubit brickwork of depth 10: 1.6e-15,
+// by FMAs 1.8e-15; 26-qubit random pairs in complex64: 2.3e-7, by FMAs 1.0e-6).
+//
+// Rows by FMAs. That is an error of the row, and an amplitude that is small beside its row's largest one would lose its
+// digits (R_y(2e-4) on five qubits of |0>: the amplitude of two flips, 1e-8, came out with 2 % error in complex64, that of
+// three as zero). So the slices take a row only where every result y_i has sum_c |U_ic| |x_c| above 2^-9 of that power of
+// two, which bounds its error by 2^-16 (2^-43) of that sum, beside 2^-18 (2^-47) for a chain of 64 FMAs: rows whose amplitudes
+// lie within kRange = 8 binades of the largest (the entries of a row of U sum to 1 or more), and rows in which every row
+// of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4. The others (0.1 % of the rows of a
+// random state) are chains of FMAs in the state's precision (rows_by_fma): a few of a quadrant's 32 rows by three
+// warps beside the MMA issuer, many by the output. So are rows outside the exponents that the slices take; a row with an
+// infinity or NaN gives NaN. One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0:
+// 276, 351 / 242, 261 us, and without this 254, 309 / 201, 239; with amplitudes over 30 binades 850 / 800 (CUDA cores 461 / 3457);
+// 16-step TFIM chains of small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 10.2 / 4.0 -> 10.2 ms. Left: all rows by the
+// three warps (11.6 / 14.9 ms there, and no faster elsewhere); one warp that decides for all rows (2.7 ms a pass at wide rows);
+// kRange = 7 (284 us in complex64).
 //
 // Layout. A tile is 128 rows (the 7 lowest index bits outside the block) by 32 columns; blocks of fewer qubits
 // take idle qubits as further columns (U x I). Digit plane s of a tile is a K-major operand of 128 x 64 FP16
@@ -29,15 +43,15 @@
 // the reads of A from shared memory would bound it).
 //
 // Roles, one CTA per SM: input warps load a tile, convert it and write its planes; one warp issues the MMAs;
-// output warps sum the positions, convert back and store. In complex64 (16 input, 8 output warps) planes and
+// output warps sum the positions, convert back and store; three more take rows by FMAs. In complex64 (16 input, 8 output warps) planes and
 // accumulators are double-buffered, and the next tile's loads are in flight in registers. In complex128 the 8
 // positions take all of tensor memory and the planes half of shared memory, so a tile's MMAs commit in four
 // groups of planes: as a group retires, the input (8 warps) writes the next tile's planes over it and the output
 // (16 warps) adds the positions it finished.
-// Bound: complex64 (26 qubits, 246 us, 0.65 of the copy rate) the input's loads and conversion; complex128 (24
-// qubits, 190 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
+// Bound: complex64 (26 qubits, 276 us, 0.57 of the copy rate) the input's loads and conversion; complex128 (24
+// qubits, 242 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
 // and on the integer pipe about as fast, so they are spread over both; the tensor cores work a quarter of the
-// time. Measured and left: one set of warps for input and output (281 us at 24 qubits), 8 output warps (208),
+// time. Measured and left (against 190 us without the rows by FMAs): one set of warps for input and output (281 us at 24 qubits), 8 output warps (208),
 // the next tile staged by cp.async (204), L2 prefetch of the next tile (212), the D_d to integers by F2I (213).
 // Every mbarrier wait is bounded (2 s); on expiry the kernel records DEVERR_TIMEOUT, waits once more (bounded)
 // for its MMAs, frees its tensor memory and returns.
@@ -66,8 +80,13 @@ template <> struct Cfg<float> {
     static constexpr int S = 4, ND = 4;        // digits; digit positions kept
     static constexpr int BUF = 2;              // tiles in flight: A planes and accumulators
     static constexpr int GROUPS = 1;           // commits per tile
-    static constexpr int IN = 16, OUT = 8, MMA = 1;  // warps: tile loads and digit planes; accumulators and stores; MMAs
+    static constexpr int IN = 16, OUT = 8, MMA = 4;  // warps: tile loads and digit planes; accumulators and stores; MMAs (one) and rows by FMAs
     static constexpr int kStepsU = 30;         // U in 2^-30 steps
+    static constexpr int kRange = 8;           // binades below the row's largest amplitude that the slices take
+    static constexpr int ROWS = 4;             // rows an output warp takes at a time by FMAs
+    static constexpr int FEW = 8;              // fewer of a quadrant's 32 rows: left to the row warps
+    static constexpr int LOOK = FEW;           // so many: the input looks at U before it gives them away
+    static constexpr int U = D;                // rows of U in shared memory, for them
     __host__ __device__ static constexpr int group_end(int) { return S; }
 };
 template <> struct Cfg<double> {
@@ -75,23 +94,34 @@ template <> struct Cfg<double> {
     static constexpr int BUF = 1;
     static constexpr int GROUPS = 4;           // planes 0-1, 2-3, 4-5, 6
     // Whole warpgroups, so that registers can move between them: launched with 72 a thread (28 warps, 64512 in
-    // all), the input takes 96, the output keeps 64, the MMA warpgroup (one warp works) 56: 64512.
+    // all), the input takes 96, the output keeps 64, the MMA warpgroup 56: 64512.
     static constexpr int IN = 8, OUT = 16, MMA = 4;
     static constexpr int kRegIn = 96, kRegOut = 64, kRegMma = 56;
     static constexpr int kStepsU = 54;
+    static constexpr int kRange = 8;
+    static constexpr int ROWS = 1;
+    static constexpr int FEW = 4;
+    static constexpr int LOOK = 1;             // (one row by FMAs is 10 us of a 12 us pass at 19 qubits)
+    static constexpr int U = 0;                // (stays in global memory: 16 KiB more would take L1 from the loads in flight)
     __host__ __device__ static constexpr int group_end(int g) { return g < 3 ? 2 * g + 2 : S; }
 };
+template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
+constexpr int kRowWarps = 3;
+constexpr int kQueue = 16;  // entries of a quadrant's queue of rows for the row warps
 template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
 template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
 template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 5; }
-template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
-// planes, column offsets, row exponents of the input [2][IN / 4][128] and of tiles in flight
-// [row_slots][128], barriers, the TMEM slot, alignment
+// planes, column offsets, largest and smallest amplitudes of the input's rows [2][IN / 4][128] and which of them are large
+// [IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the row
+// warps' queues [4][kQueue][2] and how far their producers are [4], the large entries of U [32][2], U and the rows taken by FMAs [OUT][ROWS][32] [kRowWarps][32], alignment
+template <typename R> constexpr int smem_rows() { return (Cfg<R>::OUT * Cfg<R>::ROWS + kRowWarps + Cfg<R>::U) * D * 2 * (int)sizeof(R); }
 template <typename R> constexpr size_t smem_bytes() {
-    return smem_planes<R>() + 8 * D + 4 * (2 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
-           8 * bars<R>() + 8 + 1024;
+    return smem_planes<R>() + smem_rows<R>() + 16 * D + 4 * (3 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
+           8 * bars<R>() + 8 + 4 * (8 * kQueue + 4) + 1024;
 }
-static_assert(smem_bytes<float>() <= 227 * 1024 && smem_bytes<double>() <= 227 * 1024, "");
+// With 1 KiB that the system takes, below the 196 KiB that leave 60 KiB of L1: the data of loads in flight lies there
+// (complex128, 24 qubits: 201 us a pass; with 28 KiB, 239).
+static_assert(smem_bytes<float>() <= 195 * 1024 && smem_bytes<double>() <= 195 * 1024, "");
 
 // How a thread moves its columns: one amplitude per access (lane = row); the columns of qubit 0 (target 0) as
 // one vector of two; the columns of qubits 0 and 1 (targets 0 and 1) as one 32-byte vector of four (complex64).
@@ -105,6 +135,7 @@ struct Args {
     uint64_t ntiles;
     int from_basis;      // the input is |basis>, generated in registers instead of read
     uint64_t basis;
+    int k;               // the block's own qubits: column bits 0 .. k - 1
     int32_t w[4];        // 2^30, 2^22, 2^14, 2^6 (as parameters, so that they stay multiplications)
 };
 
@@ -140,11 +171,12 @@ template <int N> __device__ __forceinline__ void st_words(void* p, const uint32_
         asm volatile("st.global.v2.b32 [%0], {%1,%2};" :: "l"(p), "r"(w[0]), "r"(w[1]) : "memory");
 }
 
-// Rows whose largest exponent is below this are scaled up first (rare), so that a zero or subnormal amplitude
-// next to a larger one falls below the fixed-point step and needs no case of its own.
+// Largest exponents of a row that the slices take: from kLowE on, a zero or subnormal real next to a larger one falls
+// below the fixed-point step and needs no case of its own, and results stay normal; up to kHighE (complex128: to_fixed_cvt
+// adds 1076 - E to exponents) they do not overflow.
 template <typename R> constexpr uint32_t kLowE = sizeof(R) == 8 ? 64 : 32;
-template <typename R> constexpr int kLowScale = sizeof(R) == 8 ? 200 : 64;  // 2^200 (2^64)
-constexpr uint32_t kHighE = 1076;  // complex128 rows above it are scaled down by 2^-1000: to_fixed adds 1076 - E to exponents
+template <typename R> constexpr uint32_t kHighE = sizeof(R) == 8 ? 1076 : 247;
+constexpr int kByFma = 1 << 20;  // in place of a row's exponent: the output takes the row by FMAs
 
 // The fixed-point value of a real whose row has largest biased exponent E, plus 128 in every base-256 digit
 // (so that the bytes of the result are the digits plus 128). |x| < 2^(E - 1022) maps to 2^54 steps. Two ways that
@@ -161,7 +193,7 @@ __device__ __forceinline__ void to_fixed_int(uint32_t& lo, uint32_t& hi, uint32_
 }
 __device__ __forceinline__ void to_fixed_cvt(uint32_t& lo, uint32_t& hi, uint32_t E) {
     // x 2^(1076 - E) by its exponent field; a zero or subnormal becomes a value below 2^-10, which rounds to 0
-    const double x = __hiloint2double((int)(hi + ((kHighE - E) << 20)), (int)lo);
+    const double x = __hiloint2double((int)(hi + ((kHighE<double> - E) << 20)), (int)lo);
     const uint64_t v = (uint64_t)__double2ll_rn(x) + 0x0080808080808080ull;
     lo = (uint32_t)v;
     hi = (uint32_t)(v >> 32);
@@ -185,6 +217,114 @@ __device__ __forceinline__ void to_double_cvt(int64_t Y, int E, uint32_t& lo, ui
     hi = h ? h + ((uint32_t)(E - 1080) << 20) : 0u;
 }
 
+__device__ __forceinline__ float fmar(float x, float y, float z) { return __fmaf_rn(x, y, z); }
+__device__ __forceinline__ double fmar(double x, double y, double z) { return __fma_rn(x, y, z); }
+
+// The rows in `mine` of 32 (`at`: the index of the lane's row) in the state's own arithmetic: sums of FMA chains over
+// eight columns each (a chain over all 32, as in the CUDA-core blocks, has 1.7 times the error: 4.8 units of 2^-24 of the
+// state's largest amplitude at 21 qubits), without the columns that are zero in every row. Nobody else stores these
+// rows. A warp takes whole rows, NROW at a time, so that it has read a row before it is written; a lane is a column of
+// the result, `col` its index bits; xs: room for NROW rows; u: U by columns.
+template <typename R, int NROW>
+__device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args& a, const typename Amp<R>::T* u, typename Amp<R>::T* xs,
+                                            uint64_t col, uint32_t mine, uint64_t at) {
+    using T = typename Amp<R>::T;
+    constexpr bool DBL = sizeof(R) == 8;
+    const int lane = threadIdx.x & 31, Du = 1 << a.k, g0 = lane & ~(Du - 1);
+    const T* const ucol = u + (lane & (Du - 1));
+    while (mine) {
+        uint64_t p[NROW];
+        uint32_t nz = 0;
+        bool finite[NROW], has[NROW];
+        T x[NROW], y[NROW];
+#pragma unroll
+        for (int q = 0; q < NROW; ++q) {
+            has[q] = mine != 0;
+            p[q] = __shfl_sync(0xffffffffu, at, mine ? __ffs(mine) - 1 : 0) + col;
+            mine &= mine - 1;
+        }
+#pragma unroll
+        for (int q = 0; q < NROW; ++q) {
+            x[q].x = x[q].y = y[q].x = y[q].y = 0;
+            if (has[q]) {
+                if (a.from_basis) x[q].x = p[q] == a.basis ? (R)1 : (R)0;
+                else x[q] = psi[p[q]];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NROW; ++q) {
+            nz |= __ballot_sync(0xffffffffu, x[q].x != 0 || x[q].y != 0);
+            finite[q] = __all_sync(0xffffffffu, isfinite(x[q].x) && isfinite(x[q].y));
+            xs[q * D + lane] = x[q];
+        }
+        __syncwarp();
+        for (int g = D / 2; g >= Du; g >>= 1) nz |= nz >> g;  // columns of the block
+        if (Du < D) nz &= (1u << Du) - 1;
+        while (nz) {
+            const int c0 = (__ffs(nz) - 1) & 24;
+            const uint32_t now = (nz >> c0) & 0xFFu;
+            nz &= ~(0xFFu << c0);
+            T part[NROW];
+#pragma unroll
+            for (int q = 0; q < NROW; ++q) part[q].x = part[q].y = 0;
+            auto column = [&](T w, int q, T z) {
+                part[q].x = fmar(w.x, z.x, part[q].x);
+                part[q].x = fmar(-w.y, z.y, part[q].x);
+                part[q].y = fmar(w.x, z.y, part[q].y);
+                part[q].y = fmar(w.y, z.x, part[q].y);
+            };
+            if (!DBL && now == 0xFFu) {  // (complex128: FP64 bounds this, not the loads)
+#pragma unroll
+                for (int c = 0; c < 8; c += 2) {
+                    const T w0 = ucol[(c0 + c) * Du], w1 = ucol[(c0 + c + 1) * Du];
+#pragma unroll
+                    for (int q = 0; q < NROW; ++q) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(xs + q * D + g0 + c0 + c);
+                        T z0, z1;
+                        z0.x = (R)__uint_as_float(v.x); z0.y = (R)__uint_as_float(v.y);
+                        z1.x = (R)__uint_as_float(v.z); z1.y = (R)__uint_as_float(v.w);
+                        column(w0, q, z0);
+                        column(w1, q, z1);
+                    }
+                }
+            } else {
+                T ahead = ucol[(c0 + __ffs(now) - 1) * Du];
+                for (uint32_t left = now; left; left &= left - 1) {
+                    const int c = c0 + __ffs(left) - 1;
+                    const T w = ahead;
+                    if (left & (left - 1)) ahead = ucol[(c0 + __ffs(left & (left - 1)) - 1) * Du];
+#pragma unroll
+                    for (int q = 0; q < NROW; ++q) column(w, q, xs[q * D + g0 + c]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < NROW; ++q) {
+                y[q].x += part[q].x;
+                y[q].y += part[q].y;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NROW; ++q) {
+            if (!finite[q]) y[q].x = y[q].y = DBL ? (R)__hiloint2double(0x7FF80000, 0) : (R)__uint_as_float(0x7FC00000u);
+            if (has[q]) psi[p[q]] = y[q];
+        }
+        __syncwarp();  // xs has been read
+    }
+}
+// Not inlined in complex64: inside the output's loop its registers cost the slices 6 % (complex128, whose warps have
+// registers of their own, inlines it: a function may use as many as the kernel was launched with).
+template <int NROW>
+__device__ __noinline__ void rows_by_fma_call(float2* psi, const Args& a, const float2* u, float2* xs, uint64_t col, uint32_t mine,
+                                              uint64_t at) {
+    rows_by_fma<float, NROW>(psi, a, u, xs, col, mine, at);
+}
+template <typename R, int NROW>
+__device__ __forceinline__ void rows_any(typename Amp<R>::T* psi, const Args& a, const typename Amp<R>::T* u, typename Amp<R>::T* xs,
+                                         uint64_t col, uint32_t mine, uint64_t at) {
+    if constexpr (sizeof(R) == 4) rows_by_fma_call<NROW>(psi, a, u, xs, col, mine, at);
+    else rows_by_fma<R, NROW>(psi, a, u, xs, col, mine, at);
+}
+
 template <typename R, int MODE>
 __global__ void __launch_bounds__(threads<R>(), 1)
 k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a, const uint4* __restrict__ bops,
@@ -203,11 +343,19 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sA = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sB = sA + BUF * S * kPlaneA;
-    uint64_t* sCol = reinterpret_cast<uint64_t*>(sB + S * kPlaneB);
-    uint32_t* sE = reinterpret_cast<uint32_t*>(sCol + D);             // [2][kIn / 4][128]
-    int* sRow = reinterpret_cast<int*>(sE + 2 * (kIn / 4) * 128);     // [row_slots][128]
+    T* sU = reinterpret_cast<T*>(sB + S * kPlaneB);                   // U by columns (complex64)
+    T* sX = sU + C::U * D;                                               // [kOut][ROWS][32], [kRowWarps][32]
+    uint64_t* sCol = reinterpret_cast<uint64_t*>(sX + (kOut * C::ROWS + kRowWarps) * D);
+    uint4* sL = reinterpret_cast<uint4*>(sCol + D);                   // [16]: of two rows of U each, large entries
+    uint32_t* sE = reinterpret_cast<uint32_t*>(sL + D / 2);           // [2][kIn / 4][128]
+    uint32_t* sBig = sE + 2 * (kIn / 4) * 128;                        // [kIn / 4][128]
+    int* sRow = reinterpret_cast<int*>(sBig + (kIn / 4) * 128);       // [row_slots][128]
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sRow + row_slots<R>() * 128);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + bars<R>());
+    volatile uint32_t* const qmask = tslot + 2;           // [4][kQueue]: rows of a quadrant, 0 = free
+    volatile uint32_t* const qtile = qmask + 4 * kQueue;  // [4][kQueue]: their tile
+    volatile uint32_t* const qdone = qtile + 4 * kQueue;  // [4]: tiles whose rows are queued; all ones after the last
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // barriers: per buffer, A stored (full), accumulators read (freed), MMAs of a plane group retired (done); the
@@ -217,6 +365,8 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     auto done = [&](uint32_t b, int g) { return smem_u32(mbar + (2 + g) * BUF + b); };
     const uint32_t bbar = smem_u32(mbar + BUF * (2 + GROUPS));
     auto rowbar = [&](int q) { return smem_u32(mbar + BUF * (2 + GROUPS) + 1 + q); };
+    for (int c = tid; c < 4 * kQueue; c += threads<R>()) qmask[c] = 0;
+    if (tid < 4) qdone[tid] = 0;
     for (int c = tid; c < D; c += threads<R>()) sCol[c] = deposit((uint64_t)c, a.tpos, K);
     if (tid == 0) {
         for (int j = 0; j < bars<R>(); ++j) {
@@ -237,6 +387,8 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     // programmatic dependent launch: the set-up above overlapped the previous kernel's tail
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int* const sums = reinterpret_cast<const int*>(reinterpret_cast<const char*>(bops) + S * kPlaneB);
+    const T* const umat = reinterpret_cast<const T*>(sums + NR + 2 * D);  // U by columns
     const uint32_t t0 = blockIdx.x, G = gridDim.x;  // (fewer than 2^32 tiles: checked by the host)
     const uint32_t m = t0 < a.ntiles ? (uint32_t)((a.ntiles - t0 + G - 1) / G) : 0u;  // tiles of this CTA
     auto tile = [&](uint32_t i) { return (uint64_t)t0 + (uint64_t)i * G; };
@@ -253,15 +405,19 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 
     bool bad = false;
     if (warp >= kIn + kOut) {
-        // ---- MMA issuer ----
+        // ---- MMA issuer, and three warps that take rows by FMAs ----
         if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegMma));
         if (warp == kIn + kOut && lane == 0) {
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bbar), "r"(S * kPlaneB) : "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bbar), "r"(S * kPlaneB + (C::U > 0 ? (int)sizeof(T) << (2 * a.k) : 0))
+                         : "memory");
 #pragma unroll 1
             for (int j = 0; j < S; ++j)
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                              :: "r"(smem_u32(sB) + j * kPlaneB), "l"(reinterpret_cast<const char*>(bops) + j * kPlaneB),
                                 "r"(kPlaneB), "r"(bbar) : "memory");
+            if constexpr (C::U > 0)
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             :: "r"(smem_u32(sU)), "l"(umat), "r"((int)sizeof(T) << (2 * a.k)), "r"(bbar) : "memory");
             const uint64_t d0 = sdesc_sw128(smem_u32(sA));
             const uint32_t hi = (uint32_t)(d0 >> 32), alo0 = (uint32_t)d0;
             const uint32_t blo = (uint32_t)sdesc_sw128(smem_u32(sB));
@@ -305,12 +461,57 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                 if (issued) mbar_wait_bounded(done(buf(issued - 1), GROUPS - 1), par(issued - 1));  // the MMAs already issued
             }
         }
+        if (warp > kIn + kOut) {
+            // Row warps: the rows of quadrants that have a few of them, any time (in the output they would hold up a tile: in
+            // complex128 a row is 8192 cycles of the FP64 units beside a warp). Warp w has every third entry of the queues.
+            const int w = warp - (kIn + kOut + 1);
+            T* const xs = sX + (kOut * C::ROWS + w) * D;
+            const uint64_t col = sCol[lane];
+            bad = !wait(bbar, 0);  // U
+            uint64_t since = globaltimer();
+            uint32_t seen = 0;
+            while (!bad) {
+                const uint32_t done_tiles = lane < 4 ? qdone[lane] : kAll;
+                const bool last = __all_sync(0xffffffffu, done_tiles == kAll);
+                __threadfence_block();  // what was queued before that
+                bool found = false;
+#pragma unroll 1
+                for (int h = 0; h < 4 * kQueue; h += 32) {
+                    const uint32_t m = (h + lane) % kRowWarps == w ? qmask[h + lane] : 0u;
+                    for (uint32_t at = __ballot_sync(0xffffffffu, m != 0); at; at &= at - 1) {
+                        const int l = __ffs(at) - 1, slot = h + l, q = slot / kQueue;
+                        const uint32_t mine = __shfl_sync(0xffffffffu, m, l);
+                        __threadfence_block();
+                        const uint64_t row = insert_zeros(tile(qtile[slot]), a.spos, a.nS) + deposit((uint64_t)(32 * q + lane), a.rpos, kRowBits);
+                        rows_any<R, 1>(psi, a, C::U > 0 ? sU : umat, xs, col, mine, row);
+                        __threadfence_block();
+                        __syncwarp();
+                        if (lane == 0) qmask[slot] = 0;
+                        found = true;
+                    }
+                }
+                if (last && !found) break;
+                const uint32_t sum = __reduce_add_sync(0xffffffffu, done_tiles);
+                if (found || sum != seen) {
+                    seen = sum;
+                    since = globaltimer();
+                } else if (__any_sync(0xffffffffu, globaltimer() - since > 2000000000ull)) {
+                    bad = true;  // no producer has moved
+                } else {
+                    __nanosleep(500);
+                }
+            }
+            if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
+        }
         __syncwarp();
     } else if (warp < kIn) {
         // ---- input: load a tile, convert it to fixed point, write its digit planes ----
         if constexpr (DBL) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegIn));
         const int c0 = CPI * (warp >> 2);
         const volatile uint64_t* vCol = sCol + c0;
+        // every warp writes the same words of sL and reads its own writes
+        reinterpret_cast<uint2*>(sL)[lane] = make_uint2((uint32_t)sums[NR + lane], (uint32_t)sums[NR + D + lane]);
+        __syncwarp();
         const T* const prow = psi + deposit((uint64_t)r, a.rpos, kRowBits);
         unsigned char* const arow = sA + (r >> 3) * 1024 + (r & 7) * 128;
         auto load_tile = [&](uint32_t (&X)[W], uint64_t t) {
@@ -328,56 +529,96 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                 for (int j = 0; j < CPI; j += VEC) ld_words<VEC * AW>(prow + b + vCol[j], X + AW * j);
             }
         };
-        // The largest magnitude (upper word) of the thread's reals: waits for the tile's loads, so that those of the
-        // next tile can start.
-        auto top = [&](const uint32_t (&X)[W]) {
-            uint32_t e = 0;
-#pragma unroll
-            for (int j = DBL ? 1 : 0; j < W; j += DBL ? 2 : 1) e = max(e, X[j] & 0x7FFFFFFFu);
-            asm volatile("" : "+r"(e) :: "memory");  // before any later load is issued (loads share scoreboards)
-            return e;
+        // The largest and the smallest magnitude (upper words; an amplitude's is that of its larger part) of the thread's
+        // amplitudes: waits for the tile's loads, so that those of the next tile can start.
+        // Packed: exponent of the largest (at least 1 unless all are zero) << 16 | 0x7FFF - exponent of the smallest.
+        constexpr int EB = DBL ? 20 : 23;  // exponent position in a real's upper word
+        auto amplitude = [&](const uint32_t (&X)[W], int j) {
+            return max(X[AW * j + (DBL ? 1 : 0)] & 0x7FFFFFFFu, X[AW * j + (DBL ? 3 : 1)] & 0x7FFFFFFFu);
         };
-        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow. The
-        // quadrant's warps meet at an mbarrier, whose wait ends when one of them has given up (no warp waits at a named
-        // barrier: it has no limit).
-        auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) -> bool {
-            constexpr int EB = DBL ? 20 : 23;  // exponent position in a real's upper word
-            uint32_t* const ex = sE + (i & 1) * (kIn / 4 * 128) + r;
-            ex[(warp >> 2) * 128] = e;
+        auto span = [&](const uint32_t (&X)[W]) {
+            uint32_t top = 0, low = kAll;
+#pragma unroll
+            for (int j = 0; j < CPI; ++j) {
+                top = max(top, amplitude(X, j));
+                low = min(low, amplitude(X, j));
+            }
+            asm volatile("" : "+r"(top), "+r"(low) :: "memory");  // before any later load is issued (loads share scoreboards)
+            return (max(top >> EB, min(top, 1u)) << 16) | (0x7FFFu - (low >> EB));
+        };
+        // Rows of the quadrant to the row warps' queue (by one warp of the quadrant). False if there was no room in 2 s.
+        uint32_t queued = 0;
+        auto queue_rows = [&](uint32_t rows, uint32_t i) -> bool {
+            const int slot = quad * kQueue + (int)(queued++ % kQueue);
+            bool ok = true;
+            if (lane == 0) {
+                const uint64_t since = globaltimer();
+                while (ok && qmask[slot] != 0) ok = globaltimer() - since <= 2000000000ull;
+                if (ok) {
+                    __threadfence_block();
+                    qtile[slot] = i;
+                    __threadfence_block();
+                    qmask[slot] = rows;
+                }
+            }
+            return __all_sync(0xffffffffu, ok);
+        };
+        // The warps of the quadrant meet at an mbarrier, whose wait ends when one of them has given up (no warp waits at a
+        // named barrier: it has no limit).
+        uint32_t met = 0;
+        auto meet = [&]() -> bool {
             __syncwarp();
             if (lane == 0) mbar_arrive(rowbar(quad));
-            if (!wait(rowbar(quad), i & 1)) return false;
+            return wait(rowbar(quad), met++ & 1);
+        };
+        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow, or kByFma
+        // for a row that the slices do not take: one with amplitudes more than kRange binades below its largest, unless
+        // every row of U has a large entry at a large amplitude. False if a wait ran out. `planes` is false where no row of
+        // the warp needs its digits.
+        auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e, bool& planes) -> bool {
+            uint32_t* const ex = sE + (i & 1) * (kIn / 4 * 128) + r;
+            ex[(warp >> 2) * 128] = e;
+            if (!meet()) return false;
 #pragma unroll
-            for (int k = 0; k < kIn / 4; ++k) e = max(e, ex[k * 128]);
-            uint32_t E = max(e >> EB, kLowE<R>);
-            int scaled = 0;  // the row was multiplied by 2^scaled
-            const bool low = e != 0 && (e >> EB) < kLowE<R>, high = DBL && (e >> EB) > kHighE;
-            if (__any_sync(0xffffffffu, low || high)) {
-                if (low || high) {
-                    if constexpr (DBL) {
-                        scaled = low ? kLowScale<R> : -1000;
-                        const double f = __longlong_as_double((long long)(1023 + scaled) << 52);
-                        const uint32_t E2 = (uint32_t)__double2hiint(__hiloint2double((int)e, low ? -1 : 0) * f) >> EB;
-                        E = (e >> EB) == 0x7FF ? kHighE : max(E2, kLowE<R>);
-                        if ((e >> EB) == 0x7FF) scaled = (int)kHighE - 0x7FF;  // E - scaled says so
+            for (int k = 0; k < kIn / 4; ++k) e = __vmaxu2(e, ex[k * 128]);
+            const uint32_t E0 = e >> 16, low = 0x7FFFu - (e & 0xFFFFu), E = min(max(E0, kLowE<R>), kHighE<R>);
+            bool by_fma = E0 != 0 && (E0 != E || E0 - low > (uint32_t)C::kRange);
+            uint32_t rows = __ballot_sync(0xffffffffu, by_fma);  // (the same in all warps of the quadrant)
+            if (__popc(rows) >= C::LOOK) {
+                // its columns within 1 and within 4 binades of the largest; has every row of U an entry of 2^-7, or of 2^-4, there?
+                uint32_t big = 0;
 #pragma unroll
-                        for (int j = 0; j < W; j += 2) {
-                            const double x = __hiloint2double((int)X[j + 1], (int)X[j]) * f;
-                            X[j] = (uint32_t)__double2loint(x);
-                            X[j + 1] = (uint32_t)__double2hiint(x);
-                        }
-                    } else {
-                        scaled = kLowScale<R>;
-                        const float f = __uint_as_float((uint32_t)(127 + kLowScale<R>) << 23);
-                        E = max(__float_as_uint(__uint_as_float(e) * f) >> EB, kLowE<R>);
-#pragma unroll
-                        for (int j = 0; j < W; ++j) X[j] = __float_as_uint(__uint_as_float(X[j]) * f);
-                    }
+                for (int j = 0; j < CPI; ++j) {
+                    const uint32_t m = amplitude(X, j) >> EB;
+                    big |= (m + 1 >= E0 ? 1u << j : 0u) | (m + 4 >= E0 ? 0x10000u << j : 0u);
                 }
+                sBig[(warp >> 2) * 128 + r] = big;
+                if (!meet()) return false;
+                uint32_t b1 = 0, b4 = 0;
+#pragma unroll
+                for (int k = 0; k < kIn / 4; ++k) {
+                    const uint32_t v = sBig[k * 128 + r];
+                    b1 |= (v & 0xFFFFu) << (CPI * k);
+                    b4 |= (v >> 16) << (CPI * k);
+                }
+                bool held = E0 == E;
+#pragma unroll (DBL ? D / 2 : 2)
+                for (int k = 0; k < D / 2; ++k) {
+                    const uint4 l = sL[k];
+                    held = held & (((b1 & l.x) | (b4 & l.y)) != 0) & (((b1 & l.z) | (b4 & l.w)) != 0);
+                }
+                by_fma = by_fma && !held;
+                rows = __ballot_sync(0xffffffffu, by_fma);
             }
             // read by the output warps after this tile's MMAs. The planes of tile i - 1 were stored, so the MMAs of
             // tile i - 1 - BUF have run, for which tile i - 1 - 2 BUF had been read: 2 BUF + 1 slots or more will do
-            if (warp < 4) sRow[i % row_slots<R>() * 128 + r] = (int)E - scaled;
+            if (warp < 4) {
+                sRow[i % row_slots<R>() * 128 + r] = by_fma ? kByFma : (int)E;
+                if (rows && __popc(rows) < C::FEW && !queue_rows(rows, i)) return false;
+                if (lane == 0) qdone[quad] = i + 1;
+            }
+            planes = rows != kAll;
+            if (!planes) return true;
             if constexpr (DBL) {
 #pragma unroll
                 for (int j = 0; j < W; j += 2) {
@@ -385,7 +626,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                     else to_fixed_cvt(X[j], X[j + 1], E);
                 }
             } else {
-                const float up = __uint_as_float((283u - min(E, 255u)) << 23);  // 2^(156 - E): |x| < 2^(E - 126) to 2^30 steps
+                const float up = __uint_as_float((283u - E) << 23);  // 2^(156 - E): |x| < 2^(E - 126) to 2^30 steps
 #pragma unroll
                 for (int j = 0; j < W; ++j) X[j] = (uint32_t)__float2int_rn(__uint_as_float(X[j]) * up) + 0x80808080u;
             }
@@ -411,12 +652,14 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         };
         // Tile i: fixed point, then its planes as the planes of tile i - BUF retire.
         auto put = [&](uint32_t (&X)[W], uint32_t i, uint32_t e) -> bool {
-            if (!convert(X, i, e)) return false;
+            bool planes;
+            if (!convert(X, i, e, planes)) return false;
 #pragma unroll
             for (int g = 0; g < GROUPS; ++g) {
                 if (i >= BUF && !wait(done(buf(i), g), par(i - BUF))) return false;
 #pragma unroll
-                for (int s = g ? C::group_end(g - 1) : 0; s < C::group_end(g); ++s) store_plane(X, s, buf(i));
+                for (int s = g ? C::group_end(g - 1) : 0; s < C::group_end(g); ++s)
+                    if (planes) store_plane(X, s, buf(i));
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -427,22 +670,25 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             uint32_t X[W];
             for (uint32_t i = 0; i < m; ++i) {
                 load_tile(X, tile(i));
-                if (!put(X, i, top(X))) { bad = true; break; }
+                if (!put(X, i, span(X))) { bad = true; break; }
             }
         } else {  // one tile ahead in registers
             uint32_t XA[W], XB[W];
             if (m > 0) load_tile(XA, tile(0));
             for (uint32_t i = 0; i < m; i += 2) {
-                const uint32_t ea = top(XA);
+                const uint32_t ea = span(XA);
                 if (i + 1 < m) load_tile(XB, tile(i + 1));
                 if (!put(XA, i, ea)) { bad = true; break; }
                 if (i + 1 >= m) break;
-                const uint32_t eb = top(XB);
+                const uint32_t eb = span(XB);
                 if (i + 2 < m) load_tile(XA, tile(i + 2));
                 if (!put(XB, i + 1, eb)) { bad = true; break; }
             }
         }
         if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
+        __threadfence_block();
+        __syncwarp();
+        if (warp < 4 && lane == 0) qdone[quad] = kAll;  // the row warps may leave
     } else {
         // ---- output: sum the digit positions, convert back, store ----
         if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegOut));
@@ -450,17 +696,30 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         const volatile uint64_t* vCol = sCol + c0;
         T* const prow = psi + deposit((uint64_t)r, a.rpos, kRowBits);
         const uint32_t trow = tbase + ((uint32_t)(quad * 32) << 16) + 2 * c0;
-        constexpr int kNan = DBL ? 0x7FF : 0xFF;  // the row held an infinity or NaN
         // whether every |D_d| <= 2^22: the digits of X are at most 128, so the sum of a row of U's bounds them
-        const int* const sums = reinterpret_cast<const int*>(reinterpret_cast<const char*>(bops) + S * kPlaneB);
         [[maybe_unused]] const bool bounded = !__any_sync(0xffffffffu, max(sums[lane], sums[lane + 32]) > (1 << 15));
         auto finish = [&](uint32_t i) {  // the accumulators have been read
             fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(freed(buf(i)));
         };
+        // The output's own rows: of quadrants that have many, shared out among the quadrant's warps.
+        bool have_u = false;
+        auto quad_rows = [&](uint32_t mask, uint64_t at) -> bool {
+            if (__popc(mask) < C::FEW) return true;
+            if (!have_u && !wait(bbar, 0)) return false;
+            have_u = true;
+            uint32_t mine = 0;
+            int rank = 0;
+            for (; mask; mask &= mask - 1, ++rank)
+                if (rank / C::ROWS % (kOut / 4) == ((warp - kIn) >> 2)) mine |= mask & (0u - mask);
+            rows_any<R, C::ROWS>(psi, a, C::U > 0 ? sU : umat, sX + (warp - kIn) * (C::ROWS * D), sCol[lane], mine, at);
+            return true;
+        };
         for (uint32_t i = 0; i < m; ++i) {
             const uint32_t td = trow + buf(i) * 64 * ND;
+            const uint64_t tb = insert_zeros(tile(i), a.spos, a.nS);
+            T* const pt = prow + tb;
             if constexpr (DBL) {
                 // Y = sum_d D_d 2^(46 - 8d), the last two positions together and rounded; y = Y 2^(E - 1080).
                 // The integers come as q + kMagic: the bits of D + 1.5 2^23 where |D| <= 2^22, else by conversion
@@ -469,9 +728,16 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                 constexpr int64_t kOff = (int64_t)kMagic * ((1ll << 30) + (1ll << 22) + (1ll << 14) + (1ll << 6));
                 constexpr uint64_t kY0 = 0ull - (uint64_t)kOff - ((uint64_t)((kMagic << 14) + (kMagic << 6)) << 32);
                 int64_t Y[2 * CPO];
+                int E = 0;
+                uint32_t mask = 0;  // the quadrant's rows that are not in the accumulators
 #pragma unroll
                 for (int g = 0; g < GROUPS; ++g) {
                     if (!wait(done(buf(i), g), par(i))) { bad = true; break; }
+                    if (g == 0) {
+                        E = sRow[i % row_slots<R>() * 128 + r];
+                        mask = __ballot_sync(0xffffffffu, E == kByFma);
+                    }
+                    if (mask == 0xffffffffu) continue;
 #pragma unroll
                     for (int c = 0; c < 2 * CPO; c += 8) {
                         uint32_t v[8], v2[8];
@@ -506,65 +772,48 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                     }
                 }
                 if (bad) break;
-                const int E = sRow[i % row_slots<R>() * 128 + r];
                 finish(i);
-                // rows near either end of the exponent range take a multiplication that can overflow or underflow
-                const bool rare = __any_sync(0xffffffffu, E < (int)kLowE<R> || E > kNan - 8);
-                T* const pt = prow + insert_zeros(tile(i), a.spos, a.nS);
 #pragma unroll
                 for (int j = 0; j < CPO; j += VEC) {
                     uint32_t w[VEC * AW];
 #pragma unroll
                     for (int k = 0; k < 2 * VEC; ++k) {
-                        const int64_t Yk = Y[2 * j + k];
-                        if (rare) {  // two steps: 2^(E - 1080) alone may be below the range
-                            double y = __ll2double_rn(Yk) * 0x1p-58;
-                            y = E >= kNan ? __hiloint2double(0x7FF80000, 0)
-                                          : E > 0 ? (y * 2.0) * __hiloint2double(E << 20, 0)
-                                                  : (y * __hiloint2double((E + 256) << 20, 0)) * 0x1p-255;
-                            w[2 * k] = (uint32_t)__double2loint(y);
-                            w[2 * k + 1] = (uint32_t)__double2hiint(y);
-                        } else if (((2 * j + k) & 3) == 0) {
-                            to_double_int(Yk, E, w[2 * k], w[2 * k + 1]);
-                        } else {
-                            to_double_cvt(Yk, E, w[2 * k], w[2 * k + 1]);
-                        }
+                        if (((2 * j + k) & 3) == 0) to_double_int(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
+                        else to_double_cvt(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
                     }
-                    st_words<VEC * AW>(pt + vCol[j], w);
+                    if (E != kByFma) st_words<VEC * AW>(pt + vCol[j], w);
                 }
+                if (!quad_rows(mask, (uint64_t)(pt - psi))) { bad = true; break; }
             } else {
                 // y = 2^(E - 138) sum_d D_d 2^(-8d)
                 if (!wait(done(buf(i), 0), par(i))) { bad = true; break; }
                 const int E = sRow[i % row_slots<R>() * 128 + r];
-                const bool rare = __any_sync(0xffffffffu, E < (int)kLowE<R> || E > kNan - 8);
+                const uint32_t mask = __ballot_sync(0xffffffffu, E == kByFma);  // rows that are not in the accumulators
                 const float sc = __uint_as_float((uint32_t)(E - 11) << 23);
-                T* const pt = prow + insert_zeros(tile(i), a.spos, a.nS);
+                if (mask == 0xffffffffu) finish(i);
+                else {
 #pragma unroll
-                for (int c = 0; c < 2 * CPO; c += 8) {
-                    uint32_t v[4][8], w[8];
+                    for (int c = 0; c < 2 * CPO; c += 8) {
+                        uint32_t v[4][8], w[8];
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) tmem_ld<8>(td + 64 * d + c, v[d]);
-                    wait_ld();
-                    if (c + 8 == 2 * CPO) finish(i);
+                        for (int d = 0; d < 4; ++d) tmem_ld<8>(td + 64 * d + c, v[d]);
+                        wait_ld();
+                        if (c + 8 == 2 * CPO) finish(i);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float y = __uint_as_float(v[3][j]);
-                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[2][j]));
-                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[1][j]));
-                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
-                        if (rare) {
-                            y *= 0x1p-12f;
-                            y = E >= kNan ? __uint_as_float(0x7FC00000u)
-                                          : E > 0 ? (y * 2.0f) * __uint_as_float((uint32_t)E << 23)
-                                                  : (y * __uint_as_float((uint32_t)(E + 96) << 23)) * 0x1p-95f;
-                        } else {
-                            y *= sc;
+                        for (int j = 0; j < 8; ++j) {
+                            float y = __uint_as_float(v[3][j]);
+                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[2][j]));
+                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[1][j]));
+                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
+                            w[j] = __float_as_uint(y * sc);
                         }
-                        w[j] = __float_as_uint(y);
-                    }
+                        if (E != kByFma) {
 #pragma unroll
-                    for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
+                            for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
+                        }
+                    }
                 }
+                if (!quad_rows(mask, (uint64_t)(pt - psi))) { bad = true; break; }
             }
         }
         if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
@@ -579,7 +828,9 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 
 // The digit planes of U (x I on the padding columns): real form B[2i][2c] = Re U_ic, B[2i][2c+1] = -Im U_ic,
 // B[2i+1][2c] = Im U_ic, B[2i+1][2c+1] = Re U_ic in fixed point, plane t = digit t (most significant first).
-// After the planes, the sum of |digits| over all planes of each row (64 integers). One block per row n.
+// After the planes: the sum of |digits| over all planes of each row (64 integers); for each complex row of U x I the columns
+// whose entry has a part of at least 2^-7, and of at least 2^-4 (32 words each); U itself by columns in the state's
+// precision. One block per row n.
 template <typename R>
 __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U, int k, unsigned char* __restrict__ out) {
     using C = Cfg<R>;
@@ -589,6 +840,19 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
     if ((i >> k) == (c >> k)) {
         const int e = 2 * ((i & (Du - 1)) * Du + (c & (Du - 1)));
         v = (n & 1) == (kk & 1) ? U[e] : ((n & 1) ? U[e + 1] : -U[e + 1]);
+        if (i < Du && c < Du && !(n & 1) && !(kk & 1)) {
+            typename Amp<R>::T u;
+            u.x = (R)U[e];
+            u.y = (R)U[e + 1];
+            reinterpret_cast<typename Amp<R>::T*>(out + C::S * kPlaneB + 4 * (NR + 2 * D))[c * Du + i] = u;
+        }
+    }
+    // thread kk of row 2 i has a part of U_ic (c = kk / 2); of the two, the larger counts
+    const double part = fmax(fabs(v), fabs(__shfl_xor_sync(0xffffffffu, v, 1)));
+    __shared__ uint32_t large[2][2];
+    for (int l = 0; l < 2; ++l) {
+        const uint32_t b = __ballot_sync(0xffffffffu, part >= (l ? 0x1p-4 : 0x1p-7));
+        if ((kk & 31) == 0) large[l][kk >> 5] = b;
     }
     const uint64_t f = (uint64_t)__double2ll_rn(scalbn(v, C::kStepsU)) + (sizeof(R) == 8 ? 0x0080808080808080ull : 0x80808080ull);
     const uint32_t off = sw128_offset(n, kk, NR, 2);
@@ -601,7 +865,13 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
     sum = __reduce_add_sync(0xffffffffu, sum);
     if ((kk & 31) == 0) total[kk >> 5] = sum;
     __syncthreads();
-    if (kk == 0) reinterpret_cast<int*>(out + C::S * kPlaneB)[n] = total[0] + total[1];
+    int* const tail = reinterpret_cast<int*>(out + C::S * kPlaneB);
+    if (kk == 0) tail[n] = total[0] + total[1];
+    if (kk < 2 && !(n & 1)) {
+        uint32_t m = 0;
+        for (int c = 0; c < D; ++c) m |= (large[kk][c >> 4] >> (2 * (c & 15)) & 1u) << c;
+        tail[NR + D * kk + i] = (int)m;
+    }
 }
 
 }  // namespace tcx
@@ -609,7 +879,8 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
 bool tcx_supported(int n, int k) { return k >= 1 && k <= tcx::K && n >= tcx::K + tcx::kRowBits && n <= 43; }
 
 size_t tcx_operand_bytes(int dtype) {
-    return (size_t)tcx::kPlaneB * (dtype == QSIM_C64 ? tcx::Cfg<float>::S : tcx::Cfg<double>::S) + sizeof(int) * tcx::NR;
+    return (size_t)tcx::kPlaneB * (dtype == QSIM_C64 ? tcx::Cfg<float>::S : tcx::Cfg<double>::S) + sizeof(int) * (tcx::NR + 2 * tcx::D) +
+           (size_t)(dtype == QSIM_C64 ? sizeof(float2) : sizeof(double2)) * tcx::D * tcx::D;
 }
 
 cudaError_t launch_tcx_prepare(int dtype, const double* dU, int k, void* dB, cudaStream_t s) {
@@ -644,6 +915,7 @@ cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targ
     for (int j = 0; j < tcx::kRowBits; ++j) smask |= 1ull << a.rpos[j];
     for (int q = 0; q < n; ++q)
         if ((smask >> q) & 1) a.spos[a.nS++] = q;
+    a.k = k;
     a.ntiles = 1ull << (n - a.nS);
     if (a.ntiles >> 32) return cudaErrorInvalidValue;  // 32-bit tile counters in the kernel
     if (from_basis) {

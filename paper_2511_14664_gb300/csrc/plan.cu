@@ -55,14 +55,16 @@ struct PlanOp {
 };
 
 // Where a composed block of k qubits leaves the CUDA cores for k_tcx.cu, by the time of one pass (microseconds, CUDA
-// cores / k_tcx, targets from qubit 6 up): complex128 k = 1 n = 18 / 19 / 20: 8.3 / 11.6, 12.4 / 11.8, 20.6 / 16.5;
-// k = 2 n = 18 / 19: 11.0 / 11.5, 22.6 / 11.8; k = 3 n = 17: 12.4 / 11.4; k = 5 n = 17: 37.0 / 11.5, n = 24: 3457 / 190.
-// complex64 k = 5 n = 18 / 19: 6.2 / 6.4, 8.2 / 6.5, n = 26: 461 / 246; k = 4 n = 20 / 21 / 24: 21.6 / 8.5, 11.6 / 12.9,
-// 61.5 / 66.2, and with qubit 0 among the targets n = 24: 129 / 79. Below 17 qubits plans run resident (k_small.cu).
+// cores / k_tcx, targets from qubit 6 up unless said): complex128 k = 2 n = 18 / 19: 11.8 / 11.5, 22.7 / 12.5; k = 3 n = 17:
+// 12.4 / 12.0; k = 5 n = 17: 37 / 12.0, n = 24: 3457 / 243; k = 1 n = 18 / 19 / 20: 8.3 / 11.6, 12.4 / 11.8, 20.6 / 16.5 (before
+// rows by FMAs). complex64 k = 5 n = 17 / 18 / 19: 6.2 / 6.7, 6.2 / 6.9, 8.3 / 7.3, from qubit 0 up 6.3 / 7.4, 8.3 / 7.6, 12.4 / 7.9, n = 26:
+// 462 / 276; k = 4 n = 17 / 20 / 21: 10.4 / 6.3, 22.2 / 9.4, 12.3 / 15 (the CUDA-core pass of 17 to 20 qubits is that slow by
+// itself, not looked into here), and with qubit 0 among the targets n = 21 / 24: 22.7 / 15.8, 130 / 90. Below 17 qubits plans run
+// resident (k_small.cu).
 constexpr int kTcxMinQubits = 17;
 static bool tcx_pays(int dtype, int n, int k, const int* targets) {
     if (dtype == QSIM_C128) return n >= (k == 1 ? 20 : (k == 2 ? 19 : kTcxMinQubits));
-    if (k == 5) return n >= kTcxMinQubits;  // (level up to 18, and the error is smaller)
+    if (k == 5) return n >= kTcxMinQubits;  // (level up to 18, and the error in norm is smaller)
     if (k != 4 || n < kTcxMinQubits) return false;
     bool q0 = false;
     for (int j = 0; j < k; ++j) q0 = q0 || targets[j] == 0;
