@@ -28,8 +28,8 @@
 // lie within kRange = 8 binades of the largest (the entries of a row of U sum to 1 or more), and rows in which every row
 // of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4. The others (0.1 % of the rows of a
 // random state) are chains of FMAs in the state's precision (rows_by_fma): a few of a quadrant's 32 rows by three
-// warps beside the MMA issuer, many by the output. So are rows outside the exponents that the slices take; a row with an
-// infinity or NaN gives NaN. One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0:
+// warps beside the MMA issuer, many by the output. So are rows outside the exponents that the slices take; amplitudes
+// that the block joins with an infinity or NaN become NaN. One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0:
 // 276, 351 / 242, 261 us, and without this 254, 309 / 201, 239; with amplitudes over 30 binades 850 / 800 (CUDA cores 461 / 3457);
 // 16-step TFIM chains of small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 10.2 / 4.0 -> 10.2 ms. Left: all rows by the
 // three warps (11.6 / 14.9 ms there, and no faster elsewhere); one warp that decides for all rows (2.7 ms a pass at wide rows);
@@ -235,7 +235,7 @@ __device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args&
     while (mine) {
         uint64_t p[NROW];
         uint32_t nz = 0;
-        bool finite[NROW], has[NROW];
+        bool has[NROW];
         T x[NROW], y[NROW];
 #pragma unroll
         for (int q = 0; q < NROW; ++q) {
@@ -254,7 +254,6 @@ __device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args&
 #pragma unroll
         for (int q = 0; q < NROW; ++q) {
             nz |= __ballot_sync(0xffffffffu, x[q].x != 0 || x[q].y != 0);
-            finite[q] = __all_sync(0xffffffffu, isfinite(x[q].x) && isfinite(x[q].y));
             xs[q * D + lane] = x[q];
         }
         __syncwarp();
@@ -305,7 +304,10 @@ __device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args&
         }
 #pragma unroll
         for (int q = 0; q < NROW; ++q) {
-            if (!finite[q]) y[q].x = y[q].y = DBL ? (R)__hiloint2double(0x7FF80000, 0) : (R)__uint_as_float(0x7FC00000u);
+            // (read again: a flag a row through the loop above would cost registers that the output's loop has to save)
+            const T own = xs[q * D + lane];
+            const uint32_t wild = __ballot_sync(0xffffffffu, !isfinite(own.x) || !isfinite(own.y));
+            if ((wild >> g0) & (Du < D ? (1u << Du) - 1 : 0xffffffffu)) y[q].x = y[q].y = DBL ? (R)__hiloint2double(0x7FF80000, 0) : (R)__uint_as_float(0x7FC00000u);
             if (has[q]) psi[p[q]] = y[q];
         }
         __syncwarp();  // xs has been read

@@ -104,3 +104,22 @@ def test_rows_of_wide_range(qsim, dtype, spread, kind, n, qubits):
     ref = x @ U.T
     total = (np.abs(x) @ np.abs(U).T).astype(np.float64)
     assert np.all(np.abs(out - ref).astype(np.float64) <= TOL[dtype] * total + np.finfo(np.float32).tiny * (dtype == C64))
+
+
+@pytest.mark.parametrize("dtype,n,qubits", [(C64, 20, (2, 6, 11, 17)), (C128, 20, (2, 6, 11, 17)), (C128, 18, (0, 5, 12)),
+                                            (C128, 20, (4, 19)), (C128, 21, (7,))])
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_non_finite_amplitudes_stay_in_their_groups(qsim, dtype, n, qubits, value):
+    """Blocks padded with idle qubits: only the amplitudes that the block joins with a non-finite one become so."""
+    rng = np.random.default_rng(n)
+    psi0 = (rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)).astype(DT[dtype])
+    c = circuit(n, qubits, "dense", seed=3)
+    good = run(qsim, c, dtype, psi0)
+    at = 0b101100111001011001101 & ((1 << n) - 1)
+    psi0[at] = value
+    out = run(qsim, c, dtype, psi0)
+    mask = sum(1 << q for q in qubits)
+    group = (np.arange(1 << n) & ~mask) == (at & ~mask)
+    assert np.count_nonzero(group) == 1 << len(qubits)
+    assert not np.any(np.isfinite(out[group]))
+    assert np.max(np.abs(out[~group] - good[~group])) <= 2 * TOL[dtype] * np.max(np.abs(good[~group]))
