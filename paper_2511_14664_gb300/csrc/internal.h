@@ -4,11 +4,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <functional>
 #include <string>
 #include <vector>
 
 #include "../../include/qsim.h"
+#include "tile_cut.h"
 
 namespace qsim {
 
@@ -72,7 +72,6 @@ cudaError_t launch_small_run(int dtype, void* psi, int n, void* dprog, int npass
                              const DevInfo& d, const uint64_t* from_basis);
 
 // ---- small states: many gates between two grid barriers (k_small_tiles.cu) ------------------------------------
-struct TileGate;
 struct SmallTiles {
     int groups = 0;          // 0: none
     int arith = 0;           // QSIM_C64 or QSIM_C128: the type of its arithmetic; the state keeps its own
@@ -117,15 +116,6 @@ cudaError_t launch_phase(int dtype, void* psi, int n, const void* dtab, const Ph
                          const DevInfo& d);
 
 // ---- many gates of a per-gate plan in one pass over the state (k_tilegates.cu) --------------------------------
-struct TileGate {
-    bool ok = false;             // tile_gate_ok: may join a group
-    bool diag = false;
-    int k = 0, nc = 0;
-    int q[2] = {0, 0};           // targets; for a diagonal (k = 1 or 2, nc = 0) all its qubits
-    int ctl[QSIM_MAX_CONTROLS] = {0};
-    uint64_t tmask = 0, all = 0; // targets; targets and controls
-    std::vector<double> mat;     // 2^k x 2^k, or the diagonal's 2^k entries (interleaved)
-};
 struct TileGroup {
     std::vector<int> members;    // gates, in the order they are applied
     int pos[12] = {0};           // index bits of the tile
@@ -133,12 +123,6 @@ struct TileGroup {
     std::vector<uint64_t> prog;
 };
 constexpr int kTileMinQubits = 17;  // narrower plans run resident (k_small.cu, k_small_tiles.cu)
-// Gates cut into groups of which each acts on `bits` qubits at most (diagonals and controls on any), in an order that keeps
-// that of gates that share a qubit (diagonals among themselves excepted). The qubits in lowset count in every group;
-// `size` adds up to max_size at most, gates to max_ops. A gate that is not ok is a group of its own.
-struct TileCut { std::vector<int> members; uint64_t set = 0; };
-std::vector<TileCut> tile_cut(const std::vector<TileGate>& g, int bits, uint64_t lowset, const std::function<int(const TileGate&)>& size,
-                              int max_size, int max_ops);
 // Dense gates on 1 or 2 targets with any controls, diagonals on at most 2 qubits in all.
 bool tile_gate_ok(bool diag, int k, int nc);
 // The groups a list of gates is applied in (each gate once; gates that share a qubit keep their order unless both are

@@ -374,26 +374,6 @@ static int gf2_rank(std::vector<uint32_t> v) {
     return rank;
 }
 
-// Operations ready in order: each takes its place unless one left behind shares a qubit (diagonals pass diagonals),
-// and its targets grow `set` up to `limit` bits (diagonals have no targets here: they go anywhere).
-static std::vector<int> collect(const std::vector<TileGate>& g, const std::vector<int>& und, int seed, uint64_t& set, int limit,
-                                uint64_t within) {
-    std::vector<int> out;
-    uint64_t bany = 0, bdiag = 0;
-    if (seed >= 0) set |= g[seed].tmask;
-    for (int i : und) {
-        const bool blocked = g[i].diag ? (g[i].all & bany) != 0 : (g[i].all & (bany | bdiag)) != 0;
-        const uint64_t want = g[i].diag ? 0 : g[i].tmask;
-        if (g[i].ok && !blocked && (want & ~within) == 0 && __builtin_popcountll(set | want) <= limit) {
-            set |= want;
-            out.push_back(i);
-        } else {
-            (g[i].diag ? bdiag : bany) |= g[i].all;
-        }
-    }
-    return out;
-}
-
 template <typename R>
 static void emit_group(const std::vector<TileGate>& g, const std::vector<int>& members, uint64_t set, int n, TileGroup& out) {
     constexpr int B = kBits<R>, TB = kThrBits<R>, LB = sizeof(R) == 4 ? 4 : 3;
@@ -416,7 +396,7 @@ static void emit_group(const std::vector<TileGate>& g, const std::vector<int>& m
             if (u > 0 && (c.diag || (c.all & seen))) { seen |= c.all; continue; }
             seen |= c.all;
             uint64_t s = 0;
-            std::vector<int> got = collect(g, und, c.diag ? -1 : und[u], s, kReg, set);
+            std::vector<int> got = tile_collect(g, und, c.diag ? -1 : und[u], s, kReg, set, ~0ull);
             if (got.size() > best.size()) { best.swap(got); best_set = s; }
         }
         for (int q = n - 1; q >= 0 && __builtin_popcountll(best_set) < kReg; --q) best_set |= set & (1ull << q);
@@ -538,46 +518,6 @@ static void emit_group(const std::vector<TileGate>& g, const std::vector<int>& m
 }  // namespace tile
 
 bool tile_gate_ok(bool diag, int k, int nc) { return diag ? k + nc <= 2 : k <= 2; }
-
-std::vector<TileCut> tile_cut(const std::vector<TileGate>& g, int bits, uint64_t lowset, const std::function<int(const TileGate&)>& size,
-                              int max_size, int max_ops) {
-    std::vector<TileCut> out;
-    std::vector<int> und;
-    for (int i = 0; i < (int)g.size(); ++i) und.push_back(i);
-    while (!und.empty()) {
-        TileCut cut;
-        if (!g[und[0]].ok) {  // no group takes it: alone
-            cut.members = {und[0]};
-            und.erase(und.begin());
-            out.push_back(std::move(cut));
-            continue;
-        }
-        uint64_t seen = 0;
-        int tried = 0;
-        for (size_t u = 0; u < und.size() && tried < 12; ++u) {
-            const TileGate& c = g[und[u]];
-            const bool free_ = (c.all & seen) == 0;
-            seen |= c.all;
-            if (!c.ok || !free_ || (u > 0 && c.diag)) continue;
-            ++tried;
-            uint64_t set = lowset;
-            std::vector<int> got = tile::collect(g, und, c.diag ? -1 : und[u], set, bits, ~0ull);
-            if (got.size() > cut.members.size()) { cut.members.swap(got); cut.set = set; }
-        }
-        // a program larger than the room set aside for it is cut short
-        int used = 0;
-        for (size_t m = 0; m < cut.members.size(); ++m) {
-            used += size(g[cut.members[m]]);
-            if ((used > max_size || m >= (size_t)max_ops) && m > 0) { cut.members.resize(m); break; }
-        }
-        std::vector<int> rest;
-        for (int i : und)
-            if (!std::binary_search(cut.members.begin(), cut.members.end(), i)) rest.push_back(i);
-        und.swap(rest);
-        out.push_back(std::move(cut));
-    }
-    return out;
-}
 
 std::vector<TileGroup> tile_groups(int dtype, int n, const std::vector<TileGate>& g) {
     const int B = dtype == QSIM_C64 ? tile::kBits<float> : tile::kBits<double>;
