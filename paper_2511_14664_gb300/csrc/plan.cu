@@ -427,6 +427,49 @@ static double op_bytes(const PlanOp& op, int n, size_t amp) {
     return 2.0 * amp * groups * (double)(1 << op.k);
 }
 
+// Whether a group of gates is faster in one pass over tiles than gate by gate: gates with controls and diagonals touch a part
+// of the state only, the pass reads and writes all of it. Estimates in microseconds from measured plans of 2 to 20 gates
+// (17 to 27 qubits). Gate by gate: a launch, 5.8 TB/s, in complex128 FP64 at 578 FMAs a nanosecond. Tiles: 5.6 TB/s, then each
+// gate's arithmetic (complex64: instruction issue, at 27 qubits 25 to 80 us; complex128: FP64), by the
+// SM with the most tiles, halved by each control outside the tile where an SM has several. Measured, gate by gate / in one pass: two X with 8 controls, 27
+// qubits complex64 15 / 383; 20 CZ, 27 qubits complex64 2061 / 679, 26 qubits complex128 2926 / 4664; 20 phases, 26 qubits
+// complex128 5685 / 9357; 750 random-circuit gates, 25 qubits complex64 53800 / 5880; four X with 3 controls, 17 qubits complex128
+// 17.6 / 25.
+static bool tile_pass_pays(int dtype, int n, const TileGroup& grp, const std::vector<TileGate>& tg, const std::vector<PlanOp>& ops,
+                           int num_sms) {
+    const bool dbl = dtype == QSIM_C128;
+    const size_t amp = dbl ? sizeof(double2) : sizeof(float2);
+    const int tile_bits = dbl ? 11 : 12;
+    const double state = std::ldexp(1.0, n), fp64 = 578e3, tiles = std::ldexp(1.0, n - tile_bits);
+    const double spread = num_sms * std::ceil(tiles / num_sms) / tiles;  // the SM with the most tiles
+    uint64_t set = 0;
+    for (int j = 0; j < tile_bits; ++j) set |= 1ull << grp.pos[j];
+    double single = 0.0, tile = std::max(4.5, 2.0 + 2.0 * amp * state / 5.6e6);
+    for (int i : grp.members) {
+        const TileGate& g = tg[i];
+        const double bytes = op_bytes(ops[i], n, amp);
+        const std::vector<double>& m = g.mat;
+        bool sign = g.diag;  // a diagonal of 1 and -1: no complex product
+        for (size_t x = 0; sign && x < m.size(); x += 2) sign = (m[x] == 1.0 || m[x] == -1.0) && m[x + 1] == 0.0;
+        bool cheap = !g.diag && g.k == 1;  // real, or real diagonal with imaginary off-diagonal
+        if (cheap) cheap = (m[1] == 0 && m[3] == 0 && m[5] == 0 && m[7] == 0) || (m[1] == 0 && m[7] == 0 && m[2] == 0 && m[4] == 0);
+        const double fmas = g.diag ? (sign ? 2.0 : 4.0) : g.k == 2 ? 16.0 : cheap && g.nc == 0 ? 4.0 : 8.0;
+        double part = 1.0;
+        if (tiles > 4.0 * num_sms)
+            for (int j = 0; j < g.nc; ++j) part *= (set >> g.ctl[j]) & 1 ? 1.0 : 0.5;
+        if (dbl) {
+            const double own = g.diag && sign ? 0.0 : g.diag ? 4.0 : g.k == 2 ? 16.0 : 8.0;
+            single += std::max(4.1, 2.0 + std::max(bytes / 5.8e6, own * bytes / (2.0 * amp) / fp64));
+            tile += 0.1 + part * fmas * state * spread / fp64;
+        } else {
+            single += std::max(4.1, 2.0 + bytes / 5.8e6);
+            const double us27 = g.diag ? (sign ? 16.0 : 25.0) : g.k == 2 ? 80.0 : g.nc > 0 ? 45.0 : cheap ? 25.0 : 33.0;
+            tile += 0.1 + part * us27 * state * spread / std::ldexp(1.0, 27);
+        }
+    }
+    return tile < single;
+}
+
 // Plan buffers come from a memory pool of the library's own (stream-ordered allocation): planning on several
 // host threads at once, and one-shot runs that create and destroy a plan per call, then avoid the device-wide
 // locking of cudaMalloc / cudaFree. Up to 256 MiB of freed plan buffers stay reserved in the pool for reuse.
@@ -976,12 +1019,16 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
             tg.push_back(tile_gate(op.kind == OP_DIAG, op.k, op.nc, op.targets, op.controls, op.mat.data()));
             tg.back().ok = tg.back().ok && (op.kind == OP_DIAG || op.kind == OP_DENSE_SMALL);
         }
-        // At 17 qubits a complex128 state has 64 tiles, fewer than the SMs: two-qubit dense gates are bound by FP64 there
-        // and faster spread over all SMs gate by gate (0.39 against 0.45 ms for 48 of them); others gain (170
-        // random-circuit gates 0.89 -> 0.37 ms).
-        size_t dense2 = 0;
-        for (const TileGate& t : tg) dense2 += t.ok && !t.diag && t.k == 2;
-        if (dtype == QSIM_C64 || n > kTileMinQubits || 4 * dense2 <= tg.size()) p->tiles = tile_groups(dtype, n, tg);
+        for (TileGroup& grp : tile_groups(dtype, n, tg)) {
+            if (grp.steps > 0 && !tile_pass_pays(dtype, n, grp, tg, p->ops, dev.num_sms)) {
+                for (int i : grp.members) {
+                    p->tiles.emplace_back();
+                    p->tiles.back().members = {i};
+                }
+            } else {
+                p->tiles.push_back(std::move(grp));
+            }
+        }
         bool any = false;
         for (const TileGroup& g : p->tiles) any = any || g.steps > 0;
         if (!any) p->tiles.clear();

@@ -1,0 +1,58 @@
+"""Per-gate plans of gates that touch little of the state: executed as a whole they are not slower than gate by gate.
+
+Bound: 1.4 times the gate-by-gate time of the same plan, medians of the same run (an estimate decides which of the two a group of
+gates takes, and was within a quarter of the measured times; a wrong choice costs 2 to 25 times)."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+C64, C128 = 0, 1
+
+
+@pytest.fixture(scope="module")
+def qsim(gpu_lib):
+    from paper_2511_14664_gb300 import qsim as q
+    return q
+
+
+def circuit(n, kind, gates):
+    rng = np.random.default_rng(n + gates)
+    c = W.Circuit(n)
+    for _ in range(gates):
+        q = [int(x) for x in rng.permutation(n)]
+        if kind == "cz":
+            c.append(W.Gate((q[0], q[1]), (), W.CZ(), "cz"))
+        elif kind == "p":
+            c.append(W.Gate((q[0],), (), np.diag([1.0, np.exp(1j * float(rng.uniform(0.1, 3)))]), "p"))
+        else:
+            c.append(W.Gate((q[0],), tuple(q[1:1 + int(kind)]), W.X(), "mcx"))
+    return c
+
+
+@pytest.mark.parametrize("dtype,n,kind,gates", [
+    (C64, 26, "8", 2), (C64, 26, "8", 20), (C64, 26, "3", 4), (C64, 26, "cz", 2), (C128, 24, "8", 2), (C128, 24, "8", 20),
+    (C128, 25, "3", 4), (C128, 25, "cz", 20), (C128, 25, "p", 20), (C128, 17, "3", 4)])
+def test_not_slower_than_gate_by_gate(qsim, dtype, n, kind, gates):
+    import torch
+    c = circuit(n, kind, gates)
+    st = qsim.State(n, dtype)
+    st.set_basis(0)
+
+    def median(p):
+        times = []
+        for _ in range(13):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(3):
+                p.execute(st)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times[3:])[5]
+
+    whole, single = qsim.Plan(c, dtype, mode=0), qsim.Plan(c, dtype, mode=0, launch_per_pass=True)
+    assert median(whole) <= 1.4 * median(single)
