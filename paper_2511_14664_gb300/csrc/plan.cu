@@ -1521,6 +1521,11 @@ int qsim_run(qsim_h h, const qsim_circuit* c, const qsim_run_opts* opts, qsim_pl
     qsim_run_opts o{};
     if (opts) o = *opts;
     o.use_graph = 0;
+    // The call waits for its work and then gives the plan's buffer and the sources of its uploads back: nothing that a
+    // graph could replay.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess) cudaGetLastError();
+    else if (capture != cudaStreamCaptureStatusNone) return cuda_fail(cudaErrorStreamCaptureUnsupported, "qsim_run");
     qsim_plan_h p = nullptr;
     int rc = plan_create(c, h->dtype, &o, h->stream, false, &p, info);
     if (rc) return rc;
