@@ -394,7 +394,7 @@ int qsim_expect_z(qsim_h h, double* zi, double* zz) {
 // With zi (and zz): the <Z> statistics first, whose segment sums the sampler then uses; one synchronisation for both.
 static int sample_common(qsim_h h, int64_t shots, uint64_t* out, const double* u_host, uint64_t seed, double* zi = nullptr,
                          double* zz = nullptr) {
-    if (!out && shots > 0) { set_error("NULL output"); return QSIM_EINVAL; }
+    if (!out) { set_error("NULL output"); return QSIM_EINVAL; }
     if (shots < 0 || shots > (1ll << 31)) { set_error("shots outside 0..2^31"); return QSIM_EINVAL; }
     if (shots == 0 && !zi) return QSIM_OK;
     if ((size_t)shots > h->samples_cap) {
@@ -438,7 +438,7 @@ int qsim_sample(qsim_h h, uint64_t seed, int64_t shots, uint64_t* out) {
 
 int qsim_expect_z_and_sample(qsim_h h, double* zi, double* zz, uint64_t seed, int64_t shots, uint64_t* out) {
     QSIM_CHECK_HANDLE(h);
-    if (!zi || (!zz && h->n > 1) || (!out && shots > 0)) { set_error("NULL output"); return QSIM_EINVAL; }
+    if (!zi || (!zz && h->n > 1) || !out) { set_error("NULL output"); return QSIM_EINVAL; }
     if (shots < 0 || shots > (1ll << 31)) { set_error("shots outside 0..2^31"); return QSIM_EINVAL; }
     double zz_dummy[1];
     return sample_common(h, shots, out, nullptr, seed, zi, zz ? zz : zz_dummy);

@@ -37,3 +37,19 @@ def test_one_shot_run_is_refused_under_capture(qsim, n, kw):
     st.set_basis(0)
     st.run(c, **kw)
     assert float(np.max(np.abs(st.get_state() - oracle.run(c)))) <= 1e-5
+
+
+def test_sampling_needs_an_output(qsim):
+    """A NULL output is an invalid argument, whatever the number of shots."""
+    import ctypes
+    L, st = qsim.lib(), qsim.State(5, qsim.C64)
+    st.set_basis(3)
+    z = (ctypes.c_double * 5)()
+    u = (ctypes.c_double * 1)(0.5)
+    for shots in (0, 1):
+        assert L.qsim_sample(st.h, 1, shots, None) == 1          # QSIM_EINVAL
+        assert L.qsim_sample_uniforms(st.h, u, shots, None) == 1
+        assert L.qsim_expect_z_and_sample(st.h, z, z, 1, shots, None) == 1
+    out = (ctypes.c_uint64 * 1)()
+    assert L.qsim_sample(st.h, 1, 0, out) == 0
+    assert L.qsim_expect_z_and_sample(st.h, z, z, 1, 1, out) == 0 and out[0] == 3
