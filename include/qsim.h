@@ -104,7 +104,8 @@ typedef struct {
 /* Options for planning a circuit. Zero-initialise, then set fields. */
 typedef struct {
     int32_t mode;       /* QSIM_RUN_PLAIN or QSIM_RUN_FUSED */
-    int32_t max_fused;  /* fusion width k for QSIM_RUN_FUSED: 1..6 (0 = 5); 7 with QSIM_PREC_FP16X3 on a
+    int32_t max_fused;  /* fusion width k for QSIM_RUN_FUSED, at most: 1..6 (0 = 5; 6 gives blocks of 5 in the
+                           state's own precision from 17 qubits on); 7 with QSIM_PREC_FP16X3 on a
                            complex64 state (7-qubit tensor-core blocks; plans of < 14 qubits or with global
                            qubits keep 6); dry runs also 7, 8 at any precision (pass counts) */
     int32_t precision;  /* QSIM_PREC_* for dense blocks of >= tc_min_k qubits (complex64 states only) */

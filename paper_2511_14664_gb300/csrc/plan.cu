@@ -687,8 +687,8 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     // composed blocks in the state's own precision on the tensor cores (k_tcx.cu): up to 5 qubits, so wider
     // groupings, which would run on CUDA cores, stay at 5
     const bool own_prec = dtype == QSIM_C128 || opts.precision == QSIM_PREC_SIMT;
-    const bool tcx_ok = !dry && opts.mode == QSIM_RUN_FUSED && own_prec && n >= kTcxMinQubits;
-    if (tcx_ok && kmax == 6) kmax = 5;
+    const bool tcx_plan = opts.mode == QSIM_RUN_FUSED && own_prec && n >= kTcxMinQubits, tcx_ok = tcx_plan && !dry;
+    if (tcx_plan && kmax == 6) kmax = 5;  // (a dry run of 7 or 8 sizes the fusion width: no plan that runs has that)
     const bool tc7 = kmax == 7 && opts.precision == QSIM_PREC_FP16X3 && dtype == QSIM_C64 && n >= 14;
     // 7-qubit blocks keep off qubits 0..2: on those the 7-qubit kernel moves partly used lines (4.0-5.5 ms at 30
     // qubits against 2.9-3.2 ms above them), while 6-qubit blocks there have the line-group and pair-rows paths
