@@ -53,10 +53,9 @@ constexpr int kThreads = 256;
 constexpr int kKmax = 4;
 constexpr int kSmallMax = 13;  // largest width kept in shared memory (2^13 x 8 B = 64 KiB)
 constexpr size_t kWideStreams = 8;  // worker streams for the circuits run as tensor-core plans
-// Circuits of at least this many qubits run as plans of 5-qubit blocks in their own precision (k_tcx.cu) where no
-// tensor-core precision takes them. 16-step chains, one / nine / forty of a width, in clusters of the persistent launch
-// and as plans: 18 qubits 0.47 / 0.76 / 2.24 ms and 0.21 / 0.69 / 2.34; 19 qubits 0.99 / 1.67 / 4.97 and 0.23 / 1.04 /
-// 3.70; one of 24 qubits 33.7 and 2.57. 64 chains of 10 to 24 qubits: 75 and 26 ms.
+// Circuits of at least this many qubits may run as plans of 5-qubit blocks in their own precision (k_tcx.cu) where no
+// tensor-core precision takes them; own_width has the rule. (16-step chains of 18 qubits, one / nine / forty: in clusters of
+// the persistent launch 0.47 / 0.76 / 2.24 ms, as plans 0.21 / 0.69 / 2.34.)
 constexpr int kOwnPlanMinN = 19;
 constexpr int kHalfGridBelow = 25;     // wide circuits narrower than this run their plans on half the SMs,
 constexpr int kQuarterGridBelow = 23;  // and narrower than this on a quarter of them
@@ -433,6 +432,64 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(const __grid_constant__ A
 }
 
 // ---- host side ----------------------------------------------------------------------------------------------
+// A circuit that may run as a plan of its own: its passes in a cluster (blocks of kKmax qubits) and as a plan (of 5).
+struct Choice { int n = 0, gates = 0, cluster = 0, own = 0; };
+
+// The width from which circuits run as plans of their own (QSIM_MAX_QUBITS + 1: none). Estimates in microseconds a pass at
+// 19, 20 and 21 qubits, from 1 to 40 circuits of one width (TFIM chains, brickwork, random circuits, random pairs): a plan 11.5,
+// 15, 20.5, among others 4.7, 7.3, 12.5; a cluster 23, 42, 82, beside others 40, 71, 143, but no less than 3, 5.6, 11.2 for each
+// circuit. A plan's passes and the tensor-core plans beside take their time from the clusters and one another. Plans where
+// they save 2 %: one or four circuits run 1.2 to 7 times as fast; forty of 19 qubits are level (4.6 against 5.0 ms chains, 2.7
+// against 2.8 brickwork, 3.2 against 2.0 random circuits of 10 gates a qubit) and stay in clusters where the passes say so;
+// 64 chains of 10 to 24 qubits 75 -> 46 ms. Where the tensor-core plans outlast the clusters these are hidden and stay
+// (256 chains of 10 to 24 qubits, FP16X3: 42.7 ms, 44.6 with the 19-qubit ones as plans).
+int own_width(const std::vector<Choice>& c, const qsim_circuit* cs, const std::vector<char>& tensor, int first) {
+    constexpr int kNone = QSIM_MAX_QUBITS + 1;
+    auto at = [](int n, double a, double b, double d) { return n <= 19 ? a : n == 20 ? b : std::ldexp(d, n - 21); };
+    double gates = 0.0, passes = 0.0, beside = 0.0;
+    int few[QSIM_MAX_QUBITS + 1] = {0}, count = 0;
+    for (const Choice& x : c) {
+        if (x.n == 0) continue;
+        gates += x.gates;
+        passes += x.own;
+        ++few[x.n];
+        ++count;
+    }
+    if (count == 0) return kNone;
+    const double per_gate = gates > 0.0 ? 0.8 * passes / gates : 0.0;  // a tensor-core plan's passes, in wider blocks
+    for (size_t i = 0; i < c.size(); ++i)
+        if (tensor[i]) beside += per_gate * cs[i].num_gates * (3.0 + std::ldexp(16.0, cs[i].n) / 4.6e6);
+    double best = 0.0, none = 0.0, clusters = 0.0;
+    int width = kNone;
+    for (int m = kNone; m >= first; --m) {
+        if (m < kNone && few[m] == 0) continue;
+        double sum = beside, longest = 0.0, cluster = 0.0;
+        int in_clusters = 0;
+        for (const Choice& x : c) in_clusters += x.n > 0 && x.n < m;
+        for (const Choice& x : c) {
+            if (x.n == 0) continue;
+            if (x.n >= m) {
+                const double one = x.own * at(x.n, 11.5, 15.0, 20.5);
+                if (one > longest) longest = one;
+                sum += x.own * at(x.n, 4.7, 7.3, 12.5);
+            } else {
+                const double one = x.cluster * (in_clusters > 1 ? at(x.n, 40.0, 71.0, 143.0) : at(x.n, 23.0, 42.0, 82.0));
+                if (one > cluster) cluster = one;
+                sum += x.cluster * at(x.n, 3.0, 5.6, 11.2);
+            }
+        }
+        const double t = std::max(std::max(longest, cluster), sum);
+        if (m == kNone) {
+            none = best = t;
+            clusters = std::max(cluster, sum - beside);
+        } else if (t < best && t < 0.98 * none) {
+            best = t;
+            width = m;
+        }
+    }
+    return beside > clusters ? kNone : width;
+}
+
 std::mutex g_tune_mu;
 int g_tuned_k[QSIM_MAX_QUBITS + 1] = {0};
 int g_tuned_tc_min_n[5] = {0, 0, 0, 0, 0};  // per tensor-core precision; 0 = not tuned (default 20)
@@ -675,25 +732,10 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
     batch::tune_cache_autoload();
     const int tc_min_n = opts.precision == QSIM_PREC_SIMT ? QSIM_MAX_QUBITS + 1
                          : (opts.batch_tc_min_n > 0 ? std::max(13, opts.batch_tc_min_n) : batch::tuned_tc_min_n(opts.precision));
-    // others this wide run as plans in the state's own precision, unless a fusion width is asked for
-    int own_min_n = opts.max_fused == 0 ? batch::kOwnPlanMinN : QSIM_MAX_QUBITS + 1;
-    // With enough tensor-core circuits beside it the persistent launch is hidden, and plans of its circuits would only
-    // take SMs from theirs (256 chains of 10 to 24 qubits, FP16X3: 42.7 ms with the 19-qubit ones in clusters, 44.6 as
-    // plans; 29 of 11 to 21 qubits: 1.15 and 0.71 ms). Estimates in microseconds: 40 gates a tensor-core pass at 4.6 TB/s;
-    // 12 gates a cluster's pass of 20 us at 19 qubits, nine clusters.
-    double beside = 0.0, longest = 0.0, all = 0.0;
-    for (int ci = 0; ci < count; ++ci) {
-        const double g = (double)cs[ci].num_gates;
-        if (cs[ci].n >= tc_min_n) beside += g / 40.0 * std::ldexp(16.0, cs[ci].n) / 4.6e6;
-        else if (cs[ci].n >= own_min_n) {
-            const double us = g / 12.0 * std::ldexp(20.0, cs[ci].n - 19);
-            longest = std::max(longest, us);
-            all += us;
-        }
-    }
-    if (beside > std::max(longest, all / 9.0)) own_min_n = QSIM_MAX_QUBITS + 1;
+    // others this wide may run as plans in the state's own precision, unless a fusion width is asked for (own_width)
+    const int own_min_n = opts.max_fused == 0 ? batch::kOwnPlanMinN : QSIM_MAX_QUBITS + 1;
     std::vector<char> wide(count, 0);
-    for (int ci = 0; ci < count; ++ci) wide[ci] = cs[ci].n >= std::min(tc_min_n, own_min_n);
+    for (int ci = 0; ci < count; ++ci) wide[ci] = cs[ci].n >= tc_min_n;
 
     // ---- plan every circuit ---------------------------------------------------------------------------
     std::vector<ComposeBlock> cblocks;
@@ -709,6 +751,7 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
     if (cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); device = 0; }
     std::vector<std::vector<uint64_t>> gmasks(count);
     std::vector<std::vector<std::vector<int>>> cblk(count);
+    std::vector<batch::Choice> choice(count);
     rc = parallel_for(count, host_threads(count), device, [&](int ci, int) -> int {
         const qsim_circuit& c = cs[ci];
         const int n = c.n;
@@ -735,10 +778,22 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
                 cblk[ci] = group_gates(gmask, gdiag, n, kmax);
                 group_cache_put(key, cblk[ci]);
             }
+            if (n >= own_min_n) {
+                key[2] = 5;  // (the passes of a plan of its own, nearly)
+                std::vector<std::vector<int>> five;
+                if (!group_cache_get(key, five)) {
+                    five = group_gates(gmask, gdiag, n, 5);
+                    group_cache_put(key, five);
+                }
+                choice[ci] = {n, c.num_gates, (int)(kmax == batch::kKmax ? cblk[ci].size() : group_gates(gmask, gdiag, n, batch::kKmax).size()),
+                              (int)five.size()};
+            }
         }
         return QSIM_OK;
     });
     if (rc) return rc;
+    const int own_width = batch::own_width(choice, cs, wide, own_min_n);
+    for (int ci = 0; ci < count; ++ci) wide[ci] = wide[ci] || cs[ci].n >= own_width;
     for (int ci = 0; ci < count; ++ci) {
         const qsim_circuit& c = cs[ci];
         const int n = c.n;
