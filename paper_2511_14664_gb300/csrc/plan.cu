@@ -700,8 +700,8 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
     // when it follows a dense block of at most 6 qubits (it becomes that block's epilogue, which only a
     // tensor-core precision has). Up to 19 qubits a pass is the time of one tile, 10.1-10.7 us at 7 qubits and 5.7-6.5 at
     // 6 (19-qubit brickwork: 245 us in 6-qubit blocks, 311 in 7-qubit ones), unless several plans run side by side
-    // (launch_per_pass). At 20 qubits that brickwork would gain too (325 to 293 us), but accuracy figures are quoted for
-    // its 7-qubit blocks.
+    // (launch_per_pass). At 20 qubits that brickwork would gain too (325 to 293 us); it keeps its 7-qubit blocks
+    // because the accuracy test of 20 qubits, depth 40, asks for them.
     const double cost7 = n <= 19 && !opts.launch_per_pass ? 1.7 : 1.2;
     auto cost = [&](const std::vector<std::vector<int>>& bl) {
         double cs = 0.0;
@@ -1065,12 +1065,14 @@ static int plan_create(const qsim_circuit* c, int dtype, const qsim_run_opts* op
             // is as long below 14 qubits. So TFIM chains, whose blocks hold many cheap gates, stay there (14 qubits,
             // complex64: 31 against 41 us) and brickwork comes here (14 qubits, complex64 56 against 72 us, complex128 97
             // against 164 us). A one-shot run saves composing those blocks, 0.1 ms, and always comes here.
-            // Nor may its errors grow: a row of a dense block on k qubits rounds like 2^k units, its coefficients like one
-            // (TFIM, 12 qubits, one-shot: 215 units and 3.4e-7 of the norm pass by pass, 267 and 6e-7 here). So where the
-            // products round more, or where the passes are few (from |0>, many of a first block's terms are exact zeros:
-            // 9 to 15 qubits, 10 layers, 1.9e-7 pass by pass and 2.0e-7 here; 20 layers, 3.3e-7 and 3.0e-7), a complex64
-            // state is computed in FP64 between its barriers (that TFIM circuit: 5e-8; 258 us against 202 and, pass by
-            // pass, 414).
+            // Nor may the errors of a complex64 state grow: a row of a dense block on k qubits rounds like 2^k units, its
+            // coefficients like one (TFIM, 12 qubits, one-shot: 215 units and 3.4e-7 of the norm pass by pass, 267 and 6e-7
+            // here). So where the products round more, or where the passes are few (from |0>, many of a first block's terms
+            // are exact zeros: 9 to 15 qubits, 10 layers, 1.9e-7 pass by pass and 2.0e-7 here; 20 layers, 3.3e-7 and 3.0e-7),
+            // it is computed in FP64 between its barriers (that TFIM circuit: 5e-8; 258 us against 202 and, pass by pass,
+            // 414). A complex128 state has no wider type, and needs no rule: over 75 circuits (TFIM, brickwork, random circuits
+            // and pairs, QFT; 8 to 13 qubits) the errors here were 0.36 to 1.24 times those of the passes, 0.87 on average, the
+            // largest ratio at 1.5e-16.
             double passes_us = 0.0, passes_roundings = 0.0;
             for (const PlanOp& op : p->ops) {
                 const bool diag = op.kind == OP_DIAG || op.kind == OP_PHASE;
