@@ -26,14 +26,16 @@
 // three as zero). So the slices take a row only where every result y_i has sum_c |U_ic| |x_c| above 2^-9 of that power of
 // two, which bounds its error by 2^-16 (2^-43) of that sum, beside 2^-18 (2^-47) for a chain of 64 FMAs: rows whose amplitudes
 // lie within kRange = 8 binades of the largest (the entries of a row of U sum to 1 or more), and rows in which every row
-// of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4. The others (0.1 % of the rows of a
-// random state) are chains of FMAs in the state's precision (rows_by_fma): a few of a quadrant's 32 rows by three
-// warps beside the MMA issuer, many by the output. So are rows outside the exponents that the slices take; amplitudes
-// that the block joins with an infinity or NaN become NaN. One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0:
-// 276, 351 / 242, 261 us, and without this 254, 309 / 201, 239; with amplitudes over 30 binades 850 / 800 (CUDA cores 461 / 3457);
-// 16-step TFIM chains of small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 10.2 / 4.0 -> 10.2 ms. Left: all rows by the
-// three warps (11.6 / 14.9 ms there, and no faster elsewhere); one warp that decides for all rows (2.7 ms a pass at wide rows);
-// kRange = 7 (284 us in complex64).
+// of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4 (the input warps look at U
+// for 0.1 % of the rows of a random state, and few of those fail). The others are sums of FMAs in the state's precision, by
+// the output (rows_by_fma). So are rows outside the exponents that the slices take; amplitudes that the block joins with an
+// infinity or NaN become NaN.
+// One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0: 275, 340 / 240, 273 us, and
+// without this 254, 309 / 201, 239; with amplitudes over 30 binades 510 / 710 (CUDA cores 461 / 3457). 16-step TFIM chains of
+// small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 9.5 / 4.0 -> 10.2 ms. Measured and left: such rows by three
+// more warps, a few of a quadrant or all of them (351 us from qubit 0 in complex64, 850 us at 30 binades); one warp that
+// decides for all rows (2.7 ms at 30 binades); rows given away unseen where a quadrant has few (301 us); ROWS = 4 (590 us at
+// 30 binades).
 //
 // Layout. A tile is 128 rows (the 7 lowest index bits outside the block) by 32 columns; blocks of fewer qubits
 // take idle qubits as further columns (U x I). Digit plane s of a tile is a K-major operand of 128 x 64 FP16
@@ -43,13 +45,13 @@
 // the reads of A from shared memory would bound it).
 //
 // Roles, one CTA per SM: input warps load a tile, convert it and write its planes; one warp issues the MMAs;
-// output warps sum the positions, convert back and store; three more take rows by FMAs. In complex64 (16 input, 8 output warps) planes and
+// output warps sum the positions, convert back and store, and take rows by FMAs. In complex64 (16 input, 8 output warps) planes and
 // accumulators are double-buffered, and the next tile's loads are in flight in registers. In complex128 the 8
 // positions take all of tensor memory and the planes half of shared memory, so a tile's MMAs commit in four
 // groups of planes: as a group retires, the input (8 warps) writes the next tile's planes over it and the output
 // (16 warps) adds the positions it finished.
-// Bound: complex64 (26 qubits, 276 us, 0.57 of the copy rate) the input's loads and conversion; complex128 (24
-// qubits, 242 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
+// Bound: complex64 (26 qubits, 275 us, 0.57 of the copy rate) the input's loads and conversion; complex128 (24
+// qubits, 240 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
 // and on the integer pipe about as fast, so they are spread over both; the tensor cores work a quarter of the
 // time. Measured and left (against 190 us without the rows by FMAs): one set of warps for input and output (281 us at 24 qubits), 8 output warps (208),
 // the next tile staged by cp.async (204), L2 prefetch of the next tile (212), the D_d to integers by F2I (213).
@@ -80,13 +82,11 @@ template <> struct Cfg<float> {
     static constexpr int S = 4, ND = 4;        // digits; digit positions kept
     static constexpr int BUF = 2;              // tiles in flight: A planes and accumulators
     static constexpr int GROUPS = 1;           // commits per tile
-    static constexpr int IN = 16, OUT = 8, MMA = 4;  // warps: tile loads and digit planes; accumulators and stores; MMAs (one) and rows by FMAs
+    static constexpr int IN = 16, OUT = 8, MMA = 1;  // warps: tile loads and digit planes; accumulators and stores; MMAs
     static constexpr int kStepsU = 30;         // U in 2^-30 steps
     static constexpr int kRange = 8;           // binades below the row's largest amplitude that the slices take
-    static constexpr int ROWS = 4;             // rows an output warp takes at a time by FMAs
-    static constexpr int FEW = 8;              // fewer of a quadrant's 32 rows: left to the row warps
-    static constexpr int LOOK = FEW;           // so many: the input looks at U before it gives them away
-    static constexpr int U = D;                // rows of U in shared memory, for them
+    static constexpr int ROWS = 2;             // rows an output warp takes at a time by FMAs
+    static constexpr int U = D;                // columns of U in shared memory, for those rows
     __host__ __device__ static constexpr int group_end(int) { return S; }
 };
 template <> struct Cfg<double> {
@@ -94,30 +94,26 @@ template <> struct Cfg<double> {
     static constexpr int BUF = 1;
     static constexpr int GROUPS = 4;           // planes 0-1, 2-3, 4-5, 6
     // Whole warpgroups, so that registers can move between them: launched with 72 a thread (28 warps, 64512 in
-    // all), the input takes 96, the output keeps 64, the MMA warpgroup 56: 64512.
+    // all), the input takes 96, the output keeps 64, the MMA warpgroup (one warp works) 56: 64512.
     static constexpr int IN = 8, OUT = 16, MMA = 4;
     static constexpr int kRegIn = 96, kRegOut = 64, kRegMma = 56;
     static constexpr int kStepsU = 54;
     static constexpr int kRange = 8;
     static constexpr int ROWS = 1;
-    static constexpr int FEW = 4;
-    static constexpr int LOOK = 1;             // (one row by FMAs is 10 us of a 12 us pass at 19 qubits)
     static constexpr int U = 0;                // (stays in global memory: 16 KiB more would take L1 from the loads in flight)
     __host__ __device__ static constexpr int group_end(int g) { return g < 3 ? 2 * g + 2 : S; }
 };
 template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
-constexpr int kRowWarps = 3;
-constexpr int kQueue = 16;  // entries of a quadrant's queue of rows for the row warps
 template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
 template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
 template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 5; }
 // planes, column offsets, largest and smallest amplitudes of the input's rows [2][IN / 4][128] and which of them are large
-// [IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the row
-// warps' queues [4][kQueue][2] and how far their producers are [4], the large entries of U [32][2], U and the rows taken by FMAs [OUT][ROWS][32] [kRowWarps][32], alignment
-template <typename R> constexpr int smem_rows() { return (Cfg<R>::OUT * Cfg<R>::ROWS + kRowWarps + Cfg<R>::U) * D * 2 * (int)sizeof(R); }
+// [IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the large entries of U [32][2], U and
+// the rows taken by FMAs [OUT][ROWS][32], alignment
+template <typename R> constexpr int smem_rows() { return (Cfg<R>::OUT * Cfg<R>::ROWS + Cfg<R>::U) * D * 2 * (int)sizeof(R); }
 template <typename R> constexpr size_t smem_bytes() {
     return smem_planes<R>() + smem_rows<R>() + 16 * D + 4 * (3 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
-           8 * bars<R>() + 8 + 4 * (8 * kQueue + 4) + 1024;
+           8 * bars<R>() + 8 + 1024;
 }
 // With 1 KiB that the system takes, below the 196 KiB that leave 60 KiB of L1: the data of loads in flight lies there
 // (complex128, 24 qubits: 201 us a pass; with 28 KiB, 239).
@@ -313,20 +309,6 @@ __device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args&
         __syncwarp();  // xs has been read
     }
 }
-// Not inlined in complex64: inside the output's loop its registers cost the slices 6 % (complex128, whose warps have
-// registers of their own, inlines it: a function may use as many as the kernel was launched with).
-template <int NROW>
-__device__ __noinline__ void rows_by_fma_call(float2* psi, const Args& a, const float2* u, float2* xs, uint64_t col, uint32_t mine,
-                                              uint64_t at) {
-    rows_by_fma<float, NROW>(psi, a, u, xs, col, mine, at);
-}
-template <typename R, int NROW>
-__device__ __forceinline__ void rows_any(typename Amp<R>::T* psi, const Args& a, const typename Amp<R>::T* u, typename Amp<R>::T* xs,
-                                         uint64_t col, uint32_t mine, uint64_t at) {
-    if constexpr (sizeof(R) == 4) rows_by_fma_call<NROW>(psi, a, u, xs, col, mine, at);
-    else rows_by_fma<R, NROW>(psi, a, u, xs, col, mine, at);
-}
-
 template <typename R, int MODE>
 __global__ void __launch_bounds__(threads<R>(), 1)
 k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a, const uint4* __restrict__ bops,
@@ -346,17 +328,14 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     unsigned char* sA = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sB = sA + BUF * S * kPlaneA;
     T* sU = reinterpret_cast<T*>(sB + S * kPlaneB);                   // U by columns (complex64)
-    T* sX = sU + C::U * D;                                               // [kOut][ROWS][32], [kRowWarps][32]
-    uint64_t* sCol = reinterpret_cast<uint64_t*>(sX + (kOut * C::ROWS + kRowWarps) * D);
+    T* sX = sU + C::U * D;                                               // [kOut][ROWS][32]
+    uint64_t* sCol = reinterpret_cast<uint64_t*>(sX + kOut * C::ROWS * D);
     uint4* sL = reinterpret_cast<uint4*>(sCol + D);                   // [16]: of two rows of U each, large entries
     uint32_t* sE = reinterpret_cast<uint32_t*>(sL + D / 2);           // [2][kIn / 4][128]
     uint32_t* sBig = sE + 2 * (kIn / 4) * 128;                        // [kIn / 4][128]
     int* sRow = reinterpret_cast<int*>(sBig + (kIn / 4) * 128);       // [row_slots][128]
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sRow + row_slots<R>() * 128);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + bars<R>());
-    volatile uint32_t* const qmask = tslot + 2;           // [4][kQueue]: rows of a quadrant, 0 = free
-    volatile uint32_t* const qtile = qmask + 4 * kQueue;  // [4][kQueue]: their tile
-    volatile uint32_t* const qdone = qtile + 4 * kQueue;  // [4]: tiles whose rows are queued; all ones after the last
     constexpr uint32_t kAll = 0xFFFFFFFFu;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -367,8 +346,6 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     auto done = [&](uint32_t b, int g) { return smem_u32(mbar + (2 + g) * BUF + b); };
     const uint32_t bbar = smem_u32(mbar + BUF * (2 + GROUPS));
     auto rowbar = [&](int q) { return smem_u32(mbar + BUF * (2 + GROUPS) + 1 + q); };
-    for (int c = tid; c < 4 * kQueue; c += threads<R>()) qmask[c] = 0;
-    if (tid < 4) qdone[tid] = 0;
     for (int c = tid; c < D; c += threads<R>()) sCol[c] = deposit((uint64_t)c, a.tpos, K);
     if (tid == 0) {
         for (int j = 0; j < bars<R>(); ++j) {
@@ -407,7 +384,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 
     bool bad = false;
     if (warp >= kIn + kOut) {
-        // ---- MMA issuer, and three warps that take rows by FMAs ----
+        // ---- MMA issuer ----
         if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegMma));
         if (warp == kIn + kOut && lane == 0) {
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bbar), "r"(S * kPlaneB + (C::U > 0 ? (int)sizeof(T) << (2 * a.k) : 0))
@@ -463,48 +440,6 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                 if (issued) mbar_wait_bounded(done(buf(issued - 1), GROUPS - 1), par(issued - 1));  // the MMAs already issued
             }
         }
-        if (warp > kIn + kOut) {
-            // Row warps: the rows of quadrants that have a few of them, any time (in the output they would hold up a tile: in
-            // complex128 a row is 8192 cycles of the FP64 units beside a warp). Warp w has every third entry of the queues.
-            const int w = warp - (kIn + kOut + 1);
-            T* const xs = sX + (kOut * C::ROWS + w) * D;
-            const uint64_t col = sCol[lane];
-            bad = !wait(bbar, 0);  // U
-            uint64_t since = globaltimer();
-            uint32_t seen = 0;
-            while (!bad) {
-                const uint32_t done_tiles = lane < 4 ? qdone[lane] : kAll;
-                const bool last = __all_sync(0xffffffffu, done_tiles == kAll);
-                __threadfence_block();  // what was queued before that
-                bool found = false;
-#pragma unroll 1
-                for (int h = 0; h < 4 * kQueue; h += 32) {
-                    const uint32_t m = (h + lane) % kRowWarps == w ? qmask[h + lane] : 0u;
-                    for (uint32_t at = __ballot_sync(0xffffffffu, m != 0); at; at &= at - 1) {
-                        const int l = __ffs(at) - 1, slot = h + l, q = slot / kQueue;
-                        const uint32_t mine = __shfl_sync(0xffffffffu, m, l);
-                        __threadfence_block();
-                        const uint64_t row = insert_zeros(tile(qtile[slot]), a.spos, a.nS) + deposit((uint64_t)(32 * q + lane), a.rpos, kRowBits);
-                        rows_any<R, 1>(psi, a, C::U > 0 ? sU : umat, xs, col, mine, row);
-                        __threadfence_block();
-                        __syncwarp();
-                        if (lane == 0) qmask[slot] = 0;
-                        found = true;
-                    }
-                }
-                if (last && !found) break;
-                const uint32_t sum = __reduce_add_sync(0xffffffffu, done_tiles);
-                if (found || sum != seen) {
-                    seen = sum;
-                    since = globaltimer();
-                } else if (__any_sync(0xffffffffu, globaltimer() - since > 2000000000ull)) {
-                    bad = true;  // no producer has moved
-                } else {
-                    __nanosleep(500);
-                }
-            }
-            if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
-        }
         __syncwarp();
     } else if (warp < kIn) {
         // ---- input: load a tile, convert it to fixed point, write its digit planes ----
@@ -548,23 +483,6 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             asm volatile("" : "+r"(top), "+r"(low) :: "memory");  // before any later load is issued (loads share scoreboards)
             return (max(top >> EB, min(top, 1u)) << 16) | (0x7FFFu - (low >> EB));
         };
-        // Rows of the quadrant to the row warps' queue (by one warp of the quadrant). False if there was no room in 2 s.
-        uint32_t queued = 0;
-        auto queue_rows = [&](uint32_t rows, uint32_t i) -> bool {
-            const int slot = quad * kQueue + (int)(queued++ % kQueue);
-            bool ok = true;
-            if (lane == 0) {
-                const uint64_t since = globaltimer();
-                while (ok && qmask[slot] != 0) ok = globaltimer() - since <= 2000000000ull;
-                if (ok) {
-                    __threadfence_block();
-                    qtile[slot] = i;
-                    __threadfence_block();
-                    qmask[slot] = rows;
-                }
-            }
-            return __all_sync(0xffffffffu, ok);
-        };
         // The warps of the quadrant meet at an mbarrier, whose wait ends when one of them has given up (no warp waits at a
         // named barrier: it has no limit).
         uint32_t met = 0;
@@ -586,7 +504,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             const uint32_t E0 = e >> 16, low = 0x7FFFu - (e & 0xFFFFu), E = min(max(E0, kLowE<R>), kHighE<R>);
             bool by_fma = E0 != 0 && (E0 != E || E0 - low > (uint32_t)C::kRange);
             uint32_t rows = __ballot_sync(0xffffffffu, by_fma);  // (the same in all warps of the quadrant)
-            if (__popc(rows) >= C::LOOK) {
+            if (rows) {
                 // its columns within 1 and within 4 binades of the largest; has every row of U an entry of 2^-7, or of 2^-4, there?
                 uint32_t big = 0;
 #pragma unroll
@@ -614,11 +532,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             }
             // read by the output warps after this tile's MMAs. The planes of tile i - 1 were stored, so the MMAs of
             // tile i - 1 - BUF have run, for which tile i - 1 - 2 BUF had been read: 2 BUF + 1 slots or more will do
-            if (warp < 4) {
-                sRow[i % row_slots<R>() * 128 + r] = by_fma ? kByFma : (int)E;
-                if (rows && __popc(rows) < C::FEW && !queue_rows(rows, i)) return false;
-                if (lane == 0) qdone[quad] = i + 1;
-            }
+            if (warp < 4) sRow[i % row_slots<R>() * 128 + r] = by_fma ? kByFma : (int)E;
             planes = rows != kAll;
             if (!planes) return true;
             if constexpr (DBL) {
@@ -688,9 +602,6 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             }
         }
         if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
-        __threadfence_block();
-        __syncwarp();
-        if (warp < 4 && lane == 0) qdone[quad] = kAll;  // the row warps may leave
     } else {
         // ---- output: sum the digit positions, convert back, store ----
         if constexpr (DBL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Cfg<double>::kRegOut));
@@ -705,17 +616,17 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             __syncwarp();
             if (lane == 0) mbar_arrive(freed(buf(i)));
         };
-        // The output's own rows: of quadrants that have many, shared out among the quadrant's warps.
+        // The rows of the quadrant that the slices do not take, shared out among its warps.
         bool have_u = false;
         auto quad_rows = [&](uint32_t mask, uint64_t at) -> bool {
-            if (__popc(mask) < C::FEW) return true;
+            if (mask == 0) return true;
             if (!have_u && !wait(bbar, 0)) return false;
             have_u = true;
             uint32_t mine = 0;
             int rank = 0;
             for (; mask; mask &= mask - 1, ++rank)
                 if (rank / C::ROWS % (kOut / 4) == ((warp - kIn) >> 2)) mine |= mask & (0u - mask);
-            rows_any<R, C::ROWS>(psi, a, C::U > 0 ? sU : umat, sX + (warp - kIn) * (C::ROWS * D), sCol[lane], mine, at);
+            rows_by_fma<R, C::ROWS>(psi, a, C::U > 0 ? sU : umat, sX + (warp - kIn) * (C::ROWS * D), sCol[lane], mine, at);
             return true;
         };
         for (uint32_t i = 0; i < m; ++i) {
