@@ -16,8 +16,9 @@
 // launch: one cluster streams a state at a fraction of the GPU's bandwidth (about 0.44 TB/s for a 16-CTA
 // cluster on a 24-qubit state, where the whole GPU does 6.5), so each becomes a fused tensor-core plan
 // (6-qubit blocks, or up to 7 with FP16X3), its first block generating |0>, its <Z> values reduced on the device
-// into the same output arrays. So do, as plans of 5-qubit blocks in their own precision, the other circuits of
-// at least kOwnPlanMinN qubits, unless the caller asks for a fusion width or the tensor-core plans hide them. These plans run on eight worker streams forked from the caller's stream before the
+// into the same output arrays. So do, as plans of 5-qubit blocks in their own precision, other circuits of at least
+// kOwnPlanMinN qubits where that is estimated faster and no fusion width is asked for (own_width). These plans run on
+// eight worker streams forked from the caller's stream before the
 // persistent launch and joined back after it: their kernels take the SMs that launch leaves (64 chains of 10 to 24
 // qubits: 12.9 ms with the plans after the launch, 11.5 ms beside it), and one circuit's pipeline fill and drain
 // overlap another's passes (the narrower circuits' kernels on a half or a quarter of the SMs, side by side). States
@@ -437,12 +438,14 @@ struct Choice { int n = 0, gates = 0, cluster = 0, own = 0; };
 
 // The width from which circuits run as plans of their own (QSIM_MAX_QUBITS + 1: none). Estimates in microseconds a pass at
 // 19, 20 and 21 qubits, from 1 to 40 circuits of one width (TFIM chains, brickwork, random circuits, random pairs): a plan 11.5,
-// 15, 20.5, among others 4.7, 7.3, 12.5; a cluster 23, 42, 82, beside others 40, 71, 143, but no less than 3, 5.6, 11.2 for each
-// circuit. A plan's passes and the tensor-core plans beside take their time from the clusters and one another. Plans where
-// they save 2 %: one or four circuits run 1.2 to 7 times as fast; forty of 19 qubits are level (4.6 against 5.0 ms chains, 2.7
-// against 2.8 brickwork, 3.2 against 2.0 random circuits of 10 gates a qubit) and stay in clusters where the passes say so;
-// 64 chains of 10 to 24 qubits 75 -> 46 ms. Where the tensor-core plans outlast the clusters these are hidden and stay
-// (256 chains of 10 to 24 qubits, FP16X3: 42.7 ms, 44.6 with the 19-qubit ones as plans).
+// 15, 20.5, among others 4.7, 7.3, 12.5 (measured 3.7 to 6, 6 to 10, 11 to 17: more where more rows go by FMAs); a cluster 23,
+// 42, 82, beside others 40, 71, 143, but no less than 3, 5.6, 11.2 for each circuit. A plan's passes and the tensor-core
+// plans beside take their time from the clusters and one another. Plans where they save 2 %.
+// Measured, clusters / as chosen (ms): one chain of 19, 20, 21 qubits 1.00 / 0.31, 1.79 / 0.44, 3.96 / 0.63; forty 5.0 / 4.1, 9.6 /
+// 7.5, 21.9 / 13.6; forty of 19 qubits stay, brickwork 2.8 (as plans 2.7), random circuits 1.9 (3.2), random pairs 2.2 (2.8);
+// forty random circuits of 20 qubits and 10 gates a qubit, whose rows the estimate does not see, 4.0 / 5.1; 64 chains of 10 to 24
+// qubits 75 / 36. Where the tensor-core plans outlast the clusters these are hidden and stay (256 chains of 10 to 24 qubits,
+// FP16X3: 42.7, and 44.6 with the 19-qubit ones as plans).
 int own_width(const std::vector<Choice>& c, const qsim_circuit* cs, const std::vector<char>& tensor, int first) {
     constexpr int kNone = QSIM_MAX_QUBITS + 1;
     auto at = [](int n, double a, double b, double d) { return n <= 19 ? a : n == 20 ? b : std::ldexp(d, n - 21); };

@@ -18,9 +18,9 @@
 // parameter.
 //
 // The lowest bits of the index (3 in complex64, 2 in complex128) always belong to the tile: 64-byte runs.
-// Bound: instruction issue in complex64 (24 qubits, 720 random-circuit gates: 3.1 ms; per gate and thread 64 FMAs or
+// Bound: instruction issue in complex64 (24 qubits, 720 random-circuit gates: 2.9 ms; per gate and thread 64 FMAs or
 // fewer and about 45 other instructions), FP64 in complex128. Measured and left: every thread decoding the program
-// from shared memory (4.1 ms) or from the parameter (3.9 ms).
+// from shared memory (4.1 ms, against 3.1 at the time) or from the parameter (3.9 ms).
 #include <algorithm>
 #include <cstring>
 
