@@ -27,9 +27,12 @@
 // two, which bounds its error by 2^-16 (2^-43) of that sum, beside 2^-18 (2^-47) for a chain of 64 FMAs: rows whose amplitudes
 // lie within kRange = 8 binades of the largest (the entries of a row of U sum to 1 or more), and rows in which every row
 // of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4 (the input warps look at U
-// for 0.1 % of the rows of a random state, and few of those fail). The others are sums of FMAs in the state's precision, by
-// the output (rows_by_fma). So are rows outside the exponents that the slices take; amplitudes that the block joins with an
-// infinity or NaN become NaN.
+// for 0.1 % of the rows of a random state, and few of those fail). The others go by FMAs in the state's precision, by the
+// output (rows_by_fma): in complex128 the whole row; in complex64, where 64 FMAs lose more than the slices, the results more
+// than kLarge = 4 binades below the row's largest amplitude (with whole rows by FMAs the norm of the error of 12 circuits,
+// sparse and structured ones among them, was 1.19 times that of the slices alone, at worst 1.56; so it is 0.98, 1.03). Rows
+// outside the exponents that the slices take go by FMAs as well; amplitudes that the block joins with an infinity or NaN
+// become NaN.
 // One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0: 275, 340 / 240, 273 us, and
 // without this 254, 309 / 201, 239; with amplitudes over 30 binades 510 / 710 (CUDA cores 461 / 3457). 16-step TFIM chains of
 // small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 9.5 / 4.0 -> 10.2 ms. Measured and left: such rows by three
@@ -106,7 +109,7 @@ template <> struct Cfg<double> {
 template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 8; }  // tiles whose row exponents are kept
 template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
 template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
-template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 5; }
+template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 9; }
 // planes, column offsets, largest and smallest amplitudes of the input's rows [2][IN / 4][128] and which of them are large
 // [IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the large entries of U [32][2], U and
 // the rows taken by FMAs [OUT][ROWS][32], alignment
@@ -172,7 +175,9 @@ template <int N> __device__ __forceinline__ void st_words(void* p, const uint32_
 // adds 1076 - E to exponents) they do not overflow.
 template <typename R> constexpr uint32_t kLowE = sizeof(R) == 8 ? 64 : 32;
 template <typename R> constexpr uint32_t kHighE = sizeof(R) == 8 ? 1076 : 247;
-constexpr int kByFma = 1 << 20;  // in place of a row's exponent: the output takes the row by FMAs
+// Beside a row's exponent: its small results come from FMAs (complex64; complex128: all), all of them.
+constexpr int kByFma = 1 << 20, kAllFma = 1 << 21, kExponent = 0xFFFF;
+constexpr int kLarge = 4;  // results within so many binades of the row's largest amplitude come from the slices all the same
 
 // The fixed-point value of a real whose row has largest biased exponent E, plus 128 in every base-256 digit
 // (so that the bytes of the result are the digits plus 128). |x| < 2^(E - 1022) maps to 2^54 steps. Two ways that
@@ -217,10 +222,9 @@ __device__ __forceinline__ float fmar(float x, float y, float z) { return __fmaf
 __device__ __forceinline__ double fmar(double x, double y, double z) { return __fma_rn(x, y, z); }
 
 // The rows in `mine` of 32 (`at`: the index of the lane's row) in the state's own arithmetic: sums of FMA chains over
-// eight columns each (a chain over all 32, as in the CUDA-core blocks, has 1.7 times the error: 4.8 units of 2^-24 of the
-// state's largest amplitude at 21 qubits), without the columns that are zero in every row. Nobody else stores these
-// rows. A warp takes whole rows, NROW at a time, so that it has read a row before it is written; a lane is a column of
-// the result, `col` its index bits; xs: room for NROW rows; u: U by columns.
+// eight columns each, without the columns that are zero in every row. A warp takes whole rows, NROW at a time, so that it
+// has read a row before it is written; a lane is a column of the result, `col` its index bits; xs: room for NROW rows; u: U
+// by columns.
 template <typename R, int NROW>
 __device__ __forceinline__ void rows_by_fma(typename Amp<R>::T* psi, const Args& a, const typename Amp<R>::T* u, typename Amp<R>::T* xs,
                                             uint64_t col, uint32_t mine, uint64_t at) {
@@ -340,16 +344,18 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // barriers: per buffer, A stored (full), accumulators read (freed), MMAs of a plane group retired (done); the
-    // operand loaded (bbar); per quadrant of 32 rows, the row exponents of its input warps written (rowbar)
+    // operand loaded (bbar); per quadrant of 32 rows, the row exponents of its input warps written (rowbar), rows by FMAs
+    // stored (fmabar)
     auto full = [&](uint32_t b) { return smem_u32(mbar + b); };
     auto freed = [&](uint32_t b) { return smem_u32(mbar + BUF + b); };
     auto done = [&](uint32_t b, int g) { return smem_u32(mbar + (2 + g) * BUF + b); };
     const uint32_t bbar = smem_u32(mbar + BUF * (2 + GROUPS));
     auto rowbar = [&](int q) { return smem_u32(mbar + BUF * (2 + GROUPS) + 1 + q); };
+    [[maybe_unused]] auto fmabar = [&](int q) { return smem_u32(mbar + BUF * (2 + GROUPS) + 5 + q); };
     for (int c = tid; c < D; c += threads<R>()) sCol[c] = deposit((uint64_t)c, a.tpos, K);
     if (tid == 0) {
         for (int j = 0; j < bars<R>(); ++j) {
-            const int count = j < BUF ? kIn : (j < 2 * BUF ? kOut : (j <= BUF * (2 + GROUPS) ? 1 : kIn / 4));
+            const int count = j < BUF ? kIn : (j < 2 * BUF ? kOut : (j <= BUF * (2 + GROUPS) ? 1 : (j < BUF * (2 + GROUPS) + 5 ? kIn / 4 : kOut / 4)));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar + j)), "r"(count) : "memory");
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -491,10 +497,9 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             if (lane == 0) mbar_arrive(rowbar(quad));
             return wait(rowbar(quad), met++ & 1);
         };
-        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow, or kByFma
-        // for a row that the slices do not take: one with amplitudes more than kRange binades below its largest, unless
-        // every row of U has a large entry at a large amplitude. False if a wait ran out. `planes` is false where no row of
-        // the warp needs its digits.
+        // In place: the thread's reals to fixed point relative to the row's largest exponent, which goes to sRow, with kByFma
+        // for a row of amplitudes more than kRange binades below its largest, unless every row of U has a large entry at a
+        // large amplitude. False if a wait ran out. `planes` is false where no row of the warp needs its digits.
         auto convert = [&](uint32_t (&X)[W], uint32_t i, uint32_t e, bool& planes) -> bool {
             uint32_t* const ex = sE + (i & 1) * (kIn / 4 * 128) + r;
             ex[(warp >> 2) * 128] = e;
@@ -532,8 +537,8 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             }
             // read by the output warps after this tile's MMAs. The planes of tile i - 1 were stored, so the MMAs of
             // tile i - 1 - BUF have run, for which tile i - 1 - 2 BUF had been read: 2 BUF + 1 slots or more will do
-            if (warp < 4) sRow[i % row_slots<R>() * 128 + r] = by_fma ? kByFma : (int)E;
-            planes = rows != kAll;
+            if (warp < 4) sRow[i % row_slots<R>() * 128 + r] = (int)E | (by_fma ? kByFma | (E0 != E ? kAllFma : 0) : 0);
+            planes = !DBL || rows != kAll;
             if (!planes) return true;
             if constexpr (DBL) {
 #pragma unroll
@@ -618,6 +623,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         };
         // The rows of the quadrant that the slices do not take, shared out among its warps.
         bool have_u = false;
+        [[maybe_unused]] uint32_t met = 0;
         auto quad_rows = [&](uint32_t mask, uint64_t at) -> bool {
             if (mask == 0) return true;
             if (!have_u && !wait(bbar, 0)) return false;
@@ -648,7 +654,8 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                     if (!wait(done(buf(i), g), par(i))) { bad = true; break; }
                     if (g == 0) {
                         E = sRow[i % row_slots<R>() * 128 + r];
-                        mask = __ballot_sync(0xffffffffu, E == kByFma);
+                        mask = __ballot_sync(0xffffffffu, E & kByFma);
+                        E &= ~kAllFma;
                     }
                     if (mask == 0xffffffffu) continue;
 #pragma unroll
@@ -694,39 +701,47 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                         if (((2 * j + k) & 3) == 0) to_double_int(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
                         else to_double_cvt(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
                     }
-                    if (E != kByFma) st_words<VEC * AW>(pt + vCol[j], w);
+                    if (E < kByFma) st_words<VEC * AW>(pt + vCol[j], w);
                 }
                 if (!quad_rows(mask, (uint64_t)(pt - psi))) { bad = true; break; }
             } else {
                 // y = 2^(E - 138) sum_d D_d 2^(-8d)
                 if (!wait(done(buf(i), 0), par(i))) { bad = true; break; }
-                const int E = sRow[i % row_slots<R>() * 128 + r];
-                const uint32_t mask = __ballot_sync(0xffffffffu, E == kByFma);  // rows that are not in the accumulators
+                const int row = sRow[i % row_slots<R>() * 128 + r], E = row & kExponent;
+                const uint32_t mask = __ballot_sync(0xffffffffu, row & kByFma);
+                if (mask) {  // by FMAs first: then no warp needs the input of these rows any more
+                    bool ok = quad_rows(mask, (uint64_t)(pt - psi));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(fmabar(quad));
+                    ok = wait(fmabar(quad), met++ & 1) && ok;
+                    if (!ok) { bad = true; break; }
+                }
                 const float sc = __uint_as_float((uint32_t)(E - 11) << 23);
-                if (mask == 0xffffffffu) finish(i);
-                else {
 #pragma unroll
-                    for (int c = 0; c < 2 * CPO; c += 8) {
-                        uint32_t v[4][8], w[8];
+                for (int c = 0; c < 2 * CPO; c += 8) {
+                    uint32_t v[4][8], w[8];
 #pragma unroll
-                        for (int d = 0; d < 4; ++d) tmem_ld<8>(td + 64 * d + c, v[d]);
-                        wait_ld();
-                        if (c + 8 == 2 * CPO) finish(i);
+                    for (int d = 0; d < 4; ++d) tmem_ld<8>(td + 64 * d + c, v[d]);
+                    wait_ld();
+                    if (c + 8 == 2 * CPO) finish(i);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            float y = __uint_as_float(v[3][j]);
-                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[2][j]));
-                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[1][j]));
-                            y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
-                            w[j] = __float_as_uint(y * sc);
-                        }
-                        if (E != kByFma) {
+                    for (int j = 0; j < 8; ++j) {
+                        float y = __uint_as_float(v[3][j]);
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[2][j]));
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[1][j]));
+                        y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
+                        w[j] = __float_as_uint(y * sc);
+                    }
+                    if (row < kByFma) {
 #pragma unroll
-                            for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
-                        }
+                        for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
+                    } else if (row < kAllFma) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if ((int)(max(w[2 * j] & 0x7FFFFFFFu, w[2 * j + 1] & 0x7FFFFFFFu) >> 23) + kLarge >= E)
+                                st_words<AW>(pt + vCol[c / 2 + j], w + 2 * j);
                     }
                 }
-                if (!quad_rows(mask, (uint64_t)(pt - psi))) { bad = true; break; }
             }
         }
         if (bad && lane == 0) atomicOr(err, DEVERR_TIMEOUT);
