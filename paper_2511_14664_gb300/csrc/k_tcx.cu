@@ -33,12 +33,12 @@
 // sparse and structured ones among them, was 1.19 times that of the slices alone, at worst 1.56; so it is 0.98, 1.03). Rows
 // outside the exponents that the slices take go by FMAs as well; amplitudes that the block joins with an infinity or NaN
 // become NaN.
-// One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0: 275, 340 / 240, 273 us, and
-// without this 254, 309 / 201, 239; with amplitudes over 30 binades 510 / 710 (CUDA cores 461 / 3457). 16-step TFIM chains of
-// small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 9.5 / 4.0 -> 10.2 ms. Measured and left: such rows by three
+// One pass, complex64 26 qubits / complex128 24 qubits, windows from qubit 8 and from qubit 0: 270, 331 / 240, 273 us, and
+// without this 254, 309 / 201, 239; with amplitudes over 30 binades 570 / 710 (CUDA cores 461 / 3457). 16-step TFIM chains of
+// small angles, 25 qubits complex64 / 23 complex128: 5.2 -> 10.1 / 4.0 -> 10.2 ms. Measured and left: such rows by three
 // more warps, a few of a quadrant or all of them (351 us from qubit 0 in complex64, 850 us at 30 binades); one warp that
 // decides for all rows (2.7 ms at 30 binades); rows given away unseen where a quadrant has few (301 us); ROWS = 4 (590 us at
-// 30 binades).
+// 30 binades, against 510 with whole rows by FMAs).
 //
 // Layout. A tile is 128 rows (the 7 lowest index bits outside the block) by 32 columns; blocks of fewer qubits
 // take idle qubits as further columns (U x I). Digit plane s of a tile is a K-major operand of 128 x 64 FP16
@@ -53,7 +53,7 @@
 // positions take all of tensor memory and the planes half of shared memory, so a tile's MMAs commit in four
 // groups of planes: as a group retires, the input (8 warps) writes the next tile's planes over it and the output
 // (16 warps) adds the positions it finished.
-// Bound: complex64 (26 qubits, 275 us, 0.57 of the copy rate) the input's loads and conversion; complex128 (24
+// Bound: complex64 (26 qubits, 270 us, 0.58 of the copy rate) the input's loads and conversion; complex128 (24
 // qubits, 240 us, 3457 on CUDA cores) the output: its conversions run on the FP64 units at two a cycle and SM,
 // and on the integer pipe about as fast, so they are spread over both; the tensor cores work a quarter of the
 // time. Measured and left (against 190 us without the rows by FMAs): one set of warps for input and output (281 us at 24 qubits), 8 output warps (208),
@@ -135,6 +135,7 @@ struct Args {
     int from_basis;      // the input is |basis>, generated in registers instead of read
     uint64_t basis;
     int k;               // the block's own qubits: column bits 0 .. k - 1
+    int split;           // 2^split CTAs share a tile: lanes 0 .. 32 / 2^split - 1 of each quadrant are the first one's rows, ...
     int32_t w[4];        // 2^30, 2^22, 2^14, 2^6 (as parameters, so that they stay multiplications)
 };
 
@@ -374,7 +375,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int* const sums = reinterpret_cast<const int*>(reinterpret_cast<const char*>(bops) + S * kPlaneB);
     const T* const umat = reinterpret_cast<const T*>(sums + NR + 2 * D);  // U by columns
-    const uint32_t t0 = blockIdx.x, G = gridDim.x;  // (fewer than 2^32 tiles: checked by the host)
+    const uint32_t t0 = blockIdx.x >> a.split, G = gridDim.x >> a.split;  // (fewer than 2^32 tiles: checked by the host)
     const uint32_t m = t0 < a.ntiles ? (uint32_t)((a.ntiles - t0 + G - 1) / G) : 0u;  // tiles of this CTA
     auto tile = [&](uint32_t i) { return (uint64_t)t0 + (uint64_t)i * G; };
     auto buf = [&](uint32_t i) { return i % BUF; };
@@ -387,6 +388,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     };
     // input and output warps: thread = row r of the tile, columns c0 ..
     const int quad = warp & 3, r = quad * 32 + lane;
+    const bool own = (uint32_t)lane >> (5 - a.split) == (blockIdx.x & ((1u << a.split) - 1));  // the row is this CTA's
 
     bool bad = false;
     if (warp >= kIn + kOut) {
@@ -459,13 +461,13 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         unsigned char* const arow = sA + (r >> 3) * 1024 + (r & 7) * 128;
         auto load_tile = [&](uint32_t (&X)[W], uint64_t t) {
             const uint64_t b = insert_zeros(t, a.spos, a.nS);
-            if (a.from_basis) {
+            if (a.from_basis || !own) {
                 const uint64_t rb = b + deposit((uint64_t)r, a.rpos, kRowBits);
 #pragma unroll
                 for (int j = 0; j < CPI; ++j) {
 #pragma unroll
                     for (int k = 0; k < AW; ++k) X[AW * j + k] = 0;
-                    if (rb + vCol[j] == a.basis) X[AW * j + (DBL ? 1 : 0)] = DBL ? 0x3FF00000u : 0x3F800000u;
+                    if (own && rb + vCol[j] == a.basis) X[AW * j + (DBL ? 1 : 0)] = DBL ? 0x3FF00000u : 0x3F800000u;
                 }
             } else {
 #pragma unroll
@@ -701,7 +703,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                         if (((2 * j + k) & 3) == 0) to_double_int(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
                         else to_double_cvt(Y[2 * j + k], E, w[2 * k], w[2 * k + 1]);
                     }
-                    if (E < kByFma) st_words<VEC * AW>(pt + vCol[j], w);
+                    if (E < kByFma && own) st_words<VEC * AW>(pt + vCol[j], w);
                 }
                 if (!quad_rows(mask, (uint64_t)(pt - psi))) { bad = true; break; }
             } else {
@@ -732,10 +734,10 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                         y = __fmaf_rn(y, 0x1p-8f, __uint_as_float(v[0][j]));
                         w[j] = __float_as_uint(y * sc);
                     }
-                    if (row < kByFma) {
+                    if (row < kByFma && own) {
 #pragma unroll
                         for (int j = 0; j < 4; j += VEC) st_words<VEC * AW>(pt + vCol[c / 2 + j], w + 2 * j);
-                    } else if (row < kAllFma) {
+                    } else if (row < kAllFma && own) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
                             if ((int)(max(w[2 * j] & 0x7FFFFFFFu, w[2 * j + 1] & 0x7FFFFFFFu) >> 23) + kLarge >= E)
@@ -851,6 +853,9 @@ cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targ
         a.basis = *from_basis;
     }
     for (int j = 0; j < 4; ++j) a.w[j] = 1 << (30 - 8 * j);
+    // Fewer tiles than SMs: several CTAs share a tile, each for a part of its rows, so that rows by FMAs are spread (9-step TFIM
+    // chains of small angles in complex128, 17 / 18 qubits: 0.83 -> 0.41, 0.97 -> 0.62 ms; random states level).
+    while (a.split < 3 && (a.ntiles << (a.split + 1)) <= (uint64_t)d.num_sms) ++a.split;
     auto launch = [&](auto kern, auto* p, int threads, size_t smem) -> cudaError_t {
         cudaError_t e = smem_optin(reinterpret_cast<const void*>(kern), (int)smem);
         if (e != cudaSuccess) return e;
@@ -859,7 +864,7 @@ cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targ
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3((unsigned)std::min<uint64_t>((uint64_t)d.num_sms, a.ntiles), 1, 1);
+        cfg.gridDim = dim3((unsigned)std::min<uint64_t>((uint64_t)d.num_sms, a.ntiles) << a.split, 1, 1);
         cfg.blockDim = dim3((unsigned)threads, 1, 1);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = s;

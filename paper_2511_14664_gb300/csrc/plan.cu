@@ -59,8 +59,8 @@ struct PlanOp {
 // complex128: k = 2 n = 18 / 19: 11.8 / 11.5, 22.7 / 12.8; k = 3 n = 17: 12.4 / 12.3; k = 5 n = 17: 37 / 12.2, n = 24: 3457 / 240;
 // k = 1 n = 18 / 19 / 20: 8.3 / 11.6, 12.4 / 11.8, 20.6 / 16.5.
 // complex64: k = 5 n = 17 / 18 / 19: 6.2 / 6.7, 6.2 / 6.8, 8.3 / 7.0, from qubit 0 up 6.3 / 7.2, 8.3 / 7.3, 12.4 / 7.6, n = 26:
-// 462 / 275; k = 4 n = 17 / 20 / 21: 10.4 / 6.7, 22.2 / 9.5, 12.3 / 14.7 (the CUDA-core pass of 17 to 20 qubits is that slow by
-// itself), and with qubit 0 among the targets n = 21 / 24: 22.7 / 16.2, 130 / 89.
+// 462 / 270; k = 4 n = 17 / 20 / 21: 10.4 / 6.7, 22.2 / 9.5, 12.3 / 14.4 (the CUDA-core pass of 17 to 20 qubits is that slow by
+// itself), and with qubit 0 among the targets n = 21 / 24: 22.7 / 15.9, 130 / 87.
 // Below 17 qubits plans run resident (k_small.cu, k_small_tiles.cu).
 constexpr int kTcxMinQubits = 17;
 static bool tcx_pays(int dtype, int n, int k, const int* targets) {
