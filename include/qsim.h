@@ -57,8 +57,7 @@ extern "C" {
                               them): in norm the error is below that of FMA, and amplitude by
                               amplitude below 2^-16 (complex64) or 2^-43 (complex128) of
                               sum_c |U_rc| |x_c|, of which a chain of FMAs may lose 2^-18 or 2^-47.
-                              Rows of too wide a range for that are taken by FMA, so that small
-                              amplitudes keep their digits */
+                              Small results of rows of too wide a range for that come from FMA */
 #define QSIM_PREC_TF32X3 1 /* tensor cores: 3 TF32 products (hi*hi + hi*lo + lo*hi), FP32 accumulation */
 #define QSIM_PREC_BF16X3 2 /* tensor cores: 2-way BF16 split, 3 products, FP32 accumulation. REDUCED
                               accuracy (~16 significant bits per product, not complex64 level): ~1e-8
