@@ -437,15 +437,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch(const __grid_constant__ A
 struct Choice { int n = 0, gates = 0, cluster = 0, own = 0; };
 
 // The width from which circuits run as plans of their own (QSIM_MAX_QUBITS + 1: none). Estimates in microseconds a pass at
-// 19, 20 and 21 qubits, from 1 to 40 circuits of one width (TFIM chains, brickwork, random circuits, random pairs): a plan 11.5,
-// 15, 20.5, among others 4.7, 7.3, 12.5 (measured 3.7 to 6, 6 to 10, 11 to 17: more where more rows go by FMAs); a cluster 23,
-// 42, 82, beside others 40, 71, 143, but no less than 3, 5.6, 11.2 for each circuit. A plan's passes and the tensor-core
-// plans beside take their time from the clusters and one another. Plans where they save 2 %.
-// Measured, clusters / as chosen (ms): one chain of 19, 20, 21 qubits 1.00 / 0.31, 1.79 / 0.44, 3.96 / 0.63; forty 5.0 / 4.1, 9.6 /
-// 7.5, 21.9 / 13.6; forty of 19 qubits stay, brickwork 2.8 (as plans 2.7), random circuits 1.9 (3.2), random pairs 2.2 (2.8);
-// forty random circuits of 20 qubits and 10 gates a qubit, whose rows the estimate does not see, 4.0 / 5.1; 64 chains of 10 to 24
-// qubits 75 / 36. Where the tensor-core plans outlast the clusters these are hidden and stay (256 chains of 10 to 24 qubits,
-// FP16X3: 42.7, and 44.6 with the 19-qubit ones as plans).
+// 19, 20 and 21 qubits, from 1 to 40 circuits of one width (TFIM chains, brickwork, random circuits, random pairs): a plan 9, 11,
+// 16, among others 4.2, 6.3, 11.5 (measured 3.4 to 4.4, 5.5 to 6.6, 10 to 11.5); a cluster 23, 42, 82, beside others 40, 71,
+// 143, but no less than 3, 5.6, 11.2 for each circuit. A plan's passes and the tensor-core plans beside take their time from
+// the clusters and one another. Plans where they save 2 %.
+// Measured, clusters / as chosen (ms): one chain of 19, 20, 21 qubits 1.00 / 0.23, 1.79 / 0.31, 3.96 / 0.46; forty 5.0 / 3.8, 9.6 /
+// 6.6, 21.9 / 12.5; forty random circuits 1.9 / 1.9 (in clusters), 4.0 / 3.4, 8.3 / 6.0; 64 chains of 10 to 24 qubits 75 / 26. Where
+// the tensor-core plans outlast the clusters these are hidden and stay (256 chains of 10 to 24 qubits, FP16X3: 42.7, and
+// 44.6 with the 19-qubit ones as plans).
 int own_width(const std::vector<Choice>& c, const qsim_circuit* cs, const std::vector<char>& tensor, int first) {
     constexpr int kNone = QSIM_MAX_QUBITS + 1;
     auto at = [](int n, double a, double b, double d) { return n <= 19 ? a : n == 20 ? b : std::ldexp(d, n - 21); };
@@ -472,9 +471,9 @@ int own_width(const std::vector<Choice>& c, const qsim_circuit* cs, const std::v
         for (const Choice& x : c) {
             if (x.n == 0) continue;
             if (x.n >= m) {
-                const double one = x.own * at(x.n, 11.5, 15.0, 20.5);
+                const double one = x.own * at(x.n, 9.0, 11.0, 16.0);
                 if (one > longest) longest = one;
-                sum += x.own * at(x.n, 4.7, 7.3, 12.5);
+                sum += x.own * at(x.n, 4.2, 6.3, 11.5);
             } else {
                 const double one = x.cluster * (in_clusters > 1 ? at(x.n, 40.0, 71.0, 143.0) : at(x.n, 23.0, 42.0, 82.0));
                 if (one > cluster) cluster = one;
@@ -1061,6 +1060,7 @@ static int batch_plan_create_impl(const qsim_circuit* cs, int count, const qsim_
             po.tc_min_k = 5;
             po.launch_per_pass = 1;  // plans run concurrently on worker streams inside a captured graph
             const int r = qsim_plan_create(&cs[wides[w]], QSIM_C64, &po, pst[my_slot], &wph[w], &wpi[w]);
+            if (r == QSIM_OK && own) plan_for_values(wph[w]);
             if (r == QSIM_OK && cudaStreamSynchronize(pst[my_slot]) != cudaSuccess)
                 return cuda_fail(cudaGetLastError(), "tensor-core plan of a wide circuit");
             if (r == QSIM_OK && enq.joinable()) {

@@ -56,6 +56,10 @@ std::vector<std::vector<int>> group_gates(const std::vector<uint64_t>& gmask, co
 bool group_cache_get(const std::vector<uint64_t>& key, std::vector<std::vector<int>>& out);
 void group_cache_put(const std::vector<uint64_t>& key, const std::vector<std::vector<int>>& blocks);
 
+// A plan whose state is only reduced to <Z> and <Z Z> values, which the norm of the error bounds: own-precision blocks need
+// not keep the digits of small amplitudes.
+void plan_for_values(qsim_plan_h p);
+
 }  // namespace qsim
 
 extern "C" int qsim_synchronize(qsim_h h);

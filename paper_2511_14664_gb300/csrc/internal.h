@@ -180,9 +180,10 @@ bool tcx_supported(int n, int k);
 // Bytes of the prepared operand, and its preparation from a device FP64 matrix U (2^k x 2^k complex).
 size_t tcx_operand_bytes(int dtype);
 cudaError_t launch_tcx_prepare(int dtype, const double* dU, int k, void* dB, cudaStream_t s);
-// Apply the prepared block; with from_basis its input is the basis state |*from_basis>, generated instead of read.
+// Apply the prepared block; with from_basis its input is the basis state |*from_basis>, generated instead of read. Without
+// `digits` amplitudes that are small beside their row's largest one may lose digits (the norm of the error is the same).
 cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targets, const void* dB, unsigned* dev_err,
-                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis = nullptr);
+                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis = nullptr, bool digits = true);
 
 // ---- two 6-qubit blocks in one pass (k_tc_pair.cu, FP16 split products) -------------------------------------
 // True when blocks on t1 and then t2 (6 targets each, in their matrices' index order) fit one 13-bit tile of

@@ -135,6 +135,7 @@ struct Args {
     int from_basis;      // the input is |basis>, generated in registers instead of read
     uint64_t basis;
     int k;               // the block's own qubits: column bits 0 .. k - 1
+    int digits;          // rows of wide range go by FMAs
     int split;           // 2^split CTAs share a tile: lanes 0 .. 32 / 2^split - 1 of each quadrant are the first one's rows, ...
     int32_t w[4];        // 2^30, 2^22, 2^14, 2^6 (as parameters, so that they stay multiplications)
 };
@@ -509,7 +510,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 #pragma unroll
             for (int k = 0; k < kIn / 4; ++k) e = __vmaxu2(e, ex[k * 128]);
             const uint32_t E0 = e >> 16, low = 0x7FFFu - (e & 0xFFFFu), E = min(max(E0, kLowE<R>), kHighE<R>);
-            bool by_fma = E0 != 0 && (E0 != E || E0 - low > (uint32_t)C::kRange);
+            bool by_fma = E0 != 0 && (E0 != E || (a.digits && E0 - low > (uint32_t)C::kRange));
             uint32_t rows = __ballot_sync(0xffffffffu, by_fma);  // (the same in all warps of the quadrant)
             if (rows) {
                 // its columns within 1 and within 4 binades of the largest; has every row of U an entry of 2^-7, or of 2^-4, there?
@@ -822,7 +823,7 @@ cudaError_t launch_tcx_prepare(int dtype, const double* dU, int k, void* dB, cud
 }
 
 cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targets, const void* dB, unsigned* dev_err,
-                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis) {
+                             cudaStream_t s, const DevInfo& d, const uint64_t* from_basis, bool digits) {
     const uintptr_t addr = reinterpret_cast<uintptr_t>(psi);
     if (!tcx_supported(n, k) || (reinterpret_cast<uintptr_t>(dB) & 15) != 0 || (addr & 15) != 0) return cudaErrorInvalidValue;
     tcx::Args a;
@@ -846,6 +847,7 @@ cudaError_t launch_tcx_apply(int dtype, void* psi, int n, int k, const int* targ
     for (int q = 0; q < n; ++q)
         if ((smask >> q) & 1) a.spos[a.nS++] = q;
     a.k = k;
+    a.digits = digits;
     a.ntiles = 1ull << (n - a.nS);
     if (a.ntiles >> 32) return cudaErrorInvalidValue;  // 32-bit tile counters in the kernel
     if (from_basis) {

@@ -93,6 +93,7 @@ struct qsim_plan {
     qsim::PlanExtra extra;
     bool dry = false;  // planned on the host only: no device buffer, cannot execute
     bool pooled = false;    // dbuf came from the library's memory pool
+    bool digits = true;     // small amplitudes keep their digits (k_tcx.cu); false: only <Z> values are read
     bool small = false;     // a whole-plan execution is one resident launch (k_small.cu)
     size_t small_off = 0;   // its program in the plan buffer
     qsim::SmallTiles stiles;  // groups > 0: the program is k_small_tiles.cu's
@@ -558,7 +559,7 @@ static int enqueue_ops(qsim_state* h, const qsim_plan* p, size_t first = 0, size
         const uint64_t* fb = oi == first ? first_from_basis : nullptr;
         if (op.tcx) {
             e = launch_tcx_apply(h->dtype, h->psi, h->n, op.k, op.targets, static_cast<char*>(p->dbuf) + op.dev_off,
-                                 h->derr, h->stream, h->dev, fb);
+                                 h->derr, h->stream, h->dev, fb, p->digits);
             if (e != cudaSuccess) return cuda_fail(e, "plan pass launch");
             continue;
         }
@@ -605,6 +606,8 @@ static int enqueue_ops(qsim_state* h, const qsim_plan* p, size_t first = 0, size
 }  // namespace qsim
 
 using namespace qsim;
+
+void qsim::plan_for_values(qsim_plan_h p) { p->digits = false; }
 
 extern "C" {
 
