@@ -26,8 +26,10 @@
 // three as zero). So the slices take a row only where every result y_i has sum_c |U_ic| |x_c| above 2^-9 of that power of
 // two, which bounds its error by 2^-16 (2^-43) of that sum, beside 2^-18 (2^-47) for a chain of 64 FMAs: rows whose amplitudes
 // lie within kRange = 8 binades of the largest (the entries of a row of U sum to 1 or more), and rows in which every row
-// of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4 (the input warps look at U
-// for 0.1 % of the rows of a random state, and few of those fail). The others go by FMAs in the state's precision, by the
+// of U has an entry of at least 2^-7 at an amplitude within 1 binade, or of 2^-4 within 4, or, in complex128, only zeros at
+// all amplitudes, for a result that is zero either way (21-qubit random circuit of 8 gates a qubit 0.80 -> 0.44 ms; in complex64
+// it cost other circuits 3 to 7 %). The input warps look at U for 0.1 % of the rows of a random state, and few of those
+// fail. The others go by FMAs in the state's precision, by the
 // output (rows_by_fma): in complex128 the whole row; in complex64, where 64 FMAs lose more than the slices, the results more
 // than kLarge = 4 binades below the row's largest amplitude (with whole rows by FMAs the norm of the error of 12 circuits,
 // sparse and structured ones among them, was 1.19 times that of the slices alone, at worst 1.56; so it is 0.98, 1.03). Rows
@@ -110,12 +112,12 @@ template <typename R> constexpr int row_slots() { return Cfg<R>::BUF == 1 ? 4 : 
 template <typename R> constexpr int threads() { return 32 * (Cfg<R>::IN + Cfg<R>::OUT + Cfg<R>::MMA); }
 template <typename R> constexpr int smem_planes() { return Cfg<R>::S * (Cfg<R>::BUF * kPlaneA + kPlaneB); }
 template <typename R> constexpr int bars() { return Cfg<R>::BUF * (2 + Cfg<R>::GROUPS) + 9; }
-// planes, column offsets, largest and smallest amplitudes of the input's rows [2][IN / 4][128] and which of them are large
-// [IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the large entries of U [32][2], U and
+// planes, column offsets, largest and smallest amplitudes of the input's rows [2][IN / 4][128] and which of them are large and
+// not zero [2][IN / 4][128], exponents of tiles in flight [row_slots][128], barriers, the TMEM slot, the large entries of U [32][4], U and
 // the rows taken by FMAs [OUT][ROWS][32], alignment
 template <typename R> constexpr int smem_rows() { return (Cfg<R>::OUT * Cfg<R>::ROWS + Cfg<R>::U) * D * 2 * (int)sizeof(R); }
 template <typename R> constexpr size_t smem_bytes() {
-    return smem_planes<R>() + smem_rows<R>() + 16 * D + 4 * (3 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
+    return smem_planes<R>() + smem_rows<R>() + 24 * D + 4 * (4 * (Cfg<R>::IN / 4) + row_slots<R>()) * 128 +
            8 * bars<R>() + 8 + 1024;
 }
 // With 1 KiB that the system takes, below the 196 KiB that leave 60 KiB of L1: the data of loads in flight lies there
@@ -336,10 +338,10 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     T* sU = reinterpret_cast<T*>(sB + S * kPlaneB);                   // U by columns (complex64)
     T* sX = sU + C::U * D;                                               // [kOut][ROWS][32]
     uint64_t* sCol = reinterpret_cast<uint64_t*>(sX + kOut * C::ROWS * D);
-    uint4* sL = reinterpret_cast<uint4*>(sCol + D);                   // [16]: of two rows of U each, large entries
-    uint32_t* sE = reinterpret_cast<uint32_t*>(sL + D / 2);           // [2][kIn / 4][128]
-    uint32_t* sBig = sE + 2 * (kIn / 4) * 128;                        // [kIn / 4][128]
-    int* sRow = reinterpret_cast<int*>(sBig + (kIn / 4) * 128);       // [row_slots][128]
+    uint4* sL = reinterpret_cast<uint4*>(sCol + D);                   // of the rows of U, the large entries (and, complex128, those not zero)
+    uint32_t* sE = reinterpret_cast<uint32_t*>(sL + D);               // [2][kIn / 4][128]
+    uint32_t* sBig = sE + 2 * (kIn / 4) * 128;                        // [2][kIn / 4][128]
+    int* sRow = reinterpret_cast<int*>(sBig + 2 * (kIn / 4) * 128);       // [row_slots][128]
     uint64_t* mbar = reinterpret_cast<uint64_t*>(sRow + row_slots<R>() * 128);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + bars<R>());
     constexpr uint32_t kAll = 0xFFFFFFFFu;
@@ -375,7 +377,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int* const sums = reinterpret_cast<const int*>(reinterpret_cast<const char*>(bops) + S * kPlaneB);
-    const T* const umat = reinterpret_cast<const T*>(sums + NR + 2 * D);  // U by columns
+    const T* const umat = reinterpret_cast<const T*>(sums + NR + 3 * D);  // U by columns
     const uint32_t t0 = blockIdx.x >> a.split, G = gridDim.x >> a.split;  // (fewer than 2^32 tiles: checked by the host)
     const uint32_t m = t0 < a.ntiles ? (uint32_t)((a.ntiles - t0 + G - 1) / G) : 0u;  // tiles of this CTA
     auto tile = [&](uint32_t i) { return (uint64_t)t0 + (uint64_t)i * G; };
@@ -456,7 +458,9 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         const int c0 = CPI * (warp >> 2);
         const volatile uint64_t* vCol = sCol + c0;
         // every warp writes the same words of sL and reads its own writes
-        reinterpret_cast<uint2*>(sL)[lane] = make_uint2((uint32_t)sums[NR + lane], (uint32_t)sums[NR + D + lane]);
+        const uint32_t l7 = (uint32_t)sums[NR + lane], l4 = (uint32_t)sums[NR + D + lane];
+        if constexpr (DBL) sL[lane] = make_uint4(l7, l4, (uint32_t)sums[NR + 2 * D + lane], 0u);
+        else reinterpret_cast<uint2*>(sL)[lane] = make_uint2(l7, l4);
         __syncwarp();
         const T* const prow = psi + deposit((uint64_t)r, a.rpos, kRowBits);
         unsigned char* const arow = sA + (r >> 3) * 1024 + (r & 7) * 128;
@@ -481,6 +485,12 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
         constexpr int EB = DBL ? 20 : 23;  // exponent position in a real's upper word
         auto amplitude = [&](const uint32_t (&X)[W], int j) {
             return max(X[AW * j + (DBL ? 1 : 0)] & 0x7FFFFFFFu, X[AW * j + (DBL ? 3 : 1)] & 0x7FFFFFFFu);
+        };
+        [[maybe_unused]] auto nonzero = [&](const uint32_t (&X)[W], int j) {
+            uint32_t any = 0;
+#pragma unroll
+            for (int k = 0; k < AW; ++k) any |= DBL && (k & 1) == 0 ? X[AW * j + k] : X[AW * j + k] & 0x7FFFFFFFu;
+            return any != 0;
         };
         auto span = [&](const uint32_t (&X)[W]) {
             uint32_t top = 0, low = kAll;
@@ -513,14 +523,18 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
             bool by_fma = E0 != 0 && (E0 != E || (a.digits && E0 - low > (uint32_t)C::kRange));
             uint32_t rows = __ballot_sync(0xffffffffu, by_fma);  // (the same in all warps of the quadrant)
             if (rows) {
-                // its columns within 1 and within 4 binades of the largest; has every row of U an entry of 2^-7, or of 2^-4, there?
+                // its columns within 1 and within 4 binades of the largest; has every row of U an entry of 2^-7, or of 2^-4, there
+                // (or, complex128, no entry but zeros where the row has amplitudes, for a result that is zero either way)?
                 uint32_t big = 0;
+                [[maybe_unused]] uint32_t some = 0, bz = 0;
 #pragma unroll
                 for (int j = 0; j < CPI; ++j) {
                     const uint32_t m = amplitude(X, j) >> EB;
+                    if constexpr (DBL) some |= nonzero(X, j) ? 1u << j : 0u;
                     big |= (m + 1 >= E0 ? 1u << j : 0u) | (m + 4 >= E0 ? 0x10000u << j : 0u);
                 }
                 sBig[(warp >> 2) * 128 + r] = big;
+                if constexpr (DBL) sBig[(kIn / 4 + (warp >> 2)) * 128 + r] = some;
                 if (!meet()) return false;
                 uint32_t b1 = 0, b4 = 0;
 #pragma unroll
@@ -528,12 +542,21 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
                     const uint32_t v = sBig[k * 128 + r];
                     b1 |= (v & 0xFFFFu) << (CPI * k);
                     b4 |= (v >> 16) << (CPI * k);
+                    if constexpr (DBL) bz |= sBig[(kIn / 4 + k) * 128 + r] << (CPI * k);
                 }
                 bool held = E0 == E;
-#pragma unroll (DBL ? D / 2 : 2)
-                for (int k = 0; k < D / 2; ++k) {
-                    const uint4 l = sL[k];
-                    held = held & (((b1 & l.x) | (b4 & l.y)) != 0) & (((b1 & l.z) | (b4 & l.w)) != 0);
+                if constexpr (DBL) {
+#pragma unroll
+                    for (int k = 0; k < D; ++k) {
+                        const uint4 l = sL[k];
+                        held = held & (((b1 & l.x) | (b4 & l.y)) != 0 || (bz & l.z) == 0);
+                    }
+                } else {
+#pragma unroll 2
+                    for (int k = 0; k < D / 2; ++k) {
+                        const uint4 l = sL[k];
+                        held = held & (((b1 & l.x) | (b4 & l.y)) != 0) & (((b1 & l.z) | (b4 & l.w)) != 0);
+                    }
                 }
                 by_fma = by_fma && !held;
                 rows = __ballot_sync(0xffffffffu, by_fma);
@@ -760,7 +783,7 @@ k_tcx_block(typename Amp<R>::T* __restrict__ psi, const __grid_constant__ Args a
 // The digit planes of U (x I on the padding columns): real form B[2i][2c] = Re U_ic, B[2i][2c+1] = -Im U_ic,
 // B[2i+1][2c] = Im U_ic, B[2i+1][2c+1] = Re U_ic in fixed point, plane t = digit t (most significant first).
 // After the planes: the sum of |digits| over all planes of each row (64 integers); for each complex row of U x I the columns
-// whose entry has a part of at least 2^-7, and of at least 2^-4 (32 words each); U itself by columns in the state's
+// whose entry has a part of at least 2^-7, of at least 2^-4, and other than zero (32 words each); U itself by columns in the state's
 // precision. One block per row n.
 template <typename R>
 __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U, int k, unsigned char* __restrict__ out) {
@@ -775,14 +798,14 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
             typename Amp<R>::T u;
             u.x = (R)U[e];
             u.y = (R)U[e + 1];
-            reinterpret_cast<typename Amp<R>::T*>(out + C::S * kPlaneB + 4 * (NR + 2 * D))[c * Du + i] = u;
+            reinterpret_cast<typename Amp<R>::T*>(out + C::S * kPlaneB + 4 * (NR + 3 * D))[c * Du + i] = u;
         }
     }
     // thread kk of row 2 i has a part of U_ic (c = kk / 2); of the two, the larger counts
     const double part = fmax(fabs(v), fabs(__shfl_xor_sync(0xffffffffu, v, 1)));
-    __shared__ uint32_t large[2][2];
-    for (int l = 0; l < 2; ++l) {
-        const uint32_t b = __ballot_sync(0xffffffffu, part >= (l ? 0x1p-4 : 0x1p-7));
+    __shared__ uint32_t large[3][2];
+    for (int l = 0; l < 3; ++l) {
+        const uint32_t b = __ballot_sync(0xffffffffu, l == 2 ? part != 0.0 : part >= (l ? 0x1p-4 : 0x1p-7));
         if ((kk & 31) == 0) large[l][kk >> 5] = b;
     }
     const uint64_t f = (uint64_t)__double2ll_rn(scalbn(v, C::kStepsU)) + (sizeof(R) == 8 ? 0x0080808080808080ull : 0x80808080ull);
@@ -798,7 +821,7 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
     __syncthreads();
     int* const tail = reinterpret_cast<int*>(out + C::S * kPlaneB);
     if (kk == 0) tail[n] = total[0] + total[1];
-    if (kk < 2 && !(n & 1)) {
+    if (kk < 3 && !(n & 1)) {
         uint32_t m = 0;
         for (int c = 0; c < D; ++c) m |= (large[kk][c >> 4] >> (2 * (c & 15)) & 1u) << c;
         tail[NR + D * kk + i] = (int)m;
@@ -810,7 +833,7 @@ __global__ void __launch_bounds__(NR) k_tcx_prepare(const double* __restrict__ U
 bool tcx_supported(int n, int k) { return k >= 1 && k <= tcx::K && n >= tcx::K + tcx::kRowBits && n <= 43; }
 
 size_t tcx_operand_bytes(int dtype) {
-    return (size_t)tcx::kPlaneB * (dtype == QSIM_C64 ? tcx::Cfg<float>::S : tcx::Cfg<double>::S) + sizeof(int) * (tcx::NR + 2 * tcx::D) +
+    return (size_t)tcx::kPlaneB * (dtype == QSIM_C64 ? tcx::Cfg<float>::S : tcx::Cfg<double>::S) + sizeof(int) * (tcx::NR + 3 * tcx::D) +
            (size_t)(dtype == QSIM_C64 ? sizeof(float2) : sizeof(double2)) * tcx::D * tcx::D;
 }
 
