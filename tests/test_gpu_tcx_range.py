@@ -123,3 +123,27 @@ def test_non_finite_amplitudes_stay_in_their_groups(qsim, dtype, n, qubits, valu
     assert np.count_nonzero(group) == 1 << len(qubits)
     assert not np.any(np.isfinite(out[group]))
     assert np.max(np.abs(out[~group] - good[~group])) <= 2 * TOL[dtype] * np.max(np.abs(good[~group]))
+
+
+@pytest.mark.parametrize("dtype", [C64, C128])
+@pytest.mark.parametrize("n,qubits", [(17, (1, 4, 8, 12, 16)), (18, (0, 1, 2, 3, 4)), (20, (3, 9, 15))])
+def test_sparse_blocks_of_sparse_states(qsim, dtype, n, qubits):
+    """Controlled-NOTs and half turns, whose products have exact zeros, on states of few amplitudes: results to which
+    nothing adds are zero, the others keep their digits."""
+    half = 0.5 * np.array([[1 + 1j, 1 - 1j], [1 - 1j, 1 + 1j]])
+    c = W.Circuit(n)
+    for a, b in zip(qubits, qubits[1:]):
+        c.append(W.Gate((b,), (a,), W.X(), "cx"))
+    for q in qubits[::2]:
+        c.append(W.Gate((q,), (), half, "sx"))
+    c.append(W.Gate((qubits[0],), (qubits[-1],), W.X(), "cx"))
+    rng = np.random.default_rng(n)
+    psi0 = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    psi0 *= (rng.random(1 << n) < 0.1) * np.exp2(-rng.uniform(0, 3, 1 << n))
+    psi0[::7] *= 2.0 ** -15
+    psi0 = psi0.astype(DT[dtype])
+    out = rows(run(qsim, c, dtype, psi0), n, qubits)
+    U, x = matrix(c, qubits), rows(psi0.astype(np.complex128), n, qubits)
+    total = np.abs(x) @ np.abs(U).T
+    assert np.any(total == 0)
+    assert np.all(np.abs(out - x @ U.T) <= TOL[dtype] * total)
